@@ -181,11 +181,13 @@ brmppi::KConst make_kconst(const brmppi_params& q) {
   k.inv_l1 = 1.0f / q.l1;
   k.inv_l2 = 1.0f / q.l2;
   k.k_hitch = q.lh / q.l1;
+  k.khl2 = static_cast<float>(static_cast<double>(q.lh) / q.l1 / q.l2);
   k.dtheta_max = q.dtheta_max;
   k.kappa = q.kappa;
   k.r_inflate = q.r_inflate;
   k.Qc = q.Qc;
   k.Ql = q.Ql;
+  k.iso = q.Qc == q.Ql ? 1 : 0;
   k.Qth = q.Qth;
   k.R0 = q.R[0];
   k.R1 = q.R[1];
@@ -198,27 +200,25 @@ brmppi::KConst make_kconst(const brmppi_params& q) {
   k.zhi0 = q.z_hi[0];
   k.zhi1 = q.z_hi[1];
   k.zhi2 = q.z_hi[2];
-  k.sig0 = q.sigma[0];
-  k.sig1 = q.sigma[1];
-  k.sig2 = q.sigma[2];
   k.alpha0 = q.alpha0;
-  k.sigma_alpha = q.sigma_alpha;
-  k.ua_lo = q.ua_lo;
-  k.ua_hi = q.ua_hi;
-  k.w_u0 = q.w_u[0];
-  k.w_u1 = q.w_u[1];
-  k.w_u2 = q.w_u[2];
-  k.pc_u0 = 0.5f * q.rho * (q.z_hi[0] + q.z_lo[0]);
-  k.pc_u1 = 0.5f * q.rho * (q.z_hi[1] + q.z_lo[1]);
-  k.pc_u2 = 0.5f * q.rho * (q.z_hi[2] + q.z_lo[2]);
+  for (int j = 0; j < 3; ++j) {
+    const double m = static_cast<double>(q.w_u[j]) + q.rho;
+    const double a = k.proj ? q.w_u[j] / m : 1.0;
+    const double b = k.proj ? 0.5 * q.rho * (static_cast<double>(q.z_hi[j]) + q.z_lo[j]) / m : 0.0;
+    k.qa[j] = static_cast<float>(a);
+    k.qb[j] = static_cast<float>(b);
+    k.qs[j] = static_cast<float>(a * q.sigma[j]);
+    k.qlo[j] = static_cast<float>(a * q.z_lo[j] + b);
+    k.qhi[j] = static_cast<float>(a * q.z_hi[j] + b);
+  }
   k.m_u0 = q.w_u[0] + q.rho;
   k.m_u1 = q.w_u[1] + q.rho;
-  k.inv_m_u0 = 1.0f / (q.w_u[0] + q.rho);
-  k.inv_m_u1 = 1.0f / (q.w_u[1] + q.rho);
-  k.inv_m_u2 = 1.0f / (q.w_u[2] + q.rho);
   const double m_alpha = static_cast<double>(q.w_alpha) + static_cast<double>(q.rho);
-  k.w_am = static_cast<float>(q.w_alpha / m_alpha);
-  k.pc_am = static_cast<float>(0.5 * q.rho * (static_cast<double>(q.ua_hi) + q.ua_lo) / m_alpha);
+  const double w_am = q.w_alpha / m_alpha, pc_am = 0.5 * q.rho * (static_cast<double>(q.ua_hi) + q.ua_lo) / m_alpha;
+  k.ps = static_cast<float>(w_am * q.sigma_alpha);
+  k.pc_am = static_cast<float>(pc_am);
+  k.pam_lo = static_cast<float>(w_am * q.ua_lo + pc_am);
+  k.pam_hi = static_cast<float>(w_am * q.ua_hi + pc_am);
   k.m_a = q.w_alpha + q.rho;
   k.h_floor = q.h_floor;
   k.q_coll = q.q_coll;
@@ -242,14 +242,15 @@ brmppi::KConst make_kconst(const brmppi_params& q) {
   return k;
 }
 
-brmppi::SmemCaps make_caps(int n_obs, int n_rows, int n_pts, int H, int tps) {
+brmppi::SmemCaps make_caps(int n_obs, int n_rows, int n_pts, int H, int tps, int bpt, bool ext) {
   brmppi::SmemCaps c{};
-  c.obs = 8 * n_obs;
+  c.obs = 8 * (n_obs + 1);  // and the null row
   c.path = brmppi::SmemCaps::pad4(3 * n_pts);
-  c.phead = brmppi::SmemCaps::pad4(2 * n_pts);
   c.unom = brmppi::SmemCaps::pad4(3 * H);
   c.ustar = brmppi::SmemCaps::pad4(3 * H + 1);
-  c.noise_per_team = tps > 1 ? 8 * philox_blocks(n_rows) : 0;
+  c.noise_per_team = tps > 1 && bpt <= 2 ? 8 * philox_blocks(n_rows) : 0;
+  // 4 rows a Philox block after the first, in passes of the team's lanes
+  c.rows_per_team = c.noise_per_team > 0 ? 0 : 4 * ((philox_blocks(n_rows) - 1 + tps - 1) / tps) * (ext ? 4 : 2) * tps;
   c.uh_per_team = 0;
   c.merge = 0;
   return c;
@@ -257,16 +258,41 @@ brmppi::SmemCaps make_caps(int n_obs, int n_rows, int n_pts, int H, int tps) {
 
 size_t smem_bytes(const brmppi::SmemCaps& c, int spb) { return sizeof(float) * static_cast<size_t>(c.total(spb)); }
 
-bool pick_bpt(int tps, int P, int* bpt) {
-  // one lane: the lane draws every block (b >= P); wider teams: the row
-  // slots of a lane (4 b) must hold its share of the at most 4 P - 4 rows
-  // (their blocks are drawn by producer warps or staged in passes)
-  for (int b : {1, 2, 3, 4, 5, 6, 8})
-    if ((tps == 1 ? b >= P : (4 * P - 4 + tps - 1) / tps <= 4 * b) && brmppi::variant_exists(tps, b)) {
-      *bpt = b;
-      return true;
-    }
+// The bytes a launch cannot do without: the rows' state goes to local memory
+// where it does not fit (fit_rows).
+size_t table_bytes(brmppi::SmemCaps c, int spb) {
+  c.rows_per_team = 0;
+  return smem_bytes(c, spb);
+}
+
+bool fit_rows(brmppi::SmemCaps* c, int spb, size_t smem_limit) {
+  if (c->rows_per_team == 0 || smem_bytes(*c, spb) <= smem_limit) return true;
+  c->rows_per_team = 0;
   return false;
+}
+
+bool pick_bpt(int tps, int P, int* bpt) {
+  // Philox blocks of rows a lane holds: up to two of them are drawn by
+  // producer warps (bpt 1, 2; teams), more by the lane itself (bpt 3; one
+  // lane always does)
+  if (tps == 1) {
+    *bpt = 1;
+    return P <= 8;
+  }
+  const int per_lane = (P - 1 + tps - 1) / tps;
+  if (per_lane > 4) return false;
+  *bpt = std::max(1, std::min(per_lane, 3));
+  return brmppi::variant_exists(tps, *bpt);
+}
+
+int samples_per_team(const Shape& sh, bool ext, long long tiles, size_t smem, int num_sms) {
+  const int threads = sh.threads / 2;
+  if (sh.threads % 64 != 0 || threads < 64 || threads > brmppi::kMaxPairBlockThreads ||
+      !brmppi::pair_exists(sh.tps, sh.bpt, ext))
+    return 1;
+  const long long resident =
+      std::min<long long>(brmppi::kMaxPairBlockThreads * brmppi::kPairCtas / threads, 227 * 1024 / (smem + 2048));
+  return tiles >= resident * num_sms ? 2 : 1;
 }
 
 int part_stride_for(int H) { return static_cast<int>(align_up(3 + 3 * static_cast<size_t>(H) + 1, 4)); }
@@ -310,7 +336,9 @@ bool heuristic_plain(const brmppi_ctx* c, int n_obs, int n_pts, Shape* out) {
       threads = 64;
   }
   if (threads < tps) return false;
-  while (smem_bytes(make_caps(n_obs, rows_of(c->prm, n_obs), n_pts, c->prm.H, tps), threads / tps) > c->smem_limit) {
+  const bool ext = brmppi::needs_ext(make_kconst(c->prm));
+  while (table_bytes(make_caps(n_obs, rows_of(c->prm, n_obs), n_pts, c->prm.H, tps, bpt, ext), threads / tps) >
+         c->smem_limit) {
     if (!fixed_threads && threads > kMinThreads) {
       threads -= 32;
     } else if (!fixed_tps && tps < 32) {
@@ -330,8 +358,9 @@ bool plain_shape(const brmppi_ctx* c, int n_obs, int n_pts, Shape* out) {
   if (c->prm.threads_per_sample == 0 && c->prm.block_threads == 0) {
     auto it = c->tuned.find(n_obs);
     if (it != c->tuned.end()) {
-      const brmppi::SmemCaps caps = make_caps(n_obs, rows_of(c->prm, n_obs), n_pts, c->prm.H, it->second.tps);
-      if (smem_bytes(caps, it->second.threads / it->second.tps) <= c->smem_limit) {
+      const brmppi::SmemCaps caps = make_caps(n_obs, rows_of(c->prm, n_obs), n_pts, c->prm.H, it->second.tps,
+                                              it->second.bpt, brmppi::needs_ext(make_kconst(c->prm)));
+      if (table_bytes(caps, it->second.threads / it->second.tps) <= c->smem_limit) {
         *out = it->second;
         return true;
       }
@@ -421,10 +450,13 @@ brmppi_status enqueue_plain_sized(brmppi_ctx* c, const Shape& sh, int S, int H, 
     L.single.tile_base = tile0;
     L.single.no_merge = 1;
   }
-  L.caps = make_caps(n_obs, rows_of(c->prm, n_obs), n_pts, H, sh.tps);
+  const brmppi::KConst k = make_kconst(c->prm);
+  const bool ext = brmppi::needs_ext(k);
+  L.caps = make_caps(n_obs, rows_of(c->prm, n_obs), n_pts, H, sh.tps, sh.bpt, ext);
+  brmppi::LaunchMode mode;
+  mode.local = !fit_rows(&L.caps, spb, c->smem_limit);
   L.uh = c->d_uh;
   L.uh_stride = 3 * H * spb;
-  const brmppi::KConst k = make_kconst(c->prm);
   single_launch_options(L, sh, k, rows_of(c->prm, n_obs), H, c->smem_limit);
   const size_t smem = smem_bytes(L.caps, spb);
   const int tiles = tiles_out ? n_tiles : L.single.tiles;  // CTAs of the launch
@@ -432,7 +464,8 @@ brmppi_status enqueue_plain_sized(brmppi_ctx* c, const Shape& sh, int S, int H, 
   if ((!tiles_out && static_cast<size_t>(tiles) > c->part_tiles) ||
       static_cast<size_t>(tiles) * static_cast<size_t>(L.uh_stride) > c->uh_floats)
     return fail(c, BRMPPI_EINVAL, "launch shape exceeds the context's scratch");
-  cudaError_t e = brmppi::launch_solve(sh.tps, sh.bpt, tiles, sh.threads, smem, stream, k, L, L.single.P);
+  if (L.rows == 0 && !mode.local) mode.ns = samples_per_team(sh, ext, tiles, smem, c->num_sms);
+  cudaError_t e = brmppi::launch_solve(sh.tps, sh.bpt, tiles, sh.threads, smem, stream, k, L, L.single.P, mode);
   if (e != cudaSuccess) return cuda_fail(c, e, "kernel launch");
   if (u_safe) {
     // the stabilizer on (x0, U*[0]): one thread, after the solve
@@ -531,7 +564,7 @@ brmppi_status launch_batch(brmppi_ctx* c, Lane& L, const BatchPlan& plan, cudaSt
   D.caps = plan.caps;
   const brmppi::KConst k = make_kconst(c->prm);
   cudaError_t e = brmppi::launch_solve(plan.shape.tps, plan.shape.bpt, plan.grid, plan.shape.threads, plan.smem,
-                                       stream, k, D, plan.P);
+                                       stream, k, D, plan.P, plan.mode);
   if (e != cudaSuccess) return cuda_fail(c, e, "batch kernel launch");
   if (plan.any_u_safe && (e = brmppi::launch_stabilize_table(k, L.d_inst, plan.n_inst, stream)) != cudaSuccess)
     return cuda_fail(c, e, "stabilizer launch");
@@ -572,7 +605,10 @@ brmppi_status plan_batch(brmppi_ctx* c, Lane& L, const brmppi_instance* inst, in
     return fail(c, BRMPPI_EINVAL, "no batch launch shape for these instances");
   }
   const int spb = sh.threads / sh.tps;
-  const brmppi::SmemCaps caps = make_caps(nobs_max, rows_of(c->prm, nobs_max), npts_max, Hmax, sh.tps);
+  const bool ext = brmppi::needs_ext(make_kconst(c->prm));
+  brmppi::SmemCaps caps = make_caps(nobs_max, rows_of(c->prm, nobs_max), npts_max, Hmax, sh.tps, sh.bpt, ext);
+  brmppi::LaunchMode mode;
+  mode.local = !fit_rows(&caps, spb, c->smem_limit);
   const size_t smem = smem_bytes(caps, spb);
   if (smem > c->smem_limit) return fail(c, BRMPPI_EINVAL, "batch tables exceed shared memory");
   size_t pool = 0;
@@ -602,8 +638,8 @@ brmppi_status plan_batch(brmppi_ctx* c, Lane& L, const brmppi_instance* inst, in
                      return a.first > b.first;
                    });
   for (size_t j = 0; j < items.size(); ++j) h_work[j] = items[j].second;
-  const int occ =
-      brmppi::variant_occupancy(sh.tps, sh.bpt, sh.threads, smem, brmppi::needs_ext(make_kconst(c->prm)), P_cap);
+  if (!mode.local) mode.ns = samples_per_team(sh, ext, static_cast<long long>(items.size()), smem, c->num_sms);
+  const int occ = brmppi::variant_occupancy(sh.tps, sh.bpt, sh.threads, smem, ext, P_cap, mode);
   if (occ < 1) return fail(c, BRMPPI_EINVAL, "batch launch shape cannot be resident");
   int grid = occ * c->num_sms;
   if (grid > static_cast<int>(items.size())) grid = static_cast<int>(items.size());
@@ -611,6 +647,7 @@ brmppi_status plan_batch(brmppi_ctx* c, Lane& L, const brmppi_instance* inst, in
     return fail(c, BRMPPI_EINVAL, "batch history scratch too small");
   plan->shape = sh;
   plan->P = P_cap;
+  plan->mode = mode;
   plan->n_inst = n;
   plan->n_work = static_cast<int>(items.size());
   plan->grid = grid;
@@ -944,8 +981,9 @@ brmppi_status brmppi_merge_tiles(brmppi_ctx* c, const brmppi_instance* q, const 
   brmppi::Inst in = make_inst(q->x0, q->U_nom, q->obs, q->n_obs, q->path, q->n_pts, q->ds, q->S, q->H, q->seed,
                               q->counter, q->U_out, q->traj_out, q->J_out, q->U_next, q->status,
                               const_cast<float*>(tiles), c->d_sync, spb, c->prm.n_discs);
-  const brmppi::SmemCaps caps = make_caps(q->n_obs, rows_of(c->prm, q->n_obs), q->n_pts, q->H, sh.tps);
-  const size_t smem = smem_bytes(caps, 1);
+  const brmppi::SmemCaps caps = make_caps(q->n_obs, rows_of(c->prm, q->n_obs), q->n_pts, q->H, sh.tps, sh.bpt,
+                                          brmppi::needs_ext(make_kconst(c->prm)));
+  const size_t smem = table_bytes(caps, 1);
   if (smem > c->smem_limit) return fail(c, BRMPPI_EINVAL, "shared memory need exceeds the device limit");
   const cudaError_t e = brmppi::launch_merge_tiles(make_kconst(c->prm), in, caps, smem, static_cast<cudaStream_t>(stream));
   if (e != cudaSuccess) return cuda_fail(c, e, "merge launch");
@@ -1054,13 +1092,14 @@ brmppi_status brmppi_autotune(brmppi_ctx* c, const double* x0, const float* U_no
   Shape best;
   float best_ms = 1e30f;
   for (int tps : {1, 2, 4, 8, 16, 32}) {
-    const brmppi::SmemCaps caps = make_caps(n_obs, rows_of(c->prm, n_obs), n_pts, H, tps);
     int bpt;
     if (!pick_bpt(tps, P, &bpt)) continue;
+    const brmppi::SmemCaps caps = make_caps(n_obs, rows_of(c->prm, n_obs), n_pts, H, tps, bpt,
+                                            brmppi::needs_ext(make_kconst(c->prm)));
     for (int threads : {64, 128, 256}) {
       if (threads < tps || threads / tps < 2) continue;
       const int spb = threads / tps;
-      if (smem_bytes(caps, spb) > c->smem_limit) continue;
+      if (table_bytes(caps, spb) > c->smem_limit) continue;
       const size_t tiles = (static_cast<size_t>(c->prm.S) + spb - 1) / spb;
       if (tiles > c->part_tiles || tiles * 3 * H * spb > c->uh_floats) continue;
       Shape sh;

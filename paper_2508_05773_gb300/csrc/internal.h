@@ -44,6 +44,10 @@ struct Shape {
   int tps = 0, bpt = 0, threads = 0;
 };
 
+// Samples a team of a launch rolls out together (2: the packed-pair
+// instantiations) for `tiles` tiles of a shape with `smem` bytes a CTA.
+int samples_per_team(const Shape& sh, bool ext, long long tiles, size_t smem, int num_sms);
+
 // Everything one in-flight batch launch needs: instance table, work list,
 // per-tile partial pool, per-instance counters, per-CTA input history, host
 // staging of the table and list, and the events that guard their reuse.
@@ -67,6 +71,7 @@ struct Lane {
 struct BatchPlan {
   Shape shape;
   int n_inst = 0, n_work = 0, grid = 0, Hmax = 0;
+  brmppi::LaunchMode mode;
   bool any_u_safe = false;  // some instance asks for the stabilized input
   int P = 1;                // Philox blocks per step the launch is shaped for
   brmppi::SmemCaps caps{};
@@ -143,6 +148,9 @@ brmppi_status fail(brmppi_ctx* c, brmppi_status st, const std::string& msg);
 brmppi_status cuda_fail(brmppi_ctx* c, cudaError_t e, const char* what);
 int philox_blocks(int n_rows);  // per step, for n_rows obstacle rows
 bool pick_bpt(int tps, int P, int* bpt);
+// Keep the rows' state of a launch in shared memory if it fits; else drop it
+// from the caps and return false (it goes to local memory).
+bool fit_rows(brmppi::SmemCaps* c, int spb, size_t smem_limit);
 int part_stride_for(int H);
 // Team width of batches and serving when the optional terms are on: at most
 // two Philox blocks per lane.

@@ -20,14 +20,18 @@ void for_each_variant(F f) {
   for (int i = 0; i < n; ++i) f(e[i]);
   const Variant* g = variants_latency_ext(&n);
   for (int i = 0; i < n; ++i) f(g[i]);
+  const Variant* p = variants_pair(&n);
+  for (int i = 0; i < n; ++i) f(p[i]);
 }
 
 // rows = 0: the general instantiation of a shape; rows > 0: the one with
 // exactly that many constraint rows a lane (null if not compiled)
-const Variant* find(int tps, int bpt, bool ext, int rows = 0) {
+const Variant* find(int tps, int bpt, bool ext, int rows = 0, LaunchMode mode = LaunchMode()) {
   const Variant* hit = nullptr;
   for_each_variant([&](const Variant& v) {
-    if (v.tps == tps && v.bpt == bpt && v.ext == ext && v.rows == rows) hit = &v;
+    if (v.tps == tps && v.bpt == bpt && v.ext == ext && v.rows == rows && v.ns == mode.ns &&
+        v.local == mode.local)
+      hit = &v;
   });
   return hit;
 }
@@ -75,14 +79,16 @@ __global__ void __launch_bounds__(256) noise_blocks_kernel(uint32_t key0, uint32
   const long long st = i / n_blocks;
   const int tau = static_cast<int>(st % H);
   const int s = static_cast<int>(st / H);
-  const uint4 w = philox4x32_10(
-      make_uint4(static_cast<uint32_t>(b), static_cast<uint32_t>(tau), static_cast<uint32_t>(s), ctr), key0, key1);
+  const PhiloxSample smp = philox_sample(static_cast<uint32_t>(s));
+  const uint4 w = philox_words(philox_block(static_cast<uint32_t>(b), ctr, key0, key1), smp,
+                               philox_step(smp, static_cast<uint32_t>(tau), key0, key1), key0, key1);
   if (words) reinterpret_cast<uint4*>(words)[i] = w;
   if (normals) {
-    float4 g;
-    box_muller(w.x, w.y, g.x, g.y);
-    box_muller(w.z, w.w, g.z, g.w);
-    reinterpret_cast<float4*>(normals)[i] = g;
+    const float* tab = reinterpret_cast<const float*>(&kNoiseTables);
+    Vec<1> n0, n1, n2, n3;
+    box_muller<1>(&w.x, &w.y, tab, n0, n1);
+    box_muller<1>(&w.z, &w.w, tab, n2, n3);
+    reinterpret_cast<float4*>(normals)[i] = make_float4(n0.x, n1.x, n2.x, n3.x);
   }
 }
 
@@ -130,6 +136,8 @@ cudaError_t launch_stabilize(const KConst& k, const double* x, const float* u_re
   return cudaGetLastError();
 }
 
+bool pair_exists(int tps, int bpt, bool ext) { return find(tps, bpt, ext, 0, LaunchMode{2, false}) != nullptr; }
+
 bool variant_exists(int tps, int bpt) { return find(tps, bpt, false) != nullptr && find(tps, bpt, true) != nullptr; }
 
 cudaError_t set_smem_limit(size_t bytes) {
@@ -142,8 +150,8 @@ cudaError_t set_smem_limit(size_t bytes) {
   return err;
 }
 
-int noise_warps(int tps, int bpt, int threads, int P) {
-  if (tps <= 1 || bpt > 2) return 0;  // the team's lanes draw (or stage) the blocks themselves
+int noise_warps(int tps, int bpt, int threads, int P, int ns) {
+  if (tps <= 1 || bpt > 2 || ns > 1) return 0;  // the team's lanes draw the blocks themselves
   const int blocks_per_step = P * (threads / tps);
   int w = (blocks_per_step + 63) / 64;  // at most two Philox blocks per producer lane and step
   // and at least one producer per compute warp: warps go to the four
@@ -157,28 +165,33 @@ int noise_warps(int tps, int bpt, int threads, int P) {
   return w < 1 ? 1 : w;
 }
 
-int block_threads(int tps, int bpt, int threads, int P) { return threads + 32 * noise_warps(tps, bpt, threads, P); }
+int block_threads(int tps, int bpt, int threads, int P, int ns) {
+  return threads / ns + 32 * noise_warps(tps, bpt, threads, P, ns);
+}
 
 int exact_rows_variant(int tps, int bpt, const KConst& k, int n_rows) {
-  if (!k.proj || tps <= 1 || bpt > 2 || n_rows <= 0) return 0;
+  if (tps <= 1 || bpt > 2 || n_rows <= 0) return 0;
   const int rows = (n_rows + tps - 1) / tps;
   return find(tps, 1, needs_ext(k), rows) ? rows : 0;
 }
 
-int variant_occupancy(int tps, int bpt, int threads, size_t smem, bool ext, int P) {
-  const Variant* v = find(tps, bpt, ext);
-  if (!v || block_threads(tps, bpt, threads, P) > kMaxBlockThreads) return 0;
+int variant_occupancy(int tps, int bpt, int threads, size_t smem, bool ext, int P, LaunchMode mode) {
+  const int ns = mode.ns;
+  const Variant* v = find(tps, bpt, ext, 0, mode);
+  if (!v || block_threads(tps, bpt, threads, P, ns) > (ns > 1 ? kMaxPairBlockThreads : kMaxBlockThreads)) return 0;
   int n = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, v->fn, block_threads(tps, bpt, threads, P), smem) !=
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, v->fn, block_threads(tps, bpt, threads, P, ns), smem) !=
       cudaSuccess)
     return 0;
   return n;
 }
 
 cudaError_t launch_solve(int tps, int bpt, int blocks, int threads, size_t smem, cudaStream_t stream,
-                         const KConst& k, const LaunchDesc& L, int P) {
-  const Variant* v = find(tps, bpt, needs_ext(k));
-  if (!v || block_threads(tps, bpt, threads, P) > kMaxBlockThreads) return cudaErrorInvalidValue;
+                         const KConst& k, const LaunchDesc& L, int P, LaunchMode mode) {
+  const int ns = mode.ns;
+  const Variant* v = find(tps, bpt, needs_ext(k), 0, mode);
+  if (!v || block_threads(tps, bpt, threads, P, ns) > (ns > 1 ? kMaxPairBlockThreads : kMaxBlockThreads))
+    return cudaErrorInvalidValue;
   if (L.rows > 0) {
     // the exact-rows variants merge in shared memory: the launch must have
     // reserved the room for the instance's partials
@@ -189,8 +202,8 @@ cudaError_t launch_solve(int tps, int bpt, int blocks, int threads, size_t smem,
     if (!v) return cudaErrorInvalidValue;
   }
   LaunchDesc D = L;
-  D.noise_warps = noise_warps(tps, bpt, threads, P);
-  v->fn<<<blocks, block_threads(tps, bpt, threads, P), smem, stream>>>(k, D);
+  D.noise_warps = noise_warps(tps, bpt, threads, P, ns);
+  v->fn<<<blocks, block_threads(tps, bpt, threads, P, ns), smem, stream>>>(k, D);
   return cudaGetLastError();
 }
 

@@ -15,6 +15,8 @@ struct Variant {
              // footprint discs other than the rear-axle point)
   KernelFn fn;
   int rows = 0;  // > 0: exactly this many constraint rows a lane (single solves)
+  int ns = 1;    // samples a team rolls out together
+  bool local = false;  // rows' state in local memory
 };
 
 // Instantiations, one translation unit per group of team widths and family
@@ -26,20 +28,29 @@ const Variant* variants_narrow_ext(int* n);  // the same, with the optional term
 const Variant* variants_wide_ext(int* n);
 const Variant* variants_latency(int* n);     // exact rows a lane, noise-warp shapes
 const Variant* variants_latency_ext(int* n); // the same with the optional terms (4 lanes)
+const Variant* variants_pair(int* n);        // two samples a team (throughput shapes)
 
 // Whether a launch with these constants needs the family with the optional terms.
 inline bool needs_ext(const KConst& k) { return k.coll || k.obs8 || k.abuf || k.discs || k.third || k.jerk; }
 
-// Threads of a launch: `threads` roll out samples; teams wider than one lane
-// with at most two Philox blocks per lane add warps that produce the noise,
-// enough for two blocks per producer lane and step where the CTA has room
-// (up to four; P blocks per sample).  Other variants draw on their own
-// lanes (0 noise warps).  At most kMaxBlockThreads (the kernels' launch
-// bound).
+// Threads of a launch shape.  `threads` / tps is the samples of a CTA's tile;
+// with ns samples a team threads / ns of them roll out.  Teams of one sample
+// wider than one lane with at most two Philox blocks per lane add warps that
+// produce the noise, enough for two blocks per producer lane and step where
+// the CTA has room (up to four; P blocks per sample).  Other variants draw on
+// their own lanes (0 noise warps).  At most kMaxBlockThreads (the kernels'
+// launch bound).
 constexpr int kMaxBlockThreads = 512;
+constexpr int kMaxPairBlockThreads = kMaxPairThreads;  // the two-sample instantiations' launch bound
 constexpr int kMaxRowsBlockThreads = 384;  // the exact-rows instantiations' launch bound
-int noise_warps(int tps, int bpt, int threads, int P);
-int block_threads(int tps, int bpt, int threads, int P);
+// How a shape is run: samples a team, and the rows' state in local memory
+// (where it does not fit in shared memory; one sample a team).
+struct LaunchMode {
+  int ns = 1;
+  bool local = false;
+};
+int noise_warps(int tps, int bpt, int threads, int P, int ns = 1);
+int block_threads(int tps, int bpt, int threads, int P, int ns = 1);
 
 // The rows a lane holds in a single solve of n_rows constraint rows on a
 // noise-warp shape, if the instantiation with exactly that many is compiled
@@ -48,12 +59,14 @@ int exact_rows_variant(int tps, int bpt, const KConst& k, int n_rows);
 
 // Supported (threads per sample, Philox blocks per lane) pairs.
 bool variant_exists(int tps, int bpt);
+// Whether a pair is compiled with two samples a team.
+bool pair_exists(int tps, int bpt, bool ext);
 
 // Raise the dynamic shared-memory limit of every variant to `bytes`.
 cudaError_t set_smem_limit(size_t bytes);
 
 // CTAs of a variant resident per SM for a launch shape (0 if it cannot run).
-int variant_occupancy(int tps, int bpt, int threads, size_t smem, bool ext, int P);
+int variant_occupancy(int tps, int bpt, int threads, size_t smem, bool ext, int P, LaunchMode mode);
 
 // Enqueue the hitch stabilizer for n states (out: n x 4 floats).
 cudaError_t launch_stabilize(const KConst& k, const double* x, const float* u_ref, int n, float* out,
@@ -76,6 +89,6 @@ cudaError_t launch_merge_tiles(const KConst& k, const Inst& in, const SmemCaps& 
 
 // Enqueue one launch of the solve kernel.
 cudaError_t launch_solve(int tps, int bpt, int blocks, int threads, size_t smem, cudaStream_t stream,
-                         const KConst& k, const LaunchDesc& L, int P);
+                         const KConst& k, const LaunchDesc& L, int P, LaunchMode mode);
 
 }  // namespace brmppi

@@ -25,7 +25,7 @@ namespace brmppi_host {
 // defined in api.cu
 std::string check_params(const brmppi_params* p);
 brmppi::KConst make_kconst(const brmppi_params& q);
-brmppi::SmemCaps make_caps(int n_obs, int n_rows, int n_pts, int H, int tps);
+brmppi::SmemCaps make_caps(int n_obs, int n_rows, int n_pts, int H, int tps, int bpt, bool ext);
 size_t smem_bytes(const brmppi::SmemCaps& c, int spb);
 brmppi::Inst make_inst(const double* x0, const float* U_nom, const float* obs, int n_obs, const float* path,
                        int n_pts, float ds, int S, int H, uint64_t seed, uint64_t counter, float* U_out,
@@ -126,14 +126,16 @@ extern "C" brmppi_status brmppi_solve_device_noalloc(const brmppi_params* p, con
   float* part = scratch + kNaSyncFloats;
   L.single = make_inst(x0_dev, U_nom_dev, obs_dev, n_obs, path_dev, n_pts, ds, p->S, p->H, seed, counter, U_out_dev,
                        traj_out_dev, J_out_dev, U_next_dev, status_dev, part, sync, kNaSpb, p->n_discs);
-  L.caps = make_caps(n_obs, n_rows, n_pts, p->H, kNaTps);
+  const brmppi::KConst k = make_kconst(*p);
+  L.caps = make_caps(n_obs, n_rows, n_pts, p->H, kNaTps, bpt, brmppi::needs_ext(k));
+  brmppi::LaunchMode mode;
+  mode.local = !fit_rows(&L.caps, kNaSpb, smem_optin);
   L.uh = part + kNaPartFloats;
   L.uh_stride = 3 * p->H * kNaSpb;
   Shape sh;
   sh.tps = kNaTps;
   sh.bpt = bpt;
   sh.threads = kNaThreads;
-  const brmppi::KConst k = make_kconst(*p);
   single_launch_options(L, sh, k, n_rows, p->H, smem_optin);
   const size_t smem = smem_bytes(L.caps, kNaSpb);
   if (smem > smem_optin)
@@ -143,7 +145,7 @@ extern "C" brmppi_status brmppi_solve_device_noalloc(const brmppi_params* p, con
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   cudaError_t e = cudaMemsetAsync(sync, 0, sizeof(float) * kNaSyncFloats, s);
   if (e != cudaSuccess) return cuda_fail(nullptr, e, "no-alloc solve: clearing counters");
-  e = brmppi::launch_solve(kNaTps, bpt, L.single.tiles, kNaThreads, smem, s, k, L, L.single.P);
+  e = brmppi::launch_solve(kNaTps, bpt, L.single.tiles, kNaThreads, smem, s, k, L, L.single.P, mode);
   if (e != cudaSuccess) return cuda_fail(nullptr, e, "no-alloc solve: kernel launch");
   return BRMPPI_OK;
 }

@@ -5,9 +5,9 @@
 // with the BR-MPPI rollout of Sec. IV-A):
 //
 //   for each sample s, step tau:
-//     noise        Philox4x32-10 + Box-Muller, recomputed (never stored in
-//                  HBM): in registers a step ahead (one lane per sample) or
-//                  by noise warps into shared memory (wider teams)
+//     noise        Philox4x32-10 + Box-Muller (noise.cuh), recomputed (never
+//                  stored in HBM): in registers where it is used, or by
+//                  noise warps into shared memory (the latency shapes)
 //     sample       z_des = clip(U_nom + sigma n), u^alpha_des = clip(sigma_a n)
 //     rows         barrier-rate equality per constraint (Eq. cbf_equality):
 //                  hitch (Eq. hitch_angle_barrier) and obstacles
@@ -30,11 +30,25 @@
 // so a solve gives the same bits alone or inside any batch with the same
 // launch shape.
 //
-// Team decomposition: TPS consecutive lanes own one sample.  Every lane of
-// a team computes the hitch row (its terms enter the team sums once); the
-// obstacle rows are spread round-robin over the team (row j on lane
-// j % TPS), each with its noise normal 4 + j.  The rank-2 structure of the
-// projection makes the cross-lane exchange five floats per step.
+// Team decomposition: TPS consecutive lanes own one sample (or two, NS = 2,
+// in packed registers).  Every lane of a team computes the hitch row (its
+// terms enter the team sums once); the obstacle rows are spread over the team
+// (row j on lane j % TPS of the latency shapes, a Philox block's four rows on
+// one lane elsewhere), each with its noise normal 4 + j.  The rank-2
+// structure of the projection makes the cross-lane exchange five floats per
+// step.  The step is written in Vec<NS> (vec.cuh), every rounding explicit:
+// a sample has the same bits in each variant of one team width, so a batch
+// may run two samples a team when it fills the GPU and one when it does not.
+//
+// What bounds it (measured on GB300, before this layout -> with it): the
+// throughput shapes are bound by issue slots and the FMA pipe.  48 solves of
+// 4096 samples, H = 50, 8 ellipses: 493 -> 400 us, 1359 -> 740 thread
+// instructions a rollout-step (packed pairs, table-driven normals, the first
+// Philox rounds shared, rows as linear forms in (Q d, Q), no subnormal
+// scaling around the MUFU); 256 uneven solves 2567 -> 1768 us; S = 65536,
+// H = 100, 64 ellipses 2030 -> 1394 us (FMA pipe 58% and ALU pipe 40% busy,
+// three warps a scheduler).  The latency shapes are bound by one compute
+// warp's dependency chain: S = 4096, H = 50, 8 ellipses 39.6 -> 34.7 us.
 //
 // Projection in Woodbury form.  A = [A_u | diag(h~)] where only the a and
 // omega columns of A_u are non-zero, M = diag(m_u, m_alpha):
@@ -59,7 +73,9 @@
 #include <cuda_runtime.h>
 #include <math_constants.h>
 
+#include "noise.cuh"
 #include "trig.cuh"
+#include "vec.cuh"
 
 namespace brmppi {
 
@@ -71,11 +87,17 @@ struct KConst {
   float Ts, hTs2, Ts2, inv_lambda;  // Ts, Ts^2 / 2, Ts^2
   float inv_l1, inv_l2, k_hitch, dtheta_max, kappa, r_inflate;
   float Qc, Ql, Qth, R0, R1, R2, mu, nu_bar;
-  float zlo0, zlo1, zlo2, zhi0, zhi1, zhi2, sig0, sig1, sig2;
-  float alpha0, sigma_alpha, ua_lo, ua_hi;
-  float w_u0, w_u1, w_u2, pc_u0, pc_u1, pc_u2;  // W_u and rho/2 (hi + lo)
-  float m_u0, m_u1, inv_m_u0, inv_m_u1, inv_m_u2;
-  float w_am, pc_am, m_a;  // W_alpha / m_alpha, rho (hi + lo) / (2 m_alpha), m_alpha = W_alpha + rho
+  int iso;         // Qc == Ql: the contouring cost needs no path direction
+  float khl2;      // k_hitch / l2
+  float zlo0, zlo1, zlo2, zhi0, zhi1, zhi2;
+  float alpha0;
+  // sampled inputs in the projection's coordinates, M_u^-1 p_u = clip(qa
+  // U_nom + qb + qs n, qlo, qhi) with qa = W_u / M_u, qb = rho (hi + lo) /
+  // (2 M_u) (without the projection qa = 1, qb = 0), and p_alpha / m_alpha =
+  // clip(ps n + pc_am, pam_lo, pam_hi)
+  float qa[3], qb[3], qs[3], qlo[3], qhi[3];
+  float ps, pc_am, pam_lo, pam_hi;
+  float m_u0, m_u1, m_a;  // M_u = W_u + rho, m_alpha = W_alpha + rho
   float h_floor;
   float q_coll, q_abuf, inv_hbuf;
   float alpha_stab, inv_qs0, inv_qs1;  // hitch stabilizer: CBF rate, Q_h^-1
@@ -115,18 +137,22 @@ struct Inst {
                      // stop; the instance's tiles are merged by merge_tiles_kernel
 };
 
+constexpr int kMaxBlocks = 32;  // Philox blocks a step: 3 inputs, the hitch and at most 124 rows
+
 // Shared-memory capacities of a launch (floats).
 // Every region is a multiple of 4 floats (16 bytes): float4 accesses stay
 // aligned.
 struct SmemCaps {
-  int obs, path, phead, unom, ustar;
+  int obs, path, unom, ustar;
   int noise_per_team;  // teams wider than one lane: staged normals, 2 steps x P blocks x 4
   int uh_per_team;     // 3 H when the applied-input history stays in shared memory, else 0
+  int rows_per_team;   // variants without producer warps: floats of row state a sample
   int merge;           // > 0: room for an instance's tile partials (merged in shared memory)
   __host__ __device__ static int pad4(int n) { return (n + 3) & ~3; }
   __host__ __device__ int total(int spb) const {
-    const int tail = noise_per_team * spb + pad4(uh_per_team * spb);  // noise, history; then the partials
-    return obs + path + phead + unom + ustar + pad4(3 * spb) + 256 + 16 + (tail > merge ? tail : merge);
+    // noise and history, or row state; then the partials
+    const int tail = (noise_per_team + rows_per_team) * spb + pad4(uh_per_team * spb);
+    return obs + path + unom + ustar + pad4(3 * spb) + 256 + 16 + kNoiseTableFloats + 4 * kMaxBlocks + (tail > merge ? tail : merge);
   }
 };
 
@@ -150,64 +176,21 @@ enum : unsigned { ERR_EXPONENT = 1u, ERR_NONFINITE_X0 = 2u, ERR_PATH_TURN = 4u }
 // cost's interpolated heading turns a row's direction by at most this.
 constexpr float kMaxPathTurn = 0.78539816339744831f;  // pi / 4
 
-// ------------------------------------------------------------------- noise
-// Philox4x32-10 (Salmon, Moraes, Dror, Shaw, SC'11): ten rounds of two 32x32
-// multiplies; the key advances by the two Weyl increments between rounds.
-__device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint32_t k0, uint32_t k1) {
-#pragma unroll
-  for (int r = 0; r < 10; ++r) {
-    const uint32_t lo0 = 0xD2511F53u * c.x;
-    const uint32_t hi0 = __umulhi(0xD2511F53u, c.x);
-    const uint32_t lo1 = 0xCD9E8D57u * c.z;
-    const uint32_t hi1 = __umulhi(0xCD9E8D57u, c.z);
-    c = make_uint4(hi1 ^ c.y ^ k0, lo1, hi0 ^ c.w ^ k1, lo0);
-    k0 += 0x9E3779B9u;
-    k1 += 0xBB67AE85u;
-  }
-  return c;
-}
-
-// Two words -> two standard normals (Box-Muller). Uniform map
-// u = ((w >> 9) + 1/2) 2^-23 in (0, 1), exact in binary32.  It is formed
-// from bits, without an integer-to-float conversion: the float with
-// exponent 0 and mantissa w >> 9 is 1 + (w >> 9) 2^-23, and subtracting
-// 1 - 2^-24 from it is exact (Sterbenz: the operands are within a factor of
-// two).  The angle 2 pi u_b is reduced from the bits of w_b >> 9 too
-// (unit_turn_sincos).
-__device__ __forceinline__ void box_muller(uint32_t wa, uint32_t wb, float& n0, float& n1) {
-  const float ua = __uint_as_float(0x3f800000u | (wa >> 9)) - 0.999999940395355224609375f;
-  // -2 ln ua lies in [1.2e-7, 33.3] (normal floats), taken without a
-  // branch (neg2_log_unit); the radius as x rsqrt(x), no slow path
-  const float r2 = neg2_log_unit(ua);
-  const float radius = r2 * rsqrtf(r2);
-  float sn, cs;
-  unit_turn_sincos(wb >> 9, &sn, &cs);
-  n0 = radius * cs;
-  n1 = radius * sn;
-}
-
 __device__ __forceinline__ float clampf(float v, float lo, float hi) { return fminf(fmaxf(v, lo), hi); }
 
 
-// into [-pi, pi]; only the square of the result is used.  The turn count
-// is rounded by the 1.5 * 2^23 shifter (as rintf for |a| < 2^22 2 pi; no
-// rounding instruction)
-__device__ __forceinline__ float wrap_pi(float a) {
-  const float n = (a * 0.15915494309189533577f + 12582912.0f) - 12582912.0f;
-  return a - 6.28318530717958647692f * n;
-}
-
-template <int TPS>
-__device__ __forceinline__ float team_sum(float v) {
-#pragma unroll
-  for (int m = 1; m < TPS; m <<= 1) v += __shfl_xor_sync(0xffffffffu, v, m, TPS);
-  return v;
-}
-
-template <int TPS>
-__device__ __forceinline__ float team_bcast0(float v) {
+// the value held by lane `src` mod TPS of the team
+template <int TPS, int N>
+__device__ __forceinline__ Vec<N> team_take(Vec<N> v, int src) {
   if constexpr (TPS == 1) return v;
-  return __shfl_sync(0xffffffffu, v, 0, TPS);
+  return vmap(v, [=](float x) { return __shfl_sync(0xffffffffu, x, src & (TPS - 1), TPS); });
+}
+
+template <int TPS, int N>
+__device__ __forceinline__ Vec<N> team_sum(Vec<N> v) {
+#pragma unroll
+  for (int m = 1; m < TPS; m <<= 1) v = v + vshfl_xor(v, m);
+  return v;
 }
 
 // (h, l) pairs: lexicographic order of normalised pairs
@@ -219,15 +202,6 @@ __device__ __forceinline__ bool pair_less(float ah, float al, float bh, float bl
 __device__ __forceinline__ void split_double(double x, float& hi, float& lo) {
   hi = static_cast<float>(x);
   lo = static_cast<float>(x - static_cast<double>(hi));
-}
-
-// Compensated accumulation (TwoSum): (h, l) += inc with the rounding error
-// of the float sum carried in l.
-__device__ __forceinline__ void acc2(float& h, float& l, float inc) {
-  const float sum = h + inc;
-  const float bp = sum - h;
-  l += (h - (sum - bp)) + (inc - bp);
-  h = sum;
 }
 
 // Barrier-rate row of the hitch barrier h = dtheta_max - kappa v - |Delta|,
@@ -391,29 +365,31 @@ struct Smem {
                  // stored negated) and the velocity in the obstacle frame
                  // (zero unless moving)
   float* path;   // 3 per row: x, y, heading (relative frame)
-  float* phead;  // 2 per row: cos, sin of the row's heading in world axes
-  float* unom;   // 3H
+  float* unom;   // 3H: the nominal inputs in the projection's coordinates
   float* ustar;  // 3H + 1 (merge)
   float* jh;     // spb
   float* jl;     // spb
   float* w;      // spb
   float* chunk;  // 256
   float* disc;   // 16: lever arms (along e1, along e2) of the footprint discs
+  float* tab;    // NoiseTables
+  uint4* blk;    // kMaxBlocks: the Philox blocks' shared words
   float* noise;  // spb x noise_per_team, then (exact-rows variants) the
                  // applied-input history, 3H x spb
   int noise_per_team;
   __device__ Smem(float* base, const SmemCaps& c, int spb) {
     obs = base;
     path = obs + c.obs;
-    phead = path + c.path;
-    unom = phead + c.phead;
+    unom = path + c.path;
     ustar = unom + c.unom;
     jh = ustar + c.ustar;
     jl = jh + spb;
     w = jl + spb;
     chunk = jh + SmemCaps::pad4(3 * spb);
     disc = chunk + 256;
-    noise = disc + 16;
+    tab = disc + 16;
+    blk = reinterpret_cast<uint4*>(tab + kNoiseTableFloats);
+    noise = tab + kNoiseTableFloats + 4 * kMaxBlocks;
     noise_per_team = c.noise_per_team;
   }
 };
@@ -433,6 +409,11 @@ __device__ __forceinline__ void cp_async4(float* smem_dst, const float* gmem_src
   const unsigned d = static_cast<unsigned>(__cvta_generic_to_shared(smem_dst));
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(gmem_src) : "memory");
 }
+// 16-byte asynchronous copy global -> shared through L2 (cp.async.cg).
+__device__ __forceinline__ void cp_async16(float* smem_dst, const float* gmem_src) {
+  const unsigned d = static_cast<unsigned>(__cvta_generic_to_shared(smem_dst));
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(gmem_src) : "memory");
+}
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // L2 prefetch of a global address (no value; null-safe).  Issued early for
@@ -441,9 +422,6 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 __device__ __forceinline__ void prefetch_l2(const void* p) {
   if (p) asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
 }
-
-// grad h . e1' in the obstacle frame.
-__device__ __forceinline__ float gda3(float hx, float hy, float dirx, float diry) { return hx * dirx + hy * diry; }
 
 // Threads of a CTA that roll out samples: all of them with one lane per
 // sample; with wider teams the last noise_warps warps produce the noise.
@@ -454,26 +432,113 @@ __device__ __forceinline__ int compute_threads(int noise_warps) {
 
 // Variants whose noise comes from producer warps: wider teams with at most
 // two Philox blocks per lane.
-template <int TPS, int BPT>
-constexpr bool kNoiseWarps = TPS > 1 && BPT <= 2;
+template <int TPS, int BPT, int NS>
+constexpr bool kNoiseWarps = TPS > 1 && BPT <= 2 && NS == 1;
+
+__device__ __forceinline__ void store_pair(float* d, Vec<1> a) { *d = a.x; }
+__device__ __forceinline__ void store_pair(float* d, Vec<2> a) { *reinterpret_cast<float2*>(d) = a.x; }
+
+// The reference path into shared memory, three floats a row (x, y, heading):
+// the raw rows in flight, then (after a barrier) their shift into the frame.
+__device__ __forceinline__ void stage_path(const Inst& in, const Smem& S) {
+  for (int j = threadIdx.x; j < 3 * in.n_pts; j += blockDim.x) cp_async4(S.path + j, in.path + j);
+}
+__device__ __forceinline__ void shift_path(const Inst& in, const Smem& S, const Frame& fr) {
+  for (int j = threadIdx.x; j < in.n_pts; j += blockDim.x) {
+    float* d = S.path + 3 * j;
+    d[0] = (d[0] - fr.ox_h) - fr.ox_l;
+    d[1] = (d[1] - fr.oy_h) - fr.oy_l;
+    d[2] = (d[2] - fr.oth_h) - fr.oth_l;
+  }
+}
+
+// The noise's tables and the Philox blocks' shared words.
+__device__ __forceinline__ void stage_noise(const Inst& in, const Smem& S) {
+  const float* t = reinterpret_cast<const float*>(&kNoiseTables);
+  for (int j = 4 * static_cast<int>(threadIdx.x); j < kNoiseTableFloats; j += 4 * static_cast<int>(blockDim.x))
+    cp_async16(S.tab + j, t + j);
+  for (int b = threadIdx.x; b < in.P; b += blockDim.x) {
+    const PhiloxBlock pb = philox_block(static_cast<uint32_t>(b), in.ctr, in.key0, in.key1);
+    S.blk[b] = make_uint4(pb.a, pb.b, pb.c, 0u);
+  }
+}
+__device__ __forceinline__ PhiloxBlock load_block(const Smem& S, int b) {
+  const uint4 v = S.blk[b];
+  return {v.x, v.y, v.z, v.w};
+}
 
 // The per-step hand-over between the noise warp and the compute warps
 // (named barrier 1, every thread of the CTA; whole warps take one role).
 __device__ __forceinline__ void step_barrier() { asm volatile("bar.sync 1, %0;" ::"r"(blockDim.x) : "memory"); }
 
+// A row's state between steps (variants without producer warps): its rate
+// less the part in y, and its columns u and (EXT) w.
+template <bool EXT, int NS>
+constexpr int kRowFloats = EXT ? 4 * NS : 2 * NS;
+constexpr int kMaxRowSlots = 32;  // a lane's rows: 4 per Philox block, at most 8 blocks
+template <bool EXT, int NS>
+__device__ __forceinline__ void store_row(float* p, Vec<NS> al, Vec<NS> u, Vec<NS> w) {
+  if constexpr (NS == 1) {
+    if constexpr (EXT) *reinterpret_cast<float4*>(p) = make_float4(al.x, u.x, w.x, 0.f);
+    else *reinterpret_cast<float2*>(p) = make_float2(al.x, u.x);
+  } else {
+    *reinterpret_cast<float4*>(p) = make_float4(al.x.x, al.x.y, u.x.x, u.x.y);
+    if constexpr (EXT) *reinterpret_cast<float2*>(p + 4) = w.x;
+  }
+}
+template <bool EXT, int NS>
+__device__ __forceinline__ void load_row(const float* p, Vec<NS>& al, Vec<NS>& u, Vec<NS>& w) {
+  if constexpr (NS == 1) {
+    if constexpr (EXT) {
+      const float4 v = *reinterpret_cast<const float4*>(p);
+      al = v.x;
+      u = v.y;
+      w = v.z;
+    } else {
+      const float2 v = *reinterpret_cast<const float2*>(p);
+      al = v.x;
+      u = v.y;
+    }
+  } else {
+    const float4 v = *reinterpret_cast<const float4*>(p);
+    al = Vec<NS>(make_float2(v.x, v.y));
+    u = Vec<NS>(make_float2(v.z, v.w));
+    if constexpr (EXT) w = Vec<NS>(*reinterpret_cast<const float2*>(p + 4));
+  }
+}
+
+// Sampled augmented input in the projection's coordinates.  The projection
+// starts from M^-1 p with p = W z_des + rho/2 (z_hi + z_lo) and
+// z_des = clip(U_nom + sigma n): a rising affine map of a clip is the clip of
+// the mapped value between the mapped bounds, so one fused multiply-add and
+// a clip give it, from the nominal input mapped once while it is staged.
+// The rate inputs' p_alpha / m_alpha likewise.  Without the projection the
+// map is the identity (KConst::qa, qb).
+template <int N>
+__device__ __forceinline__ Vec<N> sampled_input(const KConst& k, int j, float q_nom, Vec<N> n) {
+  return vclamp(fma(Vec<N>(k.qs[j]), n, Vec<N>(q_nom)), k.qlo[j], k.qhi[j]);
+}
+template <int N>
+__device__ __forceinline__ Vec<N> sampled_rate(const KConst& k, Vec<N> n) {
+  return vclamp(fma(Vec<N>(k.ps), n, Vec<N>(k.pc_am)), k.pam_lo, k.pam_hi);
+}
+
 // ----------------------------------------------------------- one sample tile
-template <int TPS, int BPT, bool EXT, int ROWS>
+// NS: samples a team rolls out together (Vec<NS>).
+// LOCAL: the rows' state in local memory (in place of shared memory).
+template <int TPS, int BPT, bool EXT, int ROWS, int NS, bool LOCAL>
 __device__ void run_tile(const KConst& k, const Inst& in, int tile, float* uh, const Smem& S,
                          Shared& sh, int noise_warps) {
+  using T = Vec<NS>;
   // Teams wider than one lane run with extra warps (the last ones) that
   // produce every team's normals a step ahead (warp specialisation: the
   // noise leaves the compute warps' dependency chain).
   const int nc = compute_threads<TPS>(noise_warps);
-  const int spb = nc / TPS;
-  const bool producer = kNoiseWarps<TPS, BPT> && static_cast<int>(threadIdx.x) >= nc;
+  const int spb = nc / TPS * NS;
+  const bool producer = kNoiseWarps<TPS, BPT, NS> && static_cast<int>(threadIdx.x) >= nc;
   const int team = producer ? 0 : static_cast<int>(threadIdx.x) / TPS;
   const int lt = threadIdx.x % TPS;
-  const int s = tile * spb + team;
+  const int s = tile * spb + team * NS;  // the team's first sample
   const int H = in.H;
   const int n_rows = EXT ? in.n_obs * k.nd : in.n_obs;  // obstacle rows (obstacle x disc)
 
@@ -491,7 +556,8 @@ __device__ void run_tile(const KConst& k, const Inst& in, int tile, float* uh, c
   // shift into the frame follows the barrier.
   const bool obs8 = EXT && k.obs8;
   const int ostride = obs8 ? 8 : 6;
-  for (int j = threadIdx.x; j < 3 * in.n_pts; j += blockDim.x) cp_async4(S.path + j, in.path + j);
+  stage_path(in, S);
+  stage_noise(in, S);
   for (int j = threadIdx.x; j < 3 * H; j += blockDim.x) cp_async4(S.unom + j, in.U_nom + j);
   float ob0[8];
   const bool has_ob0 = static_cast<int>(threadIdx.x) < in.n_obs;
@@ -529,23 +595,20 @@ __device__ void run_tile(const KConst& k, const Inst& in, int tile, float* uh, c
       d[7] = co * vy - so * vx;
     }
   };
+  // one row past the obstacles: h = -1 everywhere with no gradient, so a
+  // padding slot that reads it adds exactly nothing to the projection's sums
+  if (threadIdx.x < 8) S.obs[8 * in.n_obs + threadIdx.x] = 0.f;
   if (has_ob0) stage_obstacle(threadIdx.x, ob0[0], ob0[1], ob0[2], ob0[3], ob0[4], ob0[5], ob0[6], ob0[7]);
   for (int o = threadIdx.x + blockDim.x; o < in.n_obs; o += blockDim.x) {
     const float* ob = in.obs + ostride * o;
     stage_obstacle(o, ob[0], ob[1], ob[2], ob[3], ob[4], ob[5], obs8 ? ob[6] : 0.f, obs8 ? ob[7] : 0.f);
   }
-  for (int j = threadIdx.x; j < in.n_pts; j += blockDim.x) {
-    float* d = S.path + 3 * j;
-    d[0] = (d[0] - fr.ox_h) - fr.ox_l;
-    d[1] = (d[1] - fr.oy_h) - fr.oy_l;
-    const float th = (d[2] - fr.oth_h) - fr.oth_l;
-    d[2] = th;
-    // the row's heading direction in world axes, once per solve: the stage
-    // cost turns it by the interpolation angle instead of a sincos per step
-    float st, ct;
-    sincosf(th, &st, &ct);
-    *reinterpret_cast<float2*>(S.phead + 2 * j) = make_float2(fr.c0 * ct - fr.s0 * st, fr.s0 * ct + fr.c0 * st);
+  shift_path(in, S, fr);
+  for (int j = threadIdx.x; j < 3 * H; j += blockDim.x) {  // nominal inputs in the projection's coordinates
+    const int q = j % 3;
+    S.unom[j] = fmaf(k.qa[q], S.unom[j], k.qb[q]);
   }
+  if (threadIdx.x < 4) S.chunk[threadIdx.x] = k.pc_am;  // (free until the merge)
   if constexpr (EXT) {
 #pragma unroll
     for (int m = 0; m < 8; ++m)
@@ -557,213 +620,353 @@ __device__ void run_tile(const KConst& k, const Inst& in, int tile, float* uh, c
   __syncthreads();
 
   // --- per-sample state (relative frame)
-  const float c0 = fr.c0, s0 = fr.s0;
-  float acc = fr.a0;  // acceleration state of the jerk-input model
-  float px = 0.f, pxl = 0.f, py = 0.f, pyl = 0.f, t1 = 0.f, t2 = fr.t2, v = fr.v_h, vl = fr.v_l,
-        dl = fr.dl, ps = 0.f, psl = 0.f;
-  // obstacle slots per lane: one lane per sample holds every obstacle of
-  // its Philox blocks 1.. ; wider teams hold obstacles lt, lt + TPS, ...;
-  // ROWS > 0 (latency variants with noise warps): exactly ROWS slots a lane
-  static_assert(ROWS == 0 || kNoiseWarps<TPS, BPT>, "exact row slots need the noise-warp variants");
-  constexpr int OBS_SLOTS = ROWS > 0 ? ROWS : ((TPS == 1) ? (BPT > 1 ? 4 * (BPT - 1) : 1) : 4 * BPT);
-  float alpha_h = k.alpha0;  // the hitch's barrier rate (same on every lane)
-  float alpha[OBS_SLOTS];
+  const T c0 = fr.c0, s0 = fr.s0;
+  T acc = fr.a0;  // acceleration state of the jerk-input model
+  T px = 0.f, pxl = 0.f, py = 0.f, pyl = 0.f, t1 = 0.f, t2 = fr.t2, v = fr.v_h, vl = fr.v_l, dl = fr.dl, ps = 0.f,
+    psl = 0.f;
+  // obstacle slots per lane of the producer variants: 4 BPT; ROWS > 0: exactly
+  // ROWS
+  static_assert(ROWS == 0 || kNoiseWarps<TPS, BPT, NS>, "exact row slots need the noise-warp variants");
+  constexpr bool PRODUCED = kNoiseWarps<TPS, BPT, NS>;
+  constexpr int OBS_SLOTS = !PRODUCED ? 1 : (ROWS > 0 ? ROWS : 4 * BPT);
+  T alpha_h = k.alpha0;  // the hitch's barrier rate (same on every lane)
+  T alpha[OBS_SLOTS];    // the rows' rates (producer variants: in registers)
 #pragma unroll
   for (int q = 0; q < OBS_SLOTS; ++q) alpha[q] = k.alpha0;
-  float Jh = 0.f, Jl = 0.f;
-  float ua = 0.f, uw = 0.f, un = 0.f;  // applied input of the previous step
+  // Other variants keep a row's state (its rate without the part in y, and
+  // its columns u, w of the step before) in shared memory, one float4 a row
+  // and lane (EXT: also the w column): the pass over the team's Philox blocks is then a loop of one body
+  // for any number of rows.  Rows in registers need it unrolled: at 16 rows
+  // a lane the step was 50 KB of code and waited for instructions (stall 0.8
+  // an issue), and 64 registers more a lane cost a third of the warps.
+  float local_rows[LOCAL ? 4 * kMaxRowSlots * NS : 1];
+  const int row_stride = LOCAL ? kRowFloats<EXT, NS> : kRowFloats<EXT, NS> * static_cast<int>(blockDim.x);
+  float* rows = LOCAL ? local_rows : S.noise + kRowFloats<EXT, NS> * static_cast<int>(threadIdx.x);
+  const int passes = (in.P - 1 + TPS - 1) / TPS;  // Philox blocks 1 .. P - 1 over the team's lanes
+  if constexpr (!PRODUCED)
+    for (int q = 0; q < 4 * passes; ++q) store_row<EXT, NS>(rows + q * row_stride, T(k.alpha0), T(0.f), T(0.f));
+  T ya_p = 0.f, yw_p = 0.f;  // the step before's y
+  T Jh = 0.f, Jl = 0.f;
+  T ua = 0.f, uw = 0.f, un = 0.f;  // applied input of the previous step
   const uint32_t sid = static_cast<uint32_t>(s);
   const int n_pts = in.n_pts;
-  const float qf0 = fr.qf0;
+  const T qf0 = fr.qf0;
   const int i0 = fr.i0;
 
-  // the four normals of Philox block b at step tau
-  auto draw_block = [&](int b, int tau, float* out) {
-    const uint4 w = philox4x32_10(
-        make_uint4(static_cast<uint32_t>(b), static_cast<uint32_t>(tau), sid, in.ctr), in.key0, in.key1);
-    box_muller(w.x, w.y, out[0], out[1]);
-    box_muller(w.z, w.w, out[2], out[3]);
+  // the four normals of Philox block b, given the step's words of the samples
+  PhiloxSample smp[NS];
+#pragma unroll
+  for (int i = 0; i < NS; ++i) smp[i] = philox_sample(sid + i);
+  struct StepWords {
+    PhiloxStep w[NS];
   };
-  // block 0 of this lane (lane 0: the input normals and the hitch), drawn a
-  // step ahead; further blocks are drawn where their rows are built
-  auto draw_first = [&](int tau, float* out) {
-    if (lt < in.P) {
-      draw_block(lt, tau, out);
-    } else {
-      out[0] = out[1] = out[2] = out[3] = 0.f;
+  auto step_words = [&](int tau) {
+    StepWords r;
+#pragma unroll
+    for (int i = 0; i < NS; ++i) r.w[i] = philox_step(smp[i], static_cast<uint32_t>(tau), in.key0, in.key1);
+    return r;
+  };
+  auto draw_block = [&](int b, const StepWords& st, T* out) {
+    const PhiloxBlock pb = load_block(S, b);
+    uint32_t x[NS], y[NS], z[NS], w[NS];
+#pragma unroll
+    for (int i = 0; i < NS; ++i) {
+      const uint4 v = philox_words(pb, smp[i], st.w[i], in.key0, in.key1);
+      x[i] = v.x;
+      y[i] = v.y;
+      z[i] = v.z;
+      w[i] = v.w;
     }
+    box_muller<NS>(x, y, S.tab, out[0], out[1]);
+    box_muller<NS>(z, w, S.tab, out[2], out[3]);
   };
 
   // barrier of constraint row j (obstacle o seen from footprint disc m) at
   // the current state and time t (Eq. barrier_function; moving centres at
   // c + t v); (ce1, se1) and (ce2, se2) the unit headings of the state
-  auto row_h = [&](int j, float t, float ce1, float se1, float ce2, float se2) -> float {
+  auto row_h = [&](int j, float t, T ce1, T se1, T ce2, T se2) -> T {
     const int o = (k.nd == 1) ? j : __float2int_rz((static_cast<float>(j) + 0.5f) * k.inv_nd);
     const int m = j - o * k.nd;
     const float4 o0 = *reinterpret_cast<const float4*>(S.obs + 8 * o);
     const float4 o1 = *reinterpret_cast<const float4*>(S.obs + 8 * o + 4);
     const float2 lv = *reinterpret_cast<const float2*>(S.disc + 2 * m);
-    const float dx = (px - o0.x) + pxl + lv.x * ce1 + lv.y * ce2;
-    const float dy = (py - o0.y) + pyl + lv.x * se1 + lv.y * se2;
-    const float xp = o0.z * dx + o0.w * dy - t * o1.z;
-    const float yp = o0.z * dy - o0.w * dx - t * o1.w;
+    const T dx = fma(T(lv.y), ce2, fma(T(lv.x), ce1, (px - T(o0.x)) + pxl));
+    const T dy = fma(T(lv.y), se2, fma(T(lv.x), se1, (py - T(o0.y)) + pyl));
+    const T xp = fma(T(o0.z), dx, fma(T(o0.w), dy, T(-t * o1.z)));
+    const T yp = fma(T(o0.z), dy, fma(T(-o0.w), dx, T(-t * o1.w)));
     const bool e4 = o1.x < 0.f;
-    const float kx = fabsf(o1.x), ky = o1.y;
-    const float X = e4 ? xp * xp * kx : kx, Y = e4 ? yp * yp * ky : ky;
-    return xp * xp * X + yp * yp * Y - 1.f;
+    const T kx = fabsf(o1.x), ky = o1.y;
+    const T x2 = xp * xp, y2 = yp * yp;
+    const T X = e4 ? x2 * kx : kx, Y = e4 ? y2 * ky : ky;
+    return fma(x2, X, fma(y2, Y, T(-1.f)));
   };
 
-  // stage cost of the current state (time t) reached with input (ua, uw, un);
-  // add = false computes it and adds zero (no branch in the step)
-  auto stage_cost = [&](float t, float ce1, float se1, float ce2, float se2, bool add) {
-    const float qf = qf0 + (ps * in.inv_ds + psl * in.inv_ds);
-    const float fl = floorf(qf);
-    int ii = i0 + static_cast<int>(fl);
-    float ff = qf - fl;
-    if (ii < 0) {
-      ii = 0;
-      ff = 0.f;
-    } else if (ii > n_pts - 2) {
-      ii = n_pts - 2;
-      ff = 1.f;
+  // Stage cost of state (px .. psl) reached with input (ua, uw, un).  With
+  // equal contour and lag weights (KConst::iso, the default)
+  // Qc e_c^2 + Ql e_l^2 is the weighted distance to the path point, whatever
+  // the path's direction there: no sin / cos in the cost.
+  struct Visit {
+    T px, pxl, py, pyl, t1, t2, ps, psl, ua, uw, un;
+  };
+  auto stage_cost = [&](const Visit& x) -> T {
+    // path cell: floor of qf by the 1.5 * 2^23 shifter on qf - 1/2 (an exact
+    // integer may take the cell below with ff = 1, the same point); the
+    // clamp keeps the shifter in range far outside any path
+    const T qf = vclamp(qf0 + fma(x.ps, T(in.inv_ds), x.psl * T(in.inv_ds)), -2.0e6f, 2.0e6f);
+    const T tt = (qf + T(-0.5f)) + T(12582912.0f);
+    T ff = qf - (tt + T(-12582912.0f));
+    T x0r, y0r, t0r, x1r, y1r, t1r;
+#pragma unroll
+    for (int i = 0; i < NS; ++i) {
+      int ii = i0 + (__float_as_int(tt.get(i)) - 0x4b400000);
+      if (ii < 0) {
+        ii = 0;
+        ff.set(i, 0.f);
+      } else if (ii > n_pts - 2) {
+        ii = n_pts - 2;
+        ff.set(i, 1.f);
+      }
+      const float* r = S.path + 3 * ii;
+      x0r.set(i, r[0]);
+      y0r.set(i, r[1]);
+      t0r.set(i, r[2]);
+      x1r.set(i, r[3]);
+      y1r.set(i, r[4]);
+      t1r.set(i, r[5]);
     }
-    const float* r0 = S.path + 3 * ii;
-    const float xr = r0[0] + ff * (r0[3] - r0[0]);
-    const float yr = r0[1] + ff * (r0[4] - r0[1]);
-    const float eps = ff * (r0[5] - r0[2]);  // turn from row ii to the interpolated heading
-    const float thr = r0[2] + eps;
-    const float2 hd = *reinterpret_cast<const float2*>(S.phead + 2 * ii);
-    float se, ce;
-    turn_sincos(eps, &se, &ce);
-    const float cth = hd.x * ce - hd.y * se;  // cos / sin of the heading in world axes
-    const float sth = hd.y * ce + hd.x * se;
-    const float dxr = (px - xr) + pxl, dyr = (py - yr) + pyl;
-    const float ec = sth * dxr - cth * dyr;
-    const float el = -cth * dxr - sth * dyr;
-    const float e1 = wrap_pi(t1 - thr), e2 = wrap_pi(t2 - thr);
-    const float dn = k.nu_bar - un;
-    float rc = k.Qc * ec * ec + k.Ql * el * el + k.Qth * (e1 * e1 + e2 * e2) + k.R0 * ua * ua +
-               k.R1 * uw * uw + k.R2 * un * un + k.mu * dn * dn;
-    if (EXT && k.coll) {
-      // the comparison method's collision penalty: depth of every
-      // obstacle the state is inside (obstacles spread over the team)
-      float c = 0.f;
-      for (int j = lt; j < n_rows; j += TPS) c += fmaxf(-row_h(j, t, ce1, se1, ce2, se2), 0.f);
-      rc += k.q_coll * team_sum<TPS>(c);
+    const T xr = fma(ff, x1r - x0r, x0r), yr = fma(ff, y1r - y0r, y0r), thr = fma(ff, t1r - t0r, t0r);
+    const T dxr = (x.px - xr) + x.pxl, dyr = (x.py - yr) + x.pyl;
+    T rc;
+    if (k.iso) {
+      rc = T(k.Ql) * fma(dxr, dxr, dyr * dyr);
+    } else {
+      T sr, cr;
+      state_sincos(thr, &sr, &cr);
+      const T cth = fma(c0, cr, -(s0 * sr)), sth = fma(s0, cr, c0 * sr);  // the path's heading in world axes
+      const T ec = fma(sth, dxr, -(cth * dyr)), el = fma(cth, dxr, sth * dyr);
+      rc = fma(T(k.Ql) * el, el, T(k.Qc) * ec * ec);
     }
-    acc2(Jh, Jl, add ? rc : 0.f);
+    const T e1 = wrap_pi(x.t1 - thr), e2 = wrap_pi(x.t2 - thr);
+    const T dn = T(k.nu_bar) - x.un;
+    rc = fma(T(k.Qth), fma(e1, e1, e2 * e2), rc);
+    rc = fma(T(k.R0) * x.ua, x.ua, rc);
+    rc = fma(T(k.R1) * x.uw, x.uw, rc);
+    rc = fma(T(k.R2) * x.un, x.un, rc);
+    return fma(T(k.mu) * dn, dn, rc);
+  };
+  auto visit = [&]() { return Visit{px, pxl, py, pyl, t1, t2, ps, psl, ua, uw, un}; };
+  // The cost of a sample is summed over its team: in teams lane
+  // (tau - 1) mod TPS keeps the state after step tau, and once every TPS
+  // steps each lane evaluates the cost of the state it kept -- one cost
+  // sequence in the warp's stream in place of TPS copies of it.
+  // The producer variants (one compute warp a scheduler) evaluate it every
+  // step on every lane instead: a branch in their step costs more than the
+  // copies do (control solve of 4096 samples, H = 50: 40.0 us without the
+  // branch, 43.0 us with it).
+  constexpr bool SHARE = TPS > 1 && !kNoiseWarps<TPS, BPT, NS>;
+  Visit kept = visit();
+  auto cost_after = [&](int tau) {  // the state reached by step tau - 1
+    if constexpr (!SHARE) {
+      const T rc = stage_cost(visit());  // none before the first step: zero is added
+      acc2(Jh, Jl, tau > 0 ? rc : T(0.f));
+    } else {
+      if (lt == ((tau - 1) & (TPS - 1))) kept = visit();
+      if (tau > 0 && (tau & (TPS - 1)) == 0) acc2(Jh, Jl, stage_cost(kept));
+    }
+  };
+  // parts of the cost that every lane has its share of, summed over the team
+  // at the end
+  T Xh = 0.f, Xl = 0.f;
+  auto add_share = [&](T c) { acc2(Xh, Xl, c); };
+  // the comparison method's collision penalty at the current state (time
+  // t): depth of every obstacle it is inside (obstacles spread over the team)
+  auto collision_cost = [&](float t, T ce1, T se1, T ce2, T se2) {
+    T c = 0.f;
+    auto depth = [&](int j) {
+      c = c + vmap(row_h(j, t, ce1, se1, ce2, se2), [](float h) { return fmaxf(-h, 0.f); });
+    };
+    if constexpr (ROWS > 0) {
+#pragma unroll
+      for (int q = 0; q < ROWS; ++q)
+        if (lt + TPS * q < n_rows) depth(lt + TPS * q);
+    } else {
+      for (int j = lt; j < n_rows; j += TPS) depth(j);
+    }
+    add_share(T(k.q_coll) * c);
   };
 
-  // stored-trajectory variant: the state of this sample after step tau, in
-  // world coordinates (written by the team's first lane)
-  float* st_out = (!producer && in.states_out && lt == 0 && s < in.S)
-                      ? in.states_out + static_cast<size_t>(s) * static_cast<size_t>(H + 1) * 7
-                      : nullptr;
+  // stored-trajectory variant: the states of the team's samples after step
+  // tau, in world coordinates (written by the team's first lane)
+  const bool writer = !producer && lt == 0;
+  const bool st_out = writer && in.states_out, in_out = writer && in.inputs_out;
   auto store_state = [&](int tau) {
-    float* o = st_out + 7 * tau;
-    o[0] = (fr.ox_h + px) + (fr.ox_l + pxl);
-    o[1] = (fr.oy_h + py) + (fr.oy_l + pyl);
-    o[2] = (fr.oth_h + t1) + fr.oth_l;
-    o[3] = (fr.oth_h + t2) + fr.oth_l;
-    o[4] = v + vl;
-    o[5] = dl;
-    o[6] = (fr.psi_h + ps) + (fr.psi_l + psl);
+#pragma unroll
+    for (int i = 0; i < NS; ++i) {
+      if (s + i >= in.S) break;
+      float* o = in.states_out + (static_cast<size_t>(s + i) * static_cast<size_t>(H + 1) + tau) * 7;
+      o[0] = (fr.ox_h + px.get(i)) + (fr.ox_l + pxl.get(i));
+      o[1] = (fr.oy_h + py.get(i)) + (fr.oy_l + pyl.get(i));
+      o[2] = (fr.oth_h + t1.get(i)) + fr.oth_l;
+      o[3] = (fr.oth_h + t2.get(i)) + fr.oth_l;
+      o[4] = v.get(i) + vl.get(i);
+      o[5] = dl.get(i);
+      o[6] = (fr.psi_h + ps.get(i)) + (fr.psi_l + psl.get(i));
+    }
   };
   if (st_out) store_state(0);
-  float* in_out = (!producer && in.inputs_out && lt == 0 && s < in.S)
-                      ? in.inputs_out + static_cast<size_t>(s) * static_cast<size_t>(H) * 3
-                      : nullptr;
 
-  // Noise.  One lane per sample: the lane draws Philox block 0 a step ahead
-  // and the further blocks where their rows are built.  Wider teams: the
-  // producer warp writes the P blocks of every team's step tau + 1 into a
-  // per-team double buffer in shared memory while the compute warps run step
-  // tau; one CTA barrier per step hands the buffers over (at barrier tau the
-  // producer has written step tau and the compute warps have finished step
-  // tau - 1, whose buffer it fills next).  Constraint i is built by lane
-  // i % TPS, so rows spread evenly over the team.
-  float* nz = S.noise + team * S.noise_per_team;  // [2][P][4] (wide teams)
+  // Noise.  Teams of at most two Philox blocks per lane, one sample each (the
+  // latency shapes): the producer warps write what the P blocks of every
+  // team's step tau + 1 sample (inputs and rates) into a per-team double buffer in shared memory while the
+  // compute warps run step tau; one CTA barrier per step hands the buffers
+  // over (at barrier tau the producers have written step tau and the compute
+  // warps have finished step tau - 1, whose buffer is filled next).
+  // Constraint i is built by lane i % TPS, so rows spread evenly over the team.
+  //
+  // Other shapes draw in registers, where the normals are used: lane lt owns
+  // Philox blocks 1 + lt, 1 + lt + TPS, ... and builds their rows.  Block 0
+  // (inputs and hitch) is needed by the whole team: lane lt draws it for step
+  // tau + lt once every TPS steps, and each step takes it from its lane.
+  float* nz = S.noise + team * S.noise_per_team;  // [2][P][4] (producer variants)
   const int P_drawn = k.proj ? in.P : 1;  // standard MPPI needs the input normals only
-  // Variants with more than two blocks per lane (many constraints) stage
-  // them on the team's own lanes instead (blocks b = lt, lt + TPS, ...): a
-  // producer would need more warps than the CTA can hold.
-  constexpr bool lane_staged = TPS > 1 && !kNoiseWarps<TPS, BPT>;
-  auto stage_step = [&](int tau_d, float* buf) {
-    for (int b = lt; b < P_drawn; b += TPS) {
-      float t4[4];
-      draw_block(b, tau_d, t4);
-      *reinterpret_cast<float4*>(buf + 4 * b) = make_float4(t4[0], t4[1], t4[2], t4[3]);
-    }
-  };
-  if constexpr (lane_staged) stage_step(0, nz);
-  if constexpr (kNoiseWarps<TPS, BPT>) {
+  if constexpr (kNoiseWarps<TPS, BPT, NS>) {
     if (producer) {
+      // thread pl draws block i of the CTA's spb P_drawn each step, i = pl,
+      // pl + 32 noise_warps, ...; with at most one block a thread (the usual
+      // case) what the steps share stays in registers
       const int pl = static_cast<int>(threadIdx.x) - nc;
-      const int n_blocks = spb * P_drawn;
-      auto produce = [&](int tau_d) {
-        for (int i = pl; i < n_blocks; i += 32 * noise_warps) {
-          const int tm = i / P_drawn, b = i - tm * P_drawn;
-          const uint4 w = philox4x32_10(make_uint4(static_cast<uint32_t>(b), static_cast<uint32_t>(tau_d),
-                                                   static_cast<uint32_t>(tile * spb + tm), in.ctr),
-                                        in.key0, in.key1);
-          float4 g;
-          box_muller(w.x, w.y, g.x, g.y);
-          box_muller(w.z, w.w, g.z, g.w);
-          *reinterpret_cast<float4*>(S.noise + tm * S.noise_per_team + (tau_d & 1) * 4 * in.P + 4 * b) = g;
-        }
+      const int n_blocks = spb * P_drawn, stride = 32 * noise_warps;
+      // what block b's normals sample: block 0 the inputs (around the nominal
+      // ones) and the hitch's rate, others four rows' rates
+      struct Draw {
+        PhiloxBlock pb;
+        PhiloxSample smp;
+        float s0, s1, s2, lo0, lo1, lo2, hi0, hi1, hi2;
+        const float* nom;
+        int nom_stride;
+        float* dst;
       };
-      produce(0);
-      for (int tau = 0; tau < H; ++tau) {
-        step_barrier();
-        if (tau + 1 < H) produce(tau + 1);
+      auto make_draw = [&](int i) {
+        const int tm = i / P_drawn, b = i - tm * P_drawn;
+        const bool first = b == 0;
+        Draw d;
+        d.pb = load_block(S, b);
+        d.smp = philox_sample(static_cast<uint32_t>(tile * spb + tm));
+        d.s0 = first ? k.qs[0] : k.ps;
+        d.s1 = first ? k.qs[1] : k.ps;
+        d.s2 = first ? k.qs[2] : k.ps;
+        d.lo0 = first ? k.qlo[0] : k.pam_lo;
+        d.lo1 = first ? k.qlo[1] : k.pam_lo;
+        d.lo2 = first ? k.qlo[2] : k.pam_lo;
+        d.hi0 = first ? k.qhi[0] : k.pam_hi;
+        d.hi1 = first ? k.qhi[1] : k.pam_hi;
+        d.hi2 = first ? k.qhi[2] : k.pam_hi;
+        d.nom = first ? S.unom : S.chunk;
+        d.nom_stride = first ? 3 : 0;
+        d.dst = S.noise + tm * S.noise_per_team + 4 * b;
+        return d;
+      };
+      auto produce = [&](const Draw& d, int tau_d) {
+        const uint4 w = philox_words(d.pb, d.smp, philox_step(d.smp, static_cast<uint32_t>(tau_d), in.key0, in.key1),
+                                     in.key0, in.key1);
+        const float* nom = d.nom + tau_d * d.nom_stride;
+        Vec<1> g0, g1, g2, g3;
+        box_muller<1>(&w.x, &w.y, S.tab, g0, g1);
+        box_muller<1>(&w.z, &w.w, S.tab, g2, g3);
+        g0 = vclamp(fma(Vec<1>(d.s0), g0, Vec<1>(nom[0])), d.lo0, d.hi0);
+        g1 = vclamp(fma(Vec<1>(d.s1), g1, Vec<1>(nom[1])), d.lo1, d.hi1);
+        g2 = vclamp(fma(Vec<1>(d.s2), g2, Vec<1>(nom[2])), d.lo2, d.hi2);
+        g3 = sampled_rate(k, g3);
+        *reinterpret_cast<float4*>(d.dst + (tau_d & 1) * 4 * in.P) = make_float4(g0.x, g1.x, g2.x, g3.x);
+      };
+      if (n_blocks <= stride) {
+        const Draw d = make_draw(min(pl, n_blocks - 1));
+        const bool mine = pl < n_blocks;
+        if (mine) produce(d, 0);
+        for (int tau = 0; tau < H; ++tau) {
+          step_barrier();
+          if (mine && tau + 1 < H) produce(d, tau + 1);
+        }
+      } else {
+        auto produce_all = [&](int tau_d) {
+          for (int i = pl; i < n_blocks; i += stride) produce(make_draw(i), tau_d);
+        };
+        produce_all(0);
+        for (int tau = 0; tau < H; ++tau) {
+          step_barrier();
+          if (tau + 1 < H) produce_all(tau + 1);
+        }
       }
     }
   }
-  float nrm[4];
-  if constexpr (TPS == 1) draw_first(0, nrm);
+  T z0[4];  // in-register noise: this lane's sampled (a, omega, nu) and hitch rate
   // trigonometry of the current state, carried from step to step: the state
   // angles theta1 and phi = theta1 - theta2 of step tau + 1 follow from step
   // tau's state alone (the input enters only the speed, steer angle and
   // progress), so their sin / cos are taken before step tau's projection
   // and stay off its dependency chain; only the steer angle's trigonometry
   // waits for the projection.
-  float c1, s1, sp, cp;
+  T c1, s1, sp, cp;
   {
-    float sr, cr;
+    T sr, cr;
     state_sincos(t1, &sr, &cr);
-    c1 = c0 * cr - s0 * sr;
-    s1 = s0 * cr + c0 * sr;
+    c1 = fma(c0, cr, -(s0 * sr));
+    s1 = fma(s0, cr, c0 * sr);
     state_sincos(t1 - t2, &sp, &cp);
   }
   // One step; PROJ is fixed for the whole loop (no branch on the flag
   // inside the step).
   auto step = [&](int tau, auto proj_c) {
     constexpr bool PROJ = decltype(proj_c)::value;
-    float nxt[4];
-    float* cur = nz;
-    if constexpr (TPS == 1) {
-      draw_first(tau + 1 < H ? tau + 1 : tau, nxt);  // off the state's critical path
-    } else if constexpr (lane_staged) {
-      __syncwarp();  // this step's normals are staged; last step's reads are done
-      cur = nz + (tau & 1) * 4 * in.P;
-      if (tau + 1 < H) stage_step(tau + 1, nz + ((tau + 1) & 1) * 4 * in.P);
-    } else {
+    // the sampled input in the projection's coordinates (M_u^-1 p_u with
+    // the projection, else the sampled input itself) and the hitch's rate
+    T q0, q1, zn, pam_h;
+    const float* cur = nz + (tau & 1) * 4 * in.P;
+    if constexpr (kNoiseWarps<TPS, BPT, NS>) {
       step_barrier();  // this step's normals are staged
-      cur = nz + (tau & 1) * 4 * in.P;
+      const float4 n4 = *reinterpret_cast<const float4*>(cur);
+      q0 = n4.x;
+      q1 = n4.y;
+      zn = n4.z;
+      pam_h = n4.w;
+    } else {
+      if ((tau & (TPS - 1)) == 0) {
+        const int td = TPS == 1 ? tau : min(tau + lt, H - 1);
+        T n4[4];
+        draw_block(0, step_words(td), n4);
+#pragma unroll
+        for (int j = 0; j < 3; ++j) z0[j] = sampled_input(k, j, S.unom[3 * td + j], n4[j]);
+        z0[3] = sampled_rate(k, n4[3]);
+      }
+      q0 = team_take<TPS>(z0[0], tau);
+      q1 = team_take<TPS>(z0[1], tau);
+      zn = team_take<TPS>(z0[2], tau);
+      pam_h = team_take<TPS>(z0[3], tau);
     }
 
     // trigonometry of the steer angle (the one state angle the previous
     // projection moved)
-    float sd, cd;
+    T sd, cd;
     state_sincos(dl, &sd, &cd);
-    const float tn = __fdividef(sd, cd);  // |cos| >= 4e-9 below 2^16: MUFU reciprocal (~2 ulp)
-    const float vv = v + vl;
-    const float th1dot = vv * tn * k.inv_l1;
+    const T tn = sd * vrcp(cd);  // |cos| >= 4e-9 below 2^16: MUFU reciprocal (~2 ulp)
+    const T vv = v + vl;
+    const T tl = tn * T(k.inv_l1);
+    const T th1dot = vv * tl;
 
-    // cost of the previous step, at this state (independent of the rows);
-    // at tau = 0 there is no previous step and the increment is zero
-    // (adding zero to a compensated pair leaves it unchanged)
-    stage_cost(static_cast<float>(tau) * k.Ts, c1, s1, c1 * cp + s1 * sp, s1 * cp - c1 * sp, tau > 0);
+    // cost of the previous step, at this state (independent of the rows)
+    T c2 = 0.f, s2 = 0.f;  // the trailer's heading, where a term needs it
+    if (EXT && k.discs) {
+      c2 = fma(c1, cp, s1 * sp);
+      s2 = fma(s1, cp, -(c1 * sp));
+    }
+    cost_after(tau);
+    if (EXT && k.coll && tau > 0) collision_cost(static_cast<float>(tau) * k.Ts, c1, s1, c2, s2);
+
+    // trailer's heading rate and its parts
+    const T kt = T(k.k_hitch) * tn;
+    const T G = fma(-cp, kt, sp);
+    const T vl2 = vv * T(k.inv_l2);
+    const T th2dot = vl2 * G;
 
     // explicit Euler, the state-only part (right-hand sides at the current
     // state), and the next state's theta1 / phi trigonometry.  Latency
@@ -771,333 +974,281 @@ __device__ void run_tile(const KConst& k, const Inst& in, int tile, float* uh, c
     // chain; one-lane shapes (issue-bound, many warps) after it, so that the
     // current and next values need not be live at once (no register copies
     // at the end of the step)
-    const float Tv = k.Ts * vv;
-    float px_n, pxl_n, py_n, pyl_n, t1_n, t2_n, c1_n, s1_n, sp_n, cp_n;
+    T px_n, pxl_n, py_n, pyl_n, t1_n, t2_n, c1_n, s1_n, sp_n, cp_n;
     auto state_part = [&]() {
+      const T Tv = T(k.Ts) * vv;
       px_n = px;
       pxl_n = pxl;
       py_n = py;
       pyl_n = pyl;
       acc2(px_n, pxl_n, Tv * c1);
       acc2(py_n, pyl_n, Tv * s1);
-      t1_n = t1 + k.Ts * th1dot;
-      t2_n = t2 + Tv * k.inv_l2 * (sp - k.k_hitch * cp * tn);
+      t1_n = fma(T(k.Ts), th1dot, t1);
+      t2_n = fma(T(k.Ts), th2dot, t2);
+      T sr, cr;
       if constexpr (TPS > 1) {
         // even lanes take theta1, odd lanes phi, and each pair trades the
         // results: one sin / cos sequence in the warp's stream instead of two
         const bool odd = lt & 1;
-        float sa, ca;
+        T sa, ca;
         state_sincos(odd ? t1_n - t2_n : t1_n, &sa, &ca);
-        const float sb = __shfl_xor_sync(0xffffffffu, sa, 1);
-        const float cb = __shfl_xor_sync(0xffffffffu, ca, 1);
-        const float sr = odd ? sb : sa, cr = odd ? cb : ca;
+        const T sb = vshfl_xor(sa, 1), cb = vshfl_xor(ca, 1);
+        sr = odd ? sb : sa;
+        cr = odd ? cb : ca;
         sp_n = odd ? sa : sb;
         cp_n = odd ? ca : cb;
-        c1_n = c0 * cr - s0 * sr;
-        s1_n = s0 * cr + c0 * sr;
       } else {
-        float sr, cr;
         state_sincos(t1_n, &sr, &cr);
-        c1_n = c0 * cr - s0 * sr;
-        s1_n = s0 * cr + c0 * sr;
         state_sincos(t1_n - t2_n, &sp_n, &cp_n);
       }
+      c1_n = fma(c0, cr, -(s0 * sr));
+      s1_n = fma(s0, cr, c0 * sr);
     };
     if constexpr (TPS > 1) state_part();
 
-    float na, nw, nn;
-    if constexpr (TPS == 1) {
-      na = nrm[0];
-      nw = nrm[1];
-      nn = nrm[2];
-    } else {
-      na = cur[0];
-      nw = cur[1];
-      nn = cur[2];
-    }
-    const float zd0 = clampf(S.unom[3 * tau + 0] + k.sig0 * na, k.zlo0, k.zhi0);
-    const float zd1 = clampf(S.unom[3 * tau + 1] + k.sig1 * nw, k.zlo1, k.zhi1);
-    const float zd2 = clampf(S.unom[3 * tau + 2] + k.sig2 * nn, k.zlo2, k.zhi2);
-
-    float za, zw, zn;
+    T za = q0, zw = q1;
     if constexpr (PROJ) {
-      const float pu0 = k.w_u0 * zd0 + k.pc_u0;
-      const float pu1 = k.w_u1 * zd1 + k.pc_u1;
-      const float pu2 = k.w_u2 * zd2 + k.pc_u2;
-      const float q0 = pu0 * k.inv_m_u0, q1 = pu1 * k.inv_m_u1;  // M_u^-1 p_u
-      // hitch row: every lane of the team computes it (same state, same
-      // normal); its terms enter the team sums once (lane 0)
-      float Saa, Saw, Sww, ga, gw, ca_h, cw_h, cc_h;
+      // hitch row (Eq. hitch_angle_barrier through the second-order
+      // expansion, as hitch_row states it): every lane of the team computes
+      // it (same state, same normal); its terms enter the sums once, after
+      // the team reduction
+      T u_h, w_h, rho_h, cc_h;
+      const T sec2 = fma(tn, tn, T(1.f));
+      const T phidot = th1dot - th2dot;
+      const T kcl = fma(cp, T(k.khl2), T(k.inv_l1));  // k cos(phi) / l2 + 1 / l1
+      const T bend = fma(kt, sp, cp);                 // cos(phi) + k tan(delta) sin(phi)
       {
-        const float n_h = (TPS == 1) ? nrm[3] : cur[3];
-        HitchRow hr = hitch_row(k, t2 - t1, sp, cp, tn, vv, th1dot);
+        const T Delta = t2 - t1;
+        const T sgT = vmap(Delta, [&](float d) { return copysignf(k.hTs2, d); });
+        const T sgTs = vmap(Delta, [&](float d) { return copysignf(k.Ts, d); });
+        const T h = fma(T(-k.kappa), vv, T(k.dtheta_max)) - vmap(Delta, [](float d) { return fabsf(d); });
+        T Aa = fma(-sgT, fma(G, T(k.inv_l2), -tl), T(-k.Ts * k.kappa));
+        const T Aw = (sgT * vv) * (sec2 * kcl);
+        T c = phidot * fma(-(sgT * vl2), bend, sgTs);
         if (EXT && k.jerk) {  // a is a state: its terms join the constant; the jerk enters via -kappa
-          hr.c0 += acc * hr.Aa;
-          hr.Aa = -k.hTs2 * k.kappa;
+          c = fma(acc, Aa, c);
+          Aa = T(-k.hTs2 * k.kappa);
         }
-        const float hm = fmaxf(fabsf(hr.h), k.h_floor);
-        const float ht = copysignf(hm, hr.h);  // h's sign (h = -0 does not arise: an exact zero rounds to +0)
-        const float zda = clampf(k.sigma_alpha * n_h, k.ua_lo, k.ua_hi);
-        const float pam = k.w_am * zda + k.pc_am;  // p_alpha / m_alpha
-        const float b = -alpha_h * hr.h - hr.c0;
-        const float r = hr.Aa * q0 + hr.Aw * q1 + ht * pam - b;
-        const float iht = __fdividef(1.f, ht);  // MUFU reciprocal (~1 ulp)
-        const float rho = r * iht;
-        ca_h = hr.Aa * iht;
-        cw_h = hr.Aw * iht;
-        cc_h = pam - rho;
-        const float own = (lt == 0) ? 1.f : 0.f;  // the sums take the row once (lane 0)
-        const float ua_ = own * ca_h;
-        Saa = ua_ * ua_;
-        ga = ua_ * rho;
-        if constexpr (EXT) {
-          const float uw_ = own * cw_h;
-          Saw = ua_ * uw_;
-          Sww = uw_ * uw_;
-          gw = uw_ * rho;
-        } else {
-          // the plain family's ellipse rows have no steer-rate column: these
-          // sums hold the hitch row's terms alone, the same on every lane of
-          // the team (no team reduction; the values it would give)
-          Saw = ca_h * cw_h;
-          Sww = cw_h * cw_h;
-          gw = cw_h * rho;
-        }
+        // h's sign (h = -0 does not arise: an exact zero rounds to +0)
+        const T ht = vmap(h, [&](float x) { return copysignf(fmaxf(fabsf(x), k.h_floor), x); });
+        const T r = fma(Aa, q0, fma(Aw, q1, fma(ht, pam_h, fma(alpha_h, h, c))));
+        const T iht = vrcp(ht);
+        u_h = Aa * iht;
+        w_h = Aw * iht;
+        rho_h = r * iht;
+        cc_h = pam_h - rho_h;
       }
 
-      // obstacle rows; the steer rate does not enter at second order.  Parked ellipses (e = 2): hdot shares dh/da's
-      // direction term.  Moving or e = 4 rows (uniform branch): barrier of
-      // the relative position at this step's time, relative velocity.
-      // `live` = 0 turns a padding slot into a no-op without branching.
-      float ca[OBS_SLOTS], cc[OBS_SLOTS];
-      float cw[EXT ? OBS_SLOTS : 1];  // steer-rate column (footprint discs off the rear axle)
+      // obstacle rows; the steer rate does not enter at second order.  Parked
+      // ellipses (e = 2): hdot shares dh/da's direction term.  Moving or
+      // e = 4 rows (uniform branch): barrier of the relative position at this
+      // step's time, relative velocity.  Padding slots read the table's null
+      // row (j = n_rows).
+      T Saa = 0.f, ga = 0.f, Saw = 0.f, Sww = 0.f, gw = 0.f;
+      T ca[OBS_SLOTS];
+      T cw[EXT ? OBS_SLOTS : 1];  // steer-rate column (footprint discs off the rear axle)
       // every slot that the alpha update reads is written below (padding
       // rows as zeros)
       const float tnow = static_cast<float>(tau) * k.Ts;
-      float cbuf = 0.f;  // buffer cost of this lane's rows
-      // heading rates and accelerations of the bodies (footprint discs):
-      // th2 = th1 - phi; heading accelerations with the input held,
-      // th1ddot = a1a a + a1w omega, th2ddot = a20 + a2a a + a2w omega
-      float c2 = 0.f, s2 = 0.f, th2dot = 0.f, a1a = 0.f, a1w = 0.f, a20 = 0.f, a2a = 0.f, a2w = 0.f;
+      T cbuf = 0.f;  // buffer cost of this lane's rows
+      // heading accelerations of the bodies with the input held (footprint
+      // discs): th1ddot = a1a a + a1w omega, th2ddot = a20 + a2a a + a2w omega
+      T a1w = 0.f, a20 = 0.f, a2a = 0.f, a2w = 0.f;
       if (EXT && k.discs) {
-        c2 = c1 * cp + s1 * sp;
-        s2 = s1 * cp - c1 * sp;
-        const float G = sp - k.k_hitch * cp * tn;
-        const float sec2 = 1.f + tn * tn;
-        th2dot = vv * G * k.inv_l2;
-        a1a = tn * k.inv_l1;
-        a1w = vv * sec2 * k.inv_l1;
-        a2a = G * k.inv_l2;
-        a2w = -vv * k.k_hitch * cp * sec2 * k.inv_l2;
-        a20 = vv * k.inv_l2 * (cp + k.k_hitch * tn * sp) * (th1dot - th2dot);
+        a1w = vv * sec2 * T(k.inv_l1);
+        a2a = G * T(k.inv_l2);
+        a2w = -(vv * T(k.khl2) * cp * sec2);
+        a20 = vl2 * bend * phidot;
       }
-      // per-step factors of the parked-ellipse rows (their rest term, below)
-      const float cg_row = -2.f * k.Ts * vv, vth_row = -k.Ts2 * vv * th1dot, vq_row = -k.Ts2 * vv * vv;
-      const float qxx_row = vq_row * c1 * c1, qyy_row = vq_row * s1 * s1, qxy_row = 2.f * vq_row * c1 * s1;
-      auto obstacle_row = [&](int j, float n_alpha, int slot, float live) {
-        float h, Aa, Aw = 0.f, brest;
+      // per-step factors of the parked-ellipse rows.  With (gx, gy) =
+      // grad h / 2 = Q d and the heading e1 = (c1, s1): the a-column is
+      // Ts^2/2 dh/da = Ts^2 (gx, gy) . e1 and the rest term
+      // -(Ts hdot + Ts^2/2 hddot0) = -2 Ts v g - Ts^2 (v th1dot turn + v^2
+      // e1^T Q e1), g and turn the products of (gx, gy) with e1 and n1:
+      // linear in (gx, gy, Qxx, Qxy, Qyy) with factors of the state alone
+      const T ax_row = T(k.Ts2) * c1, ay_row = T(k.Ts2) * s1;
+      const T cg_row = T(-2.f * k.Ts) * vv, vth_row = T(-k.Ts2) * (vv * th1dot), vq_row = T(-k.Ts2) * (vv * vv);
+      const T bx_row = fma(cg_row, c1, -(vth_row * s1)), by_row = fma(cg_row, s1, vth_row * c1);
+      const T qxx_row = vq_row * (c1 * c1), qyy_row = vq_row * (s1 * s1), qxy_row = (vq_row + vq_row) * (c1 * s1);
+      auto obstacle_row = [&](int j, T pam, T& al, T& u, T& w) {  // pam: p_alpha / m_alpha
+        T h, Aa, Aw = 0.f, brest;
         if constexpr (!EXT) {
           // staged as (cx, cy, Qxx, Qxy, Qyy): h = d^T Q d - 1 in world axes
           const float4 o0 = *reinterpret_cast<const float4*>(S.obs + 8 * j);
-          const float qyy = S.obs[8 * j + 4];
-          const float dx = (px - o0.x) + pxl, dy = (py - o0.y) + pyl;
-          // with (gx, gy) = grad h / 2 = Q d and the heading e1 = (c1, s1):
-          // h = d . (gx, gy) - 1; hdot = 2 v g, g = grad h . e1 / 2;
-          // hddot (input part aside) = 2 v th1dot turn + 2 v^2 curv, turn =
-          // grad h . n1 / 2, curv = e1^T (Hess h / 2) e1 = e1^T Q e1; so the
-          // row's a-column Ts^2/2 dh/da = Ts^2 g and its rest
-          // -(Ts hdot + Ts^2/2 hddot0) = -2 Ts v g - Ts^2 (v th1dot turn + v^2 curv)
-          const float gx = fmaf(o0.z, dx, o0.w * dy), gy = fmaf(o0.w, dx, qyy * dy);
-          h = fmaf(gx, dx, fmaf(gy, dy, -1.f));
-          const float g = fmaf(gx, c1, gy * s1);
-          const float turn = fmaf(gy, c1, -(gx * s1));
-          Aa = k.Ts2 * g;
-          brest = fmaf(cg_row, g, fmaf(vth_row, turn, fmaf(qxx_row, o0.z, fmaf(qxy_row, o0.w, qyy_row * qyy))));
+          const T qxx = o0.z, qxy = o0.w, qyy = S.obs[8 * j + 4];
+          const T dx = (px - T(o0.x)) + pxl, dy = (py - T(o0.y)) + pyl;
+          const T gx = fma(qxx, dx, qxy * dy), gy = fma(qxy, dx, qyy * dy);
+          h = fma(gx, dx, fma(gy, dy, T(-1.f)));
+          Aa = fma(gx, ax_row, gy * ay_row);
+          brest = fma(gx, bx_row, fma(gy, by_row, fma(qxx_row, qxx, fma(qxy_row, qxy, qyy_row * qyy))));
         } else {
           // row j: obstacle o seen from footprint disc m (obstacle-major)
           const int o = (k.nd == 1) ? j : __float2int_rz((static_cast<float>(j) + 0.5f) * k.inv_nd);
           const int m = j - o * k.nd;
           const float4 o0 = *reinterpret_cast<const float4*>(S.obs + 8 * o);
           const float4 o1 = *reinterpret_cast<const float4*>(S.obs + 8 * o + 4);
-          const float2 lv = *reinterpret_cast<const float2*>(S.disc + 2 * m);  // lever arms on e1, e2
-          const float co = o0.z, so = o0.w;
+          const float2 lvp = *reinterpret_cast<const float2*>(S.disc + 2 * m);  // lever arms on e1, e2
+          const T lx = lvp.x, ly = lvp.y;
+          const T co = o0.z, so = o0.w;
           // unit headings in the obstacle frame: e1' = (dirx, diry),
           // n1' = (-diry, dirx), e2' = (d2x, d2y), n2' = (-d2y, d2x)
-          const float dirx = co * c1 + so * s1, diry = co * s1 - so * c1;
-          const float d2x = co * c2 + so * s2, d2y = co * s2 - so * c2;
-          const float dx = (px - o0.x) + pxl, dy = (py - o0.y) + pyl;
+          const T dirx = fma(co, c1, so * s1), diry = fma(co, s1, -(so * c1));
+          const T d2x = fma(co, c2, so * s2), d2y = fma(co, s2, -(so * c2));
+          const T dx = (px - T(o0.x)) + pxl, dy = (py - T(o0.y)) + pyl;
           // disc centre relative to the (moving) obstacle centre at tnow;
           // e = 4 flagged by a negated kx; X = xp^(e-2) / Ax^e:
           // h = xp^2 X + ..., h_x = e xp X, h_xx = e (e-1) X
-          const float xp = co * dx + so * dy + lv.x * dirx + lv.y * d2x - tnow * o1.z;
-          const float yp = co * dy - so * dx + lv.x * diry + lv.y * d2y - tnow * o1.w;
+          const T xp = fma(lx, dirx, fma(ly, d2x, fma(co, dx, fma(so, dy, T(-tnow * o1.z)))));
+          const T yp = fma(lx, diry, fma(ly, d2y, fma(co, dy, fma(-so, dx, T(-tnow * o1.w)))));
           const bool e4 = o1.x < 0.f;
-          const float kx = fabsf(o1.x), ky = o1.y;
-          const float X = e4 ? xp * xp * kx : kx, Y = e4 ? yp * yp * ky : ky;
-          const float ce = e4 ? 4.f : 2.f, cee = e4 ? 12.f : 2.f;
-          h = xp * xp * X + yp * yp * Y - 1.f;
-          const float hx = ce * xp * X, hy = ce * yp * Y;
+          const T kx = fabsf(o1.x), ky = o1.y;
+          const T x2 = xp * xp, y2 = yp * yp;
+          const T X = e4 ? x2 * kx : kx, Y = e4 ? y2 * ky : ky;
+          const T ce = e4 ? 4.f : 2.f, cee = e4 ? 12.f : 2.f;
+          h = fma(x2, X, fma(y2, Y, T(-1.f)));
+          const T hx = ce * xp * X, hy = ce * yp * Y;
           // disc velocity relative to the obstacle
-          const float velx = vv * dirx - lv.x * th1dot * diry - lv.y * th2dot * d2y - o1.z;
-          const float vely = vv * diry + lv.x * th1dot * dirx + lv.y * th2dot * d2x - o1.w;
+          const T lt1 = lx * th1dot, lt2 = ly * th2dot;
+          const T velx = fma(vv, dirx, T(-o1.z)) - fma(lt1, diry, lt2 * d2y);
+          const T vely = fma(vv, diry, T(-o1.w)) + fma(lt1, dirx, lt2 * d2x);
           // disc acceleration = acc0 + a acc_a + omega acc_w
-          const float aax = dirx - lv.x * a1a * diry - lv.y * a2a * d2y;
-          const float aay = diry + lv.x * a1a * dirx + lv.y * a2a * d2x;
-          const float awx = -lv.x * a1w * diry - lv.y * a2w * d2y;
-          const float awy = lv.x * a1w * dirx + lv.y * a2w * d2x;
-          const float t1q = th1dot * th1dot, t2q = th2dot * th2dot;
-          const float a0x = -vv * th1dot * diry - lv.x * t1q * dirx - lv.y * (a20 * d2y + t2q * d2x);
-          const float a0y = vv * th1dot * dirx - lv.x * t1q * diry + lv.y * (a20 * d2x - t2q * d2y);
-          const float hdot = hx * velx + hy * vely;
-          const float hdd0 = hx * a0x + hy * a0y + cee * (X * velx * velx + Y * vely * vely);
-          Aa = k.hTs2 * (hx * aax + hy * aay);
-          Aw = k.hTs2 * (hx * awx + hy * awy);
-          brest = -k.Ts * hdot - k.hTs2 * hdd0;
+          const T la1 = lx * tl, la2 = ly * a2a, lw1 = lx * a1w, lw2 = ly * a2w;
+          const T aax = dirx - fma(la1, diry, la2 * d2y);
+          const T aay = diry + fma(la1, dirx, la2 * d2x);
+          const T awx = -fma(lw1, diry, lw2 * d2y);
+          const T awy = fma(lw1, dirx, lw2 * d2x);
+          const T vw = vv * th1dot;
+          const T q1c = lt1 * th1dot, q2c = lt2 * th2dot, q20 = ly * a20;
+          const T a0x = -fma(vw, diry, fma(q1c, dirx, fma(q20, d2y, q2c * d2x)));
+          const T a0y = fma(vw, dirx, -fma(q1c, diry, fma(-q20, d2x, q2c * d2y)));
+          const T hdot = fma(hx, velx, hy * vely);
+          const T wHx = cee * X * velx, wHy = cee * Y * vely;  // Hess h w
+          const T hdd0 = fma(hx, a0x, fma(hy, a0y, fma(wHx, velx, wHy * vely)));
+          Aa = T(k.hTs2) * fma(hx, aax, hy * aay);
+          Aw = T(k.hTs2) * fma(hx, awx, hy * awy);
+          brest = fma(T(-k.Ts), hdot, T(-k.hTs2) * hdd0);
           if (k.third) {
             // Ts^3/6 hdddot at the rear axle (lever arms zero), affine in
             // (a, omega): pdddot = 2 a th1dot n1 + v th1ddot n1 - v th1dot^2 e1,
             // hdddot = grad h . pdddot + 3 w^T Hess h pddot + D3 h [w, w, w]
-            const float gn = hy * dirx - hx * diry;  // grad h . n1'
-            const float hxxx = e4 ? 24.f * xp * kx : 0.f, hyyy = e4 ? 24.f * yp * ky : 0.f;
-            const float wHx = cee * X * velx, wHy = cee * Y * vely;  // Hess h w
-            const float ca3 = (2.f * th1dot + vv * tn * k.inv_l1) * gn + 3.f * (wHx * dirx + wHy * diry);
-            const float cw3 = vv * vv * (1.f + tn * tn) * k.inv_l1 * gn;
-            const float c03 = -vv * th1dot * th1dot * gda3(hx, hy, dirx, diry) +
-                              3.f * vv * th1dot * (wHy * dirx - wHx * diry) +
-                              hxxx * velx * velx * velx + hyyy * vely * vely * vely;
-            Aa += k.Ts3_6 * ca3;
-            Aw += k.Ts3_6 * cw3;
-            brest -= k.Ts3_6 * c03;
+            const T ge = fma(hx, dirx, hy * diry);     // grad h . e1'
+            const T gn = fma(hy, dirx, -(hx * diry));  // grad h . n1'
+            const T ca3 = fma(fma(T(2.f), th1dot, vv * tl), gn, T(3.f) * fma(wHx, dirx, wHy * diry));
+            const T cw3 = vv * vv * sec2 * T(k.inv_l1) * gn;
+            T c03 = fma(-(vw * th1dot), ge, T(3.f) * vw * fma(wHy, dirx, -(wHx * diry)));
+            const T k3x = e4 ? 24.f * fabsf(o1.x) : 0.f, k3y = e4 ? 24.f * o1.y : 0.f;
+            c03 = fma(xp * k3x * velx * velx, velx, fma(yp * k3y * vely * vely, vely, c03));
+            Aa = fma(T(k.Ts3_6), ca3, Aa);
+            Aw = fma(T(k.Ts3_6), cw3, Aw);
+            brest = fma(T(-k.Ts3_6), c03, brest);
           }
           if (k.jerk) {
             // a is a state (rear-axle point): its terms join the constant;
             // the jerk enters only at third order, through grad h . e1'
-            brest -= acc * Aa;
-            Aa = k.third ? k.Ts3_6 * gda3(hx, hy, dirx, diry) : 0.f;
+            brest = fma(-acc, Aa, brest);
+            Aa = k.third ? T(k.Ts3_6) * fma(hx, dirx, hy * diry) : T(0.f);
           }
         }
-        const float hm = fmaxf(fabsf(h), k.h_floor);
-        const float ht = copysignf(hm, h);
-        const float zda = clampf(k.sigma_alpha * n_alpha, k.ua_lo, k.ua_hi);
-        const float pam = k.w_am * zda + k.pc_am;  // p_alpha / m_alpha
-        const float b = -alpha[slot] * h + brest;
-        float r = fmaf(Aa, q0, fmaf(ht, pam, -b));
-        if constexpr (EXT) r = fmaf(Aw, q1, r);
-        // MUFU reciprocal (~1 ulp); a padding slot (live = 0) gets 0: its
-        // u, w and rho vanish, so it adds nothing to the sums (its own rate
-        // drifts by p_alpha a step and is never read by a live row)
-        const float iht = live * __fdividef(1.f, ht);
-        const float u = Aa * iht;
-        const float rho = r * iht;
-        Saa += u * u;
-        ga += u * rho;
-        ca[slot] = u;
-        cc[slot] = pam - rho;
-        if constexpr (EXT) {
-          const float w = Aw * iht;
-          Saw += u * w;
-          Sww += w * w;
-          gw += w * rho;
-          cw[slot] = w;
-        }
+        const T ht = vmap(h, [&](float x) { return copysignf(fmaxf(fabsf(x), k.h_floor), x); });
+        T r = fma(Aa, q0, fma(ht, pam, fma(al, h, -brest)));
+        if constexpr (EXT) r = fma(Aw, q1, r);
+        const T iht = vrcp(ht);  // MUFU reciprocal (~1 ulp)
+        u = Aa * iht;
+        const T rho = r * iht;
+        Saa = fma(u, u, Saa);
+        ga = fma(u, rho, ga);
         if (EXT && k.abuf) {
           // buffer zone: positive rates charged with weight clip(1 - h/h_buf)
-          const float wz = clampf(1.f - h * k.inv_hbuf, 0.f, 1.f);
-          const float ap = fmaxf(alpha[slot], 0.f);
-          cbuf += live * (k.q_abuf * wz * ap * ap);
+          const T wz = vclamp(fma(h, T(-k.inv_hbuf), T(1.f)), 0.f, 1.f);
+          const T ap = vmap(al, [](float x) { return fmaxf(x, 0.f); });
+          cbuf = fma(T(j < n_rows ? k.q_abuf : 0.f) * wz, ap * ap, cbuf);
+        }
+        // the rate's update without its part in y, added after the 2x2 solve
+        al = al + (pam - rho);
+        if constexpr (EXT) {
+          w = Aw * iht;
+          Saw = fma(u, w, Saw);
+          Sww = fma(w, w, Sww);
+          gw = fma(w, rho, gw);
         }
       };
 
-      if constexpr (TPS == 1) {
-        // row j uses normal 4 + j: block 1 + j/4, drawn here
+      if constexpr (!kNoiseWarps<TPS, BPT, NS>) {
+        // row j uses normal 4 + j: block 1 + j/4, drawn here, a pass over the
+        // team's lanes at a time
+        const StepWords now = step_words(tau);
+#pragma unroll 1
+        for (int g = 0; g < passes; ++g) {
+          const int b = 1 + g * TPS + lt;
+          T nb[4];
+          draw_block(TPS == 1 ? b : min(b, in.P - 1), now, nb);
+          float* row = rows + 4 * g * row_stride;
 #pragma unroll
-        for (int b8 = 1; b8 < BPT; ++b8) {
-          if (b8 < in.P) {
-            float nb[4];
-            draw_block(b8, tau, nb);
-#pragma unroll
-            for (int m = 0; m < 4; ++m) {
-              const int j = 4 * (b8 - 1) + m;
-              ca[j] = 0.f;
-              cc[j] = 0.f;
-              if constexpr (EXT) cw[j] = 0.f;
-              if (j < n_rows) obstacle_row(j, nb[m], j, 1.f);
+          for (int m = 0; m < 4; ++m) {
+            const int j = 4 * (b - 1) + m;
+            if (TPS > 1 || j < n_rows) {
+              T al, u, w = 0.f;
+              load_row<EXT, NS>(row + m * row_stride, al, u, w);
+              al = fma(u, ya_p, al);
+              if constexpr (EXT) al = fma(w, yw_p, al);
+              obstacle_row(min(j, n_rows), sampled_rate(k, nb[m]), al, u, w);
+              store_row<EXT, NS>(row + m * row_stride, al, u, w);
             }
           }
         }
-      } else if constexpr (ROWS > 0) {
-        // exactly ROWS row slots a lane (row j on lane j % TPS): every slot
-        // runs, padding rows masked by `live`; no branch in the step
-#pragma unroll
-        for (int slot = 0; slot < ROWS; ++slot) {
-          const int j = lt + TPS * slot;
-          const bool live = j < n_rows;
-          const int jj = live ? j : 0;
-          obstacle_row(jj, cur[4 + jj], slot, live ? 1.f : 0.f);
-        }
       } else {
-        // row j on lane j % TPS; every lane runs the team's slot count
+        // row j on lane j % TPS.  ROWS > 0: exactly ROWS slots a lane, all
+        // of them run, no branch in the step; else the team's slot count
         const int per_lane = (n_rows + TPS - 1) / TPS;
 #pragma unroll
         for (int slot = 0; slot < OBS_SLOTS; ++slot) {
-          ca[slot] = 0.f;
-          cc[slot] = 0.f;
-          if constexpr (EXT) cw[slot] = 0.f;
-          if (slot < per_lane) {
+          if (ROWS == 0) {
+            ca[slot] = 0.f;
+            if constexpr (EXT) cw[slot] = 0.f;
+          }
+          if (ROWS > 0 || slot < per_lane) {
             const int j = lt + TPS * slot;
-            const bool live = j < n_rows;
-            const int jj = live ? j : 0;
-            obstacle_row(jj, cur[4 + jj], slot, live ? 1.f : 0.f);
+            T w = 0.f;
+            obstacle_row(min(j, n_rows), T(cur[4 + min(j, n_rows - 1)]), alpha[slot], ca[slot], w);
+            if constexpr (EXT) cw[slot] = w;
           }
         }
       }
-      if (EXT && k.abuf) acc2(Jh, Jl, team_sum<TPS>(cbuf));
-      Saa = k.m_a * team_sum<TPS>(Saa) + k.m_u0;
-      ga = k.m_a * team_sum<TPS>(ga);
+      if (EXT && k.abuf) add_share(cbuf);
+      const T m_a = k.m_a;
+      Saa = fma(m_a, fma(u_h, u_h, team_sum<TPS>(Saa)), T(k.m_u0));
+      ga = m_a * fma(u_h, rho_h, team_sum<TPS>(ga));
       if constexpr (EXT) {
-        Saw = k.m_a * team_sum<TPS>(Saw);
-        Sww = k.m_a * team_sum<TPS>(Sww) + k.m_u1;
-        gw = k.m_a * team_sum<TPS>(gw);
+        Saw = m_a * fma(u_h, w_h, team_sum<TPS>(Saw));
+        Sww = fma(m_a, fma(w_h, w_h, team_sum<TPS>(Sww)), T(k.m_u1));
+        gw = m_a * fma(w_h, rho_h, team_sum<TPS>(gw));
       } else {
-        Saw = k.m_a * Saw;
-        Sww = k.m_a * Sww + k.m_u1;
-        gw = k.m_a * gw;
+        // the plain family's ellipse rows have no steer-rate column
+        Saw = m_a * (u_h * w_h);
+        Sww = fma(m_a, w_h * w_h, T(k.m_u1));
+        gw = m_a * (w_h * rho_h);
       }
-      const float idet = __fdividef(1.f, Saa * Sww - Saw * Saw);  // SPD: det > 0
-      const float ya = (Sww * ga - Saw * gw) * idet;
-      const float yw = (Saa * gw - Saw * ga) * idet;
+      const T idet = vrcp(fma(Saa, Sww, -(Saw * Saw)));  // SPD: det > 0
+      const T ya = fma(Sww, ga, -(Saw * gw)) * idet;
+      const T yw = fma(Saa, gw, -(Saw * ga)) * idet;
       za = q0 - ya;
       zw = q1 - yw;
-      zn = pu2 * k.inv_m_u2;
-      alpha_h += cc_h + ca_h * ya + cw_h * yw;
+      alpha_h = alpha_h + fma(w_h, yw, fma(u_h, ya, cc_h));
       auto alpha_update = [&](int slot) {
-        if constexpr (EXT) {
-          alpha[slot] += cc[slot] + ca[slot] * ya + cw[slot] * yw;
-        } else {
-          alpha[slot] += cc[slot] + ca[slot] * ya;
-        }
+        alpha[slot] = fma(ca[slot], ya, alpha[slot]);
+        if constexpr (EXT) alpha[slot] = fma(cw[slot], yw, alpha[slot]);
       };
-      if constexpr (TPS == 1) {
-        // the blocks this instance draws (a uniform branch per block): rows
-        // of the blocks beyond it are never read
-#pragma unroll
-        for (int b8 = 1; b8 < BPT; ++b8)
-          if (b8 < in.P) {
-#pragma unroll
-            for (int m = 0; m < 4; ++m) alpha_update(4 * (b8 - 1) + m);
-          }
+      if constexpr (!PRODUCED) {
+        ya_p = ya;
+        yw_p = yw;
       } else {
 #pragma unroll
         for (int slot = 0; slot < OBS_SLOTS; ++slot) alpha_update(slot);
       }
-    } else {
-      za = zd0;
-      zw = zd1;
-      zn = zd2;
     }
-    ua = clampf(za, k.zlo0, k.zhi0);
-    uw = clampf(zw, k.zlo1, k.zhi1);
-    un = clampf(zn, k.zlo2, k.zhi2);
+    ua = vclamp(za, k.zlo0, k.zhi0);
+    uw = vclamp(zw, k.zlo1, k.zhi1);
+    un = vclamp(zn, k.zlo2, k.zhi2);
     if constexpr (TPS == 1) state_part();
 
     // explicit Euler, the input-driven part; the state-only part was formed
@@ -1109,32 +1260,33 @@ __device__ void run_tile(const KConst& k, const Inst& in, int tile, float* uh, c
     t1 = t1_n;
     t2 = t2_n;
     if (EXT && k.jerk) {  // input 0 is the jerk; the acceleration state drives the speed
-      acc2(v, vl, k.Ts * acc);
-      acc += k.Ts * ua;
+      acc2(v, vl, T(k.Ts) * acc);
+      acc = fma(T(k.Ts), ua, acc);
     } else {
-      acc2(v, vl, k.Ts * ua);
+      acc2(v, vl, T(k.Ts) * ua);
     }
-    dl += k.Ts * uw;
-    acc2(ps, psl, k.Ts * un);
+    dl = fma(T(k.Ts), uw, dl);
+    acc2(ps, psl, T(k.Ts) * un);
     c1 = c1_n;
     s1 = s1_n;
     sp = sp_n;
     cp = cp_n;
 
     if (lt == 0) {
-      uh[(3 * tau + 0) * spb + team] = ua;
-      uh[(3 * tau + 1) * spb + team] = uw;
-      uh[(3 * tau + 2) * spb + team] = un;
+      store_pair(uh + (3 * tau + 0) * spb + team * NS, ua);
+      store_pair(uh + (3 * tau + 1) * spb + team * NS, uw);
+      store_pair(uh + (3 * tau + 2) * spb + team * NS, un);
     }
     if (st_out) store_state(tau + 1);
     if (in_out) {
-      in_out[3 * tau + 0] = ua;
-      in_out[3 * tau + 1] = uw;
-      in_out[3 * tau + 2] = un;
-    }
-    if constexpr (TPS == 1) {
 #pragma unroll
-      for (int q = 0; q < 4; ++q) nrm[q] = nxt[q];
+      for (int i = 0; i < NS; ++i) {
+        if (s + i >= in.S) break;
+        float* o = in.inputs_out + (static_cast<size_t>(s + i) * static_cast<size_t>(H) + tau) * 3;
+        o[0] = ua.get(i);
+        o[1] = uw.get(i);
+        o[2] = un.get(i);
+      }
     }
   };
   if (!producer) {
@@ -1144,33 +1296,47 @@ __device__ void run_tile(const KConst& k, const Inst& in, int tile, float* uh, c
       for (int tau = 0; tau < H; ++tau) step(tau, std::false_type{});
     }
   }
-  if (!producer) {  // cost of the last step
-    float ce1 = 0.f, se1 = 0.f, ce2 = 0.f, se2 = 0.f;
-    if (EXT && k.coll && k.discs) {
-      float sr, cr, sq, cq;
-      sincosf(t1, &sr, &cr);
-      sincosf(t1 - t2, &sq, &cq);
-      ce1 = c0 * cr - s0 * sr;
-      se1 = s0 * cr + c0 * sr;
-      ce2 = ce1 * cq + se1 * sq;
-      se2 = se1 * cq - ce1 * sq;
+  if (!producer) {  // cost of the last step, and the team's sum
+    if constexpr (!SHARE) {
+      cost_after(H);
+    } else {
+      if (lt == ((H - 1) & (TPS - 1))) kept = visit();
+      const T last = stage_cost(kept);  // lanes past the last step were summed already
+      acc2(Jh, Jl, lt <= ((H - 1) & (TPS - 1)) ? last : T(0.f));
     }
-    stage_cost(static_cast<float>(H) * k.Ts, ce1, se1, ce2, se2, true);
+    if (EXT && k.coll)
+      collision_cost(static_cast<float>(H) * k.Ts, c1, s1, fma(c1, cp, s1 * sp), fma(s1, cp, -(c1 * sp)));
+    auto team_pair = [&](T& h, T& l) {
+#pragma unroll
+      for (int m = 1; m < TPS; m <<= 1) {
+        const T oh = vshfl_xor(h, m), ol = vshfl_xor(l, m);
+        acc2(h, l, oh);
+        l = l + ol;
+      }
+    };
+    if constexpr (SHARE) team_pair(Jh, Jl);
+    if constexpr (EXT) {
+      if (k.coll || k.abuf) {
+        team_pair(Xh, Xl);
+        acc2(Jh, Jl, Xh);
+        Jl = Jl + Xl;
+      }
+    }
   }
 
   // --- per-sample cost: normalise the pair
-  {
-    const float sum = Jh + Jl;
-    Jl = Jl - (sum - Jh);
-    Jh = sum;
-  }
-  const bool valid = s < in.S;
-  if (!producer && lt == 0) {
-    const bool fin = valid && isfinite(Jh) && isfinite(Jl);
-    S.jh[team] = fin ? Jh : CUDART_INF_F;
-    S.jl[team] = fin ? Jl : 0.f;
-    if (valid && in.J_out) in.J_out[s] = Jh;  // the normalised pair's high part
-    if (valid && in.J_lo_out) in.J_lo_out[s] = Jl;
+  if (writer) {
+#pragma unroll
+    for (int i = 0; i < NS; ++i) {
+      const float jh = Jh.get(i) + Jl.get(i);
+      const float jl = Jl.get(i) - (jh - Jh.get(i));
+      const bool valid = s + i < in.S;
+      const bool fin = valid && isfinite(jh) && isfinite(jl);
+      S.jh[team * NS + i] = fin ? jh : CUDART_INF_F;
+      S.jl[team * NS + i] = fin ? jl : 0.f;
+      if (valid && in.J_out) in.J_out[s + i] = jh;  // the normalised pair's high part
+      if (valid && in.J_lo_out) in.J_lo_out[s + i] = jl;
+    }
   }
   __syncthreads();
 
@@ -1406,12 +1572,6 @@ static __device__ void serial_trajectory(const KConst& k, const Inst& in, const 
   }
 }
 
-// 16-byte asynchronous copy global -> shared through L2 (cp.async.cg).
-__device__ __forceinline__ void cp_async16(float* smem_dst, const float* gmem_src) {
-  const unsigned d = static_cast<unsigned>(__cvta_generic_to_shared(smem_dst));
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(gmem_src) : "memory");
-}
-
 // Minimum pair over the partials of an instance held in shared memory
 // (tile b at mp + b * stride), into sh.red_h[1] / sh.red_l[1].
 static __device__ void smem_pair_min(const float* mp, int nb, int stride, Shared& sh) {
@@ -1608,7 +1768,7 @@ static __device__ void merge_instance(const KConst& k, const Inst& in, const Sme
   const float lsum = ustar[3 * H];
   const unsigned err = sh.err | (turns_bad ? ERR_PATH_TURN : 0u);
   for (int q = threadIdx.x; q < 3 * H; q += blockDim.x) {
-    const float u = ok ? ustar[q] / lsum : S.unom[q];
+    const float u = ok ? ustar[q] / lsum : in.U_nom[q];
     ustar[q] = u;
     in.U_out[q] = u;
   }
@@ -1661,16 +1821,18 @@ __device__ __forceinline__ void discard_history(const float* uh, int n_floats) {
 }
 
 // -------------------------------------------------------------- the kernel
+// Launch bound of the two-sample variants: three CTAs of 128 threads an SM
+constexpr int kMaxPairThreads = 128, kPairCtas = 3;
 // EXT: the instantiations that also carry the optional terms (moving and
 // e = 4 obstacles, collision cost, buffer cost); the others compile them out.
-template <int TPS, int BPT, bool EXT, int ROWS = 0>
+template <int TPS, int BPT, bool EXT, int ROWS = 0, int NS = 1, bool LOCAL = false>
 // Launch bound: 512 threads (128 registers a thread); the exact-rows
 // single-solve instantiations 384 (up to 170 registers: one CTA per SM on
 // the latency shapes, where registers buy a longer schedule)
-__global__ void __launch_bounds__(ROWS > 0 ? 384 : 512) solve_kernel(const KConst k, const LaunchDesc L) {
+__global__ void __launch_bounds__(ROWS > 0 ? 384 : (NS > 1 ? kMaxPairThreads : 512), NS > 1 ? kPairCtas : 1) solve_kernel(const KConst k, const LaunchDesc L) {
   extern __shared__ float dyn[];
   __shared__ Shared sh;
-  const int spb = compute_threads<TPS>(L.noise_warps) / TPS;
+  const int spb = compute_threads<TPS>(L.noise_warps) / TPS * NS;
   const Smem S(dyn, L.caps, spb);
   // applied-input history of the CTA's tile: shared memory in the exact-rows
   // variants (the launch reserved it), else the CTA's global slot
@@ -1699,12 +1861,12 @@ __global__ void __launch_bounds__(ROWS > 0 ? 384 : 512) solve_kernel(const KCons
     Inst in;
     if (L.work) in = L.inst[inst_id];
     else in = L.single;
-    run_tile<TPS, BPT, EXT, ROWS>(k, in, tile, uh, S, sh, L.noise_warps);
+    run_tile<TPS, BPT, EXT, ROWS, NS, LOCAL>(k, in, tile, uh, S, sh, L.noise_warps);
 
     // the CTA that completes an instance's last tile merges its partials
     __threadfence();
     __syncthreads();
-    if constexpr (ROWS == 0) discard_history(uh, 3 * in.H * (compute_threads<TPS>(L.noise_warps) / TPS));
+    if constexpr (ROWS == 0) discard_history(uh, 3 * in.H * spb);
     if (in.no_merge) continue;  // a share of the tiles: merged elsewhere (single launches only)
     if (threadIdx.x == 0) sh.last = (atomicAdd(in.sync, 1u) == static_cast<unsigned>(in.tiles - 1));
     __syncthreads();
@@ -1737,8 +1899,7 @@ __global__ void __launch_bounds__(256) merge_tiles_kernel(const KConst k, const 
   extern __shared__ float dyn[];
   __shared__ Shared sh;
   const Smem S(dyn, caps, 1);
-  for (int j = threadIdx.x; j < 3 * in.n_pts; j += blockDim.x) cp_async4(S.path + j, in.path + j);
-  for (int j = threadIdx.x; j < 3 * in.H; j += blockDim.x) cp_async4(S.unom + j, in.U_nom + j);
+  stage_path(in, S);
   if (threadIdx.x < 32) make_frame_warp(in.x0, in.inv_ds_d, in.sync + 1, sh.fr, EXT && k.jerk);
   const bool obs8 = EXT && k.obs8;
   for (int o = threadIdx.x; o < in.n_obs; o += blockDim.x) {
@@ -1748,12 +1909,7 @@ __global__ void __launch_bounds__(256) merge_tiles_kernel(const KConst k, const 
   cp_async_wait_all();
   __syncthreads();
   const Frame& fr = sh.fr;
-  for (int j = threadIdx.x; j < in.n_pts; j += blockDim.x) {  // the path in the frame, as the tiles stage it
-    float* d = S.path + 3 * j;
-    d[0] = (d[0] - fr.ox_h) - fr.ox_l;
-    d[1] = (d[1] - fr.oy_h) - fr.oy_l;
-    d[2] = (d[2] - fr.oth_h) - fr.oth_l;
-  }
+  shift_path(in, S, fr);  // as the tiles stage it
   __syncthreads();
   merge_instance<false>(k, in, S, sh);
 }

@@ -1,6 +1,9 @@
-// variants_narrow_ext.cu -- solve-kernel instantiations carrying the optional
-// terms (moving and e = 4 obstacles, collision cost, buffer cost), with 1
-// or 2 lanes per sample.
+// variants_narrow_ext.cu -- solve-kernel instantiations with the optional
+// terms (moving and e = 4 obstacles, collision and buffer costs, footprint
+// discs, third-order rows, the jerk-input model) that draw their noise in
+// registers and keep the rows' state in shared memory (or, where it does not
+// fit there, in local memory): 1, 2, 4 or 8 lanes per sample, any number of
+// rows, one sample a team.
 #include "launch.h"
 
 namespace brmppi {
@@ -8,16 +11,13 @@ namespace brmppi {
 const Variant* variants_narrow_ext(int* n) {
   static const Variant v[] = {
       {1, 1, true, &solve_kernel<1, 1, true>},
-      {1, 2, true, &solve_kernel<1, 2, true>},
-      {1, 3, true, &solve_kernel<1, 3, true>},
-      {1, 4, true, &solve_kernel<1, 4, true>},
-      {1, 5, true, &solve_kernel<1, 5, true>},
-      {1, 6, true, &solve_kernel<1, 6, true>},
-      {1, 8, true, &solve_kernel<1, 8, true>},
-      {2, 1, true, &solve_kernel<2, 1, true>},
-      {2, 2, true, &solve_kernel<2, 2, true>},
       {2, 3, true, &solve_kernel<2, 3, true>},
-      {2, 4, true, &solve_kernel<2, 4, true>},
+      {4, 3, true, &solve_kernel<4, 3, true>},
+      {8, 3, true, &solve_kernel<8, 3, true>},
+      {1, 1, true, &solve_kernel<1, 1, true, 0, 1, true>, 0, 1, true},
+      {2, 3, true, &solve_kernel<2, 3, true, 0, 1, true>, 0, 1, true},
+      {4, 3, true, &solve_kernel<4, 3, true, 0, 1, true>, 0, 1, true},
+      {8, 3, true, &solve_kernel<8, 3, true, 0, 1, true>, 0, 1, true},
   };
   *n = static_cast<int>(sizeof(v) / sizeof(v[0]));
   return v;
