@@ -297,46 +297,65 @@ int samples_per_team(const Shape& sh, bool ext, long long tiles, size_t smem, in
 
 int part_stride_for(int H) { return static_cast<int>(align_up(3 + 3 * static_cast<size_t>(H) + 1, 4)); }
 
-// Heuristic plain shape: a team just wide enough for the Philox blocks (one
-// block per lane), 128-thread blocks while that leaves at least two CTAs per
-// SM, else 64.  Narrower blocks (then wider teams) while the shared-memory
-// tables do not fit.
+// Default shape of a plain solve (no autotuning): tiles that spread the
+// samples evenly over the SMs, and a team as wide as keeps an SM at a few
+// warps.
+//
+// Team width.  A team one Philox block a lane wide has the shortest step, but
+// repeats the step's base on every lane: it is halved while that leaves an SM
+// more than `most` warps.  Measured on GB300 (S samples, n ellipses, H = 30
+// or 20; us at the wider / the narrower team): n = 8, P = 3: S = 6500 33.7 /
+// 35.9 with 5.3 warps an SM at the wider, 8192 41.9 / 36.2 with 6.7; two
+// lanes to one: 16384 50.2 / 54.3 with 6.7, 24000 76.3 / 68.5 with 9.9.
+// n = 20, P = 6: 4096 42.0 / 41.4 with 6.7, 5000 52 / 48.3 with 8.2; two lanes
+// to one: 24000 93 / 114 with 9.9, 32768 117 / 116 with 13.5.  n = 64,
+// P = 17: 4096 48.1 / 54.4 with 6.7, 5000 67.7 / 64.8 with 8.2.  No rows,
+// P = 1: 4096 27.6 / 29.5 with 1.7 (the noise leaves the chain), 10000 34.0 /
+// 30.8 with 4.1.  The optional terms' longer rows take wider teams further:
+// n = 8: 8000 47.5 / 54.6 with 6.6, two lanes to one 20000 93.6 / 105 with 8.2.
+//
+// Tile.  One CTA an SM that holds ceil(S / SMs) samples, where that fits the
+// block: a tile count just over the SM count leaves most of them idle for a
+// second round (S = 5000, n = 8: 4 lanes x 160 threads 31.6 us, x 128 or 64
+// 40 to 52 us).  Else two or three even CTAs an SM (S = 16384, n = 64: 105.5
+// us at 224 threads, 114 at 128); beyond, 256 threads (two samples a lane).
+// Narrower blocks (then wider teams) while the shared-memory tables do not fit.
 bool heuristic_plain(const brmppi_ctx* c, int n_obs, int n_pts, Shape* out) {
-  const int P = philox_blocks(rows_of(c->prm, n_obs));
+  const int rows = rows_of(c->prm, n_obs);
+  const int P = philox_blocks(rows);
+  const long long S = c->prm.S, sms = c->num_sms;
   const bool fixed_tps = c->prm.threads_per_sample != 0;
+  const bool ext = brmppi::needs_ext(make_kconst(c->prm));
   int tps = c->prm.threads_per_sample;
   if (!fixed_tps) {
-    // latency shape: one Philox block per lane; then, while the GPU stays
-    // full (at least 4 warps per SM), fewer lanes per sample and more blocks
-    // per lane (less work repeated across a team)
-    tps = 1;
-    while (tps < P && tps < 32) tps <<= 1;
+    tps = 2;
+    while (tps < P && tps < 16) tps <<= 1;
     int b2 = 0;
-    while (tps > 1 && pick_bpt(tps / 2, P, &b2) &&
-           static_cast<long long>(c->prm.S) * (tps / 2) / 32 >= 4LL * c->num_sms)
+    while (tps > 1 && pick_bpt(tps / 2, P, &b2)) {
+      double most = ext ? 9.0 : (tps == 2 ? 12.0 : 7.5);
+      if (P <= 4) most = tps == 2 ? (P == 1 ? 3.0 : (ext ? 9.0 : 7.0)) : (ext ? 7.0 : (P == 4 ? 6.5 : 5.75));
+      if (static_cast<double>(S) * tps <= most * 32.0 * static_cast<double>(sms)) break;
       tps >>= 1;
+    }
   }
   int bpt = 0;
   if (!pick_bpt(tps, P, &bpt)) return false;
   int threads = c->prm.block_threads;
   const bool fixed_threads = threads != 0;
   if (!fixed_threads) {
-    // 128 threads, one CTA per SM where the tiles fit; just over one wave:
-    // 64 (a short second wave of small CTAs); more: 256; very few tiles: 64
-    // (shapes measured on GB300; the autotuner refines per workload)
-    threads = 128;
-    const long long tiles = (c->prm.S + threads / tps - 1) / (threads / tps);
-    const bool small_ok = 64 / tps >= 2;
-    // (producer-warp variants stay at 128: their CTAs grow by up to four
-    // warps, and 256 + 128 threads of 128 registers fit one CTA per SM)
-    const bool producers = tps > 1 && bpt <= 2;
-    if (tiles > c->num_sms)
-      threads = (tiles <= c->num_sms + c->num_sms / 4 && small_ok) ? 64 : (producers ? 128 : 256);
-    else if (tiles < c->num_sms / 2 && small_ok)
-      threads = 64;
+    // blocks that the exact-rows variants take, where one holds the rows
+    const bool exact = bpt <= 2 && (ext ? tps == 4 : tps <= 8) && (rows + tps - 1) / tps <= 4;
+    const long long limit = exact || bpt == 3 || tps == 1 ? 256 : 384;
+    threads = 256;
+    for (long long k = 1; k <= 3; ++k) {
+      const long long even = ((S + k * sms - 1) / (k * sms) * tps + 31) / 32 * 32;
+      if (even <= (k == 1 ? limit : 256)) {
+        threads = static_cast<int>(std::max<long long>(kMinThreads, even));
+        break;
+      }
+    }
   }
   if (threads < tps) return false;
-  const bool ext = brmppi::needs_ext(make_kconst(c->prm));
   while (table_bytes(make_caps(n_obs, rows_of(c->prm, n_obs), n_pts, c->prm.H, tps, bpt, ext), threads / tps) >
          c->smem_limit) {
     if (!fixed_threads && threads > kMinThreads) {
@@ -392,8 +411,8 @@ brmppi::Inst make_inst(const double* x0, const float* U_nom, const float* obs, i
   in.tiles = (S + spb - 1) / spb;
   in.part_stride = part_stride_for(H);
   in.ds = ds;
-  in.inv_ds = 1.0f / ds;
   in.inv_ds_d = 1.0 / static_cast<double>(ds);
+  in.inv_ds = static_cast<float>(in.inv_ds_d);
   in.key0 = static_cast<uint32_t>(seed);
   in.key1 = static_cast<uint32_t>(seed >> 32);
   in.ctr = static_cast<uint32_t>(counter);
