@@ -245,7 +245,7 @@ brmppi::KConst make_kconst(const brmppi_params& q) {
 brmppi::SmemCaps make_caps(int n_obs, int n_rows, int n_pts, int H, int tps, int bpt, bool ext) {
   brmppi::SmemCaps c{};
   c.obs = 8 * (n_obs + 1);  // and the null row
-  c.path = brmppi::SmemCaps::pad4(3 * n_pts);
+  c.path = 4 * n_pts;
   c.unom = brmppi::SmemCaps::pad4(3 * H);
   c.ustar = brmppi::SmemCaps::pad4(3 * H + 1);
   c.noise_per_team = tps > 1 && bpt <= 2 ? 8 * philox_blocks(n_rows) : 0;
@@ -285,14 +285,17 @@ bool pick_bpt(int tps, int P, int* bpt) {
   return brmppi::variant_exists(tps, *bpt);
 }
 
+// CTAs of `threads` threads of the two-sample variants on an SM.
+long long pair_residency(int threads, size_t smem) {
+  return std::min<long long>(brmppi::kMaxPairBlockThreads * brmppi::kPairCtas / threads, 227 * 1024 / (smem + 2048));
+}
+
 int samples_per_team(const Shape& sh, bool ext, long long tiles, size_t smem, int num_sms) {
   const int threads = sh.threads / 2;
   if (sh.threads % 64 != 0 || threads < 64 || threads > brmppi::kMaxPairBlockThreads ||
       !brmppi::pair_exists(sh.tps, sh.bpt, ext))
     return 1;
-  const long long resident =
-      std::min<long long>(brmppi::kMaxPairBlockThreads * brmppi::kPairCtas / threads, 227 * 1024 / (smem + 2048));
-  return tiles >= resident * num_sms ? 2 : 1;
+  return tiles >= pair_residency(threads, smem) * num_sms ? 2 : 1;
 }
 
 int part_stride_for(int H) { return static_cast<int>(align_up(3 + 3 * static_cast<size_t>(H) + 1, 4)); }
@@ -346,13 +349,18 @@ bool heuristic_plain(const brmppi_ctx* c, int n_obs, int n_pts, Shape* out) {
     // blocks that the exact-rows variants take, where one holds the rows
     const bool exact = bpt <= 2 && (ext ? tps == 4 : tps <= 8) && (rows + tps - 1) / tps <= 4;
     const long long limit = exact || bpt == 3 || tps == 1 ? 256 : 384;
-    threads = 256;
-    for (long long k = 1; k <= 3; ++k) {
+    for (long long k = 1; k <= 3 && threads == 0; ++k) {
       const long long even = ((S + k * sms - 1) / (k * sms) * tps + 31) / 32 * 32;
-      if (even <= (k == 1 ? limit : 256)) {
-        threads = static_cast<int>(std::max<long long>(kMinThreads, even));
-        break;
-      }
+      if (even <= (k == 1 ? limit : 256)) threads = static_cast<int>(std::max<long long>(kMinThreads, even));
+    }
+    if (threads == 0) {
+      // 256, or 384 (more samples share the CTA's tables) where that keeps
+      // more samples on an SM
+      auto resident = [&](int t) {
+        const size_t smem = smem_bytes(make_caps(n_obs, rows, n_pts, c->prm.H, tps, bpt, ext), t / tps);
+        return pair_residency(t / 2, smem) * t;
+      };
+      threads = (bpt == 3 || tps == 1) && resident(384) > resident(256) ? 384 : 256;
     }
   }
   if (threads < tps) return false;
@@ -413,6 +421,7 @@ brmppi::Inst make_inst(const double* x0, const float* U_nom, const float* obs, i
   in.ds = ds;
   in.inv_ds_d = 1.0 / static_cast<double>(ds);
   in.inv_ds = static_cast<float>(in.inv_ds_d);
+  in.inv_ds_l = static_cast<float>(in.inv_ds_d - static_cast<double>(in.inv_ds));
   in.key0 = static_cast<uint32_t>(seed);
   in.key1 = static_cast<uint32_t>(seed >> 32);
   in.ctr = static_cast<uint32_t>(counter);

@@ -93,14 +93,14 @@ __device__ __forceinline__ uint4 philox_words(PhiloxBlock b, PhiloxSample s, Phi
 // table of cosines serves both, 128 entries (a quarter turn) apart.  It needs
 // no quadrant selection.
 // Logarithm: u = 2^e m with m in [0.705, 1.410), the next 7 bits pick
-// 1/c and -2 ln c of a centre c of m's cell (c = 1 in the cell around 1, so
+// 1/c and 2 ln c of a centre c of m's cell (c = 1 in the cell around 1, so
 // that u near 1 keeps its relative accuracy), t = m/c - 1 in one fused
-// multiply-add, |t| <= 2^-8, and -2 ln(1 + t) = t (-2 + t (1 - 2/3 t)):
+// multiply-add, |t| <= 2^-8, and 2 ln(1 + t) = t (2 + t (-1 + 2/3 t)):
 // within 1.42 ulp, 3.0e-8 relative in the root mean square, over all 2^23
 // uniforms (neg2_log_unit with an exact division: 2.5 ulp, 4.1e-8).
 struct NoiseTables {
   float cosine[640];  // cos(2 pi (i + 1/2) / 512 - pi/2), so sin at i and cos at i + 128
-  float rcp[128], log[128];  // 1 / c, -2 ln c
+  float rcp[128], log[128];  // 1 / c, 2 ln c
 };
 constexpr int kNoiseTableFloats = 896;
 constexpr uint32_t kLogBase = 0x3f348000u;  // the float 0.705078125: where m's cells begin
@@ -155,7 +155,7 @@ constexpr NoiseTables make_noise_tables() {
     const double c = bits < 0x800000 ? 0.5 + bits / 16777216.0 : 1.0 + (bits - 0x800000) / 8388608.0;
     const float r = i == 75 ? 1.0f : static_cast<float>(1.0 / c);
     t.rcp[i] = r;
-    t.log[i] = static_cast<float>(2.0 * table_math::log_near_one(static_cast<double>(r)));  // -2 ln(1 / r)
+    t.log[i] = static_cast<float>(-2.0 * table_math::log_near_one(static_cast<double>(r)));  // 2 ln(1 / r)
   }
   return t;
 }
@@ -183,21 +183,25 @@ __device__ __forceinline__ void box_muller(const uint32_t* wa, const uint32_t* w
     rc.set(i, cell[0]);
     lg.set(i, cell[128]);
     o.set(i, __uint_as_float(0x3f800000u | (wb[i] & 0x007ffe00u)));  // 1 + (14 bits) 2^-14
-    const float* dir = tab + (wb[i] >> 23);
+    const float* dir = tab + ((wb[i] >> 23) ^ 256u);  // the opposite direction: minus signs
     sn.set(i, dir[0]);
     cs.set(i, dir[128]);
   }
   const T t = fma(m, rc, T(-1.0f));
-  const T lm = fma(t, fma(t, fma(t, T(-0.666666666666666667f), T(1.0f)), T(-2.0f)), lg);  // -2 ln m
-  const T r2 = fma(ef, T(-1.6525916589735634e-07f), lm);                                   // -2 ln 2 2^-23
-  const T radius = r2 * vrsqrt(r2);  // r2 in [1.2e-7, 33.3]
+  const T lm = fma(t, fma(t, fma(t, T(0.666666666666666667f), T(-1.0f)), T(2.0f)), lg);  // 2 ln m
+  const T q2 = fma(ef, T(1.6525916589735634e-07f), lm);                                  // 2 ln u; 2 ln 2 2^-23
+  // -sqrt(-q2), -q2 in [1.2e-7, 33.3]: MUFU reciprocal square root and one
+  // Newton step (0.6 ulp against 2.5)
+  const T y = vrsqrt(-q2);
+  T nrad = q2 * y;
+  nrad = fma(T(0.5f) * y, fma(nrad, nrad, q2), nrad);
   // d = (o + 2^-15 - 3/2) 2 pi / 512
   const T dd = fma(o, T(0.01227184630308513f), T(-0.018407394947599402f));
   const T w = (T(-0.5f) * dd) * dd;  // cos d - 1
   const T sd = dd * fma(w, T(0.333333333333333333f), T(1.0f));
   // the turn's small part by itself: one rounding at the size of the result
-  n0 = radius * (cs + fma(T(-1.0f) * sn, sd, cs * w));
-  n1 = radius * (sn + fma(cs, sd, sn * w));
+  n0 = nrad * (cs + fma(-sn, sd, cs * w));
+  n1 = nrad * (sn + fma(cs, sd, sn * w));
 }
 
 }  // namespace brmppi

@@ -61,11 +61,11 @@
 //   S2 = M_u + m_alpha sum u_i u_i^T,  g = m_alpha sum u_i rho_i,
 // so the rows accumulate the sums and m_alpha is applied once.
 //
-// Numerics: states are carried relative to the initial pose (position
-// relative to (px0, py0), angles relative to theta1_0, progress relative to
-// psi0) so that binary32 rounding is relative to the few metres a rollout
-// travels; position, speed, progress and the cost sum are compensated pairs
-// (TwoSum); the softmin works on pair differences.
+// Numerics: states are carried in the frame of the initial pose (position
+// along and across the initial heading, angles and progress relative to it)
+// so that binary32 rounding is relative to the few metres a rollout travels;
+// position, speed, progress and the cost sum are compensated pairs (TwoSum),
+// the path table holds low parts; the softmin works on pair differences.
 #pragma once
 
 #include <cstdint>
@@ -128,7 +128,7 @@ struct Inst {
   float* part;       // tiles * part_stride floats
   unsigned int* sync;  // [0] finished tiles, [1] error bits
   int S, H, n_obs, n_pts, tiles, part_stride;
-  float ds, inv_ds;
+  float ds, inv_ds, inv_ds_l;  // 1 / ds and its low part
   double inv_ds_d;   // 1 / ds in FP64 (path cell of psi0)
   uint32_t key0, key1, ctr;
   int P;             // Philox blocks per step, ceil((4 + n_obs) / 4)
@@ -300,11 +300,14 @@ __device__ __forceinline__ void hitch_stabilize(const KConst& k, float Delta, fl
   out[3] = (g0 * a + g1 * w) - rhs;
 }
 
-// Frame of one solve (relative coordinates).  Doubles of x0 enter as
-// unevaluated float pairs (hi + lo), so the staging needs no FP64 trig.
+// Frame of one solve: origin and heading of the tractor at x0.  Rollouts run
+// in it: x along the initial heading, angles relative to it, so neither the
+// step nor the cost turns by the initial heading, and the rounding of its cos
+// / sin (3e-8, the same at every step, so a drift of the whole rollout) enters
+// nowhere.  Doubles of x0 enter as unevaluated float pairs (hi + lo).
 struct Frame {
   float ox_h, ox_l, oy_h, oy_l, oth_h, oth_l;  // origin (px0, py0, theta1_0)
-  float c0, s0;                                // cos / sin of theta1_0
+  float c0, s0, c0l, s0l;                      // cos / sin of theta1_0, and their low parts
   float t2, v_h, v_l, dl;                      // theta2 - theta1_0, speed, steer angle
   float a0;                                    // acceleration (jerk-input model)
   float qf0;                                   // fractional path cell of psi0
@@ -312,6 +315,42 @@ struct Frame {
   float psi_h, psi_l;                          // psi0
   double psi0;
 };
+
+// sin and cos of the frame's heading hi + lo as float pairs, to about 2e-9:
+// Cody-Waite reduction by pi/2 in three parts, then the Taylor series with its
+// leading terms in pairs (one lane a CTA; in FP64 it took 0.4 us).
+__device__ __forceinline__ void frame_sincos(float hi, float lo, float* s, float* sl, float* c, float* cl) {
+  if (!(fabsf(hi) < 1.0e6f)) {  // (NaN too) a float's accuracy
+    sincosf(hi, s, c);
+    *sl = *c * lo;
+    *cl = -*s * lo;
+    return;
+  }
+  const float k = rintf(hi * 0.636619746685028f);
+  const float r0 = __fmaf_rn(-k, 1.5707963705062866f, hi);  // exact
+  const float r = __fmaf_rn(k, 4.371138828673793e-08f, r0);
+  const float rl = __fmaf_rn(k, 4.371138828673793e-08f, __fsub_rn(r0, r)) + fmaf(k, 1.7151245100058e-15f, lo);
+  const float z = __fmul_rn(r, r), zl = __fmaf_rn(r, r, -z);  // of r alone: rl turns the result below
+  // sin = r + r w, w = z (-1/6 + z/120 - ...)
+  const float A = fmaf(z, fmaf(z, fmaf(z, 2.7557319e-06f, -1.9841270e-04f), 8.3333333e-03f), -0.16666667f);
+  const float w = __fmul_rn(z, A), wl = __fmaf_rn(z, A, -w) + zl * A;
+  const float p = __fmul_rn(r, w), pl = __fmaf_rn(r, w, -p) + r * wl;
+  const float sh = __fadd_rn(r, p), se = __fadd_rn(__fsub_rn(r, sh), p) + pl;  // |r| >= |p|
+  // cos = 1 - z/2 + z^2 (1/24 - z/720 + ...)
+  const float C = fmaf(z, fmaf(z, fmaf(z, -2.7557319e-07f, 2.4801587e-05f), -1.3888889e-03f), 0.041666667f);
+  const float ch = __fmaf_rn(-0.5f, z, 1.f);
+  const float ce = __fmaf_rn(-0.5f, z, __fsub_rn(1.f, ch)) + fmaf(z * z, C, -0.5f * zl);
+  const float sl_ = fmaf(ch, rl, se), cl_ = fmaf(-sh, rl, ce);
+  const float s1 = __fadd_rn(sh, sl_), s1l = __fadd_rn(__fsub_rn(sh, s1), sl_);
+  const float c1 = __fadd_rn(ch, cl_), c1l = __fadd_rn(__fsub_rn(ch, c1), cl_);
+  const int q = static_cast<int>(k);
+  const bool odd = q & 1, sneg = q & 2, cneg = (q + 1) & 2;
+  const float ss = odd ? c1 : s1, ssl = odd ? c1l : s1l, cc = odd ? s1 : c1, ccl = odd ? s1l : c1l;
+  *s = sneg ? -ss : ss;
+  *sl = sneg ? -ssl : ssl;
+  *c = cneg ? -cc : cc;
+  *cl = cneg ? -ccl : ccl;
+}
 
 // The frame of x0, built by warp 0: lane j takes state component j, so the
 // FP64 work runs side by side; the path cell of psi0 uses the host's FP64
@@ -333,10 +372,7 @@ __device__ __forceinline__ void make_frame_warp(const double* x0, double inv_ds,
     case 2: {
       fr.oth_h = hi;
       fr.oth_l = lo;
-      float sn, cs;
-      sincosf(hi, &sn, &cs);
-      fr.c0 = cs - sn * lo;  // cos(hi + lo), lo below one ulp of hi
-      fr.s0 = sn + cs * lo;
+      frame_sincos(hi, lo, &fr.s0, &fr.s0l, &fr.c0, &fr.c0l);
       break;
     }
     case 3: fr.t2 = static_cast<float>(x - x0[2]); break;
@@ -364,7 +400,7 @@ struct Smem {
                  // ky, vx', vy' with k = 1/A^2 (e = 2) or 1/A^4 (e = 4, kx
                  // stored negated) and the velocity in the obstacle frame
                  // (zero unless moving)
-  float* path;   // 3 per row: x, y, heading (relative frame)
+  float* path;   // 4 per row: x, y, heading in the frame, low parts of x and y
   float* unom;   // 3H: the nominal inputs in the projection's coordinates
   float* ustar;  // 3H + 1 (merge)
   float* jh;     // spb
@@ -423,6 +459,9 @@ __device__ __forceinline__ void prefetch_l2(const void* p) {
   if (p) asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
 }
 
+// Barrier of the whole CTA that its roles reach at different places.
+__device__ __forceinline__ void staging_barrier() { asm volatile("bar.sync 0;" ::: "memory"); }
+
 // Threads of a CTA that roll out samples: all of them with one lane per
 // sample; with wider teams the last noise_warps warps produce the noise.
 template <int TPS>
@@ -438,17 +477,48 @@ constexpr bool kNoiseWarps = TPS > 1 && BPT <= 2 && NS == 1;
 __device__ __forceinline__ void store_pair(float* d, Vec<1> a) { *d = a.x; }
 __device__ __forceinline__ void store_pair(float* d, Vec<2> a) { *reinterpret_cast<float2*>(d) = a.x; }
 
-// The reference path into shared memory, three floats a row (x, y, heading):
-// the raw rows in flight, then (after a barrier) their shift into the frame.
-__device__ __forceinline__ void stage_path(const Inst& in, const Smem& S) {
-  for (int j = threadIdx.x; j < 3 * in.n_pts; j += blockDim.x) cp_async4(S.path + j, in.path + j);
+// (hi, lo) = (x, y) - origin in the frame's axes: c dx + s dy as a float pair
+// (for the y axis, called with (dy, -dx)).
+__device__ __forceinline__ void frame_axis(const Frame& fr, float dxh, float dxl, float dyh, float dyl, float& hi,
+                                           float& lo) {
+  const float p = __fmul_rn(fr.c0, dxh), q = __fmul_rn(fr.s0, dyh);
+  const float pe = __fmaf_rn(fr.c0, dxh, -p), qe = __fmaf_rn(fr.s0, dyh, -q);
+  const float sum = __fadd_rn(p, q), bp = __fsub_rn(sum, p);
+  const float se = __fadd_rn(__fsub_rn(p, __fsub_rn(sum, bp)), __fsub_rn(q, bp));
+  const float l = (se + (pe + qe)) + fmaf(fr.c0, dxl, fmaf(fr.s0, dyl, fmaf(fr.c0l, dxh, fr.s0l * dyh)));
+  hi = __fadd_rn(sum, l);
+  lo = __fadd_rn(__fsub_rn(sum, hi), l);
 }
-__device__ __forceinline__ void shift_path(const Inst& in, const Smem& S, const Frame& fr) {
-  for (int j = threadIdx.x; j < in.n_pts; j += blockDim.x) {
-    float* d = S.path + 3 * j;
-    d[0] = (d[0] - fr.ox_h) - fr.ox_l;
-    d[1] = (d[1] - fr.oy_h) - fr.oy_l;
-    d[2] = (d[2] - fr.oth_h) - fr.oth_l;
+// a - (oh + ol) as a float pair
+__device__ __forceinline__ void minus_origin(float a, float oh, float ol, float& hi, float& lo) {
+  hi = __fsub_rn(a, oh);
+  const float bp = __fsub_rn(hi, a);
+  lo = __fsub_rn(__fsub_rn(__fsub_rn(a, __fsub_rn(hi, bp)), __fadd_rn(oh, bp)), ol);
+}
+__device__ __forceinline__ void into_frame(const Frame& fr, float x, float y, float& xh, float& xl, float& yh, float& yl) {
+  float dxh, dxl, dyh, dyl;
+  minus_origin(x, fr.ox_h, fr.ox_l, dxh, dxl);
+  minus_origin(y, fr.oy_h, fr.oy_l, dyh, dyl);
+  frame_axis(fr, dxh, dxl, dyh, dyl, xh, xl);
+  frame_axis(fr, dyh, dyl, -dxh, -dxl, yh, yl);
+}
+
+// The reference path into shared memory, one float4 a row: x, y, heading in
+// the frame, and the low parts of x and y (bfloat16 each, in one word): at
+// 15 m a float's half ulp is 5e-7 m, and the softmin sees the costs of errors
+// of that size.  First the raw rows in flight, then (after a barrier) their
+// move into the frame.
+__device__ __forceinline__ void stage_path(const Inst& in, const Smem& S) {
+  for (int j = threadIdx.x; j < 3 * in.n_pts; j += blockDim.x) cp_async4(S.path + j + j / 3, in.path + j);
+}
+__device__ __forceinline__ void shift_path(const Inst& in, const Smem& S, const Frame& fr, int threads) {
+  for (int j = threadIdx.x; j < in.n_pts; j += threads) {
+    float4* d = reinterpret_cast<float4*>(S.path) + j;
+    const float4 raw = *d;
+    float xh, xl, yh, yl;
+    into_frame(fr, raw.x, raw.y, xh, xl, yh, yl);
+    const uint32_t lo = ((__float_as_uint(xl) + 0x8000u) >> 16) | ((__float_as_uint(yl) + 0x8000u) & 0xffff0000u);
+    *d = make_float4(xh, yh, (raw.z - fr.oth_h) - fr.oth_l, __uint_as_float(lo));
   }
 }
 
@@ -535,7 +605,8 @@ __device__ void run_tile(const KConst& k, const Inst& in, int tile, float* uh, c
   // noise leaves the compute warps' dependency chain).
   const int nc = compute_threads<TPS>(noise_warps);
   const int spb = nc / TPS * NS;
-  const bool producer = kNoiseWarps<TPS, BPT, NS> && static_cast<int>(threadIdx.x) >= nc;
+  constexpr bool PRODUCED = kNoiseWarps<TPS, BPT, NS>;
+  const bool producer = PRODUCED && static_cast<int>(threadIdx.x) >= nc;
   const int team = producer ? 0 : static_cast<int>(threadIdx.x) / TPS;
   const int lt = threadIdx.x % TPS;
   const int s = tile * spb + team * NS;  // the team's first sample
@@ -559,26 +630,32 @@ __device__ void run_tile(const KConst& k, const Inst& in, int tile, float* uh, c
   stage_path(in, S);
   stage_noise(in, S);
   for (int j = threadIdx.x; j < 3 * H; j += blockDim.x) cp_async4(S.unom + j, in.U_nom + j);
+  // obstacles by the compute threads after warp 0 (which builds the frame)
+  const int n_stage = PRODUCED ? nc : static_cast<int>(blockDim.x);
+  const int o0_ = static_cast<int>(threadIdx.x) - 32;
+  const bool has_ob0 = !producer && o0_ >= 0 && o0_ < in.n_obs;
   float ob0[8];
-  const bool has_ob0 = static_cast<int>(threadIdx.x) < in.n_obs;
 #pragma unroll
-  for (int q = 0; q < 8; ++q) ob0[q] = (has_ob0 && q < ostride) ? in.obs[ostride * threadIdx.x + q] : 0.f;
+  for (int q = 0; q < 8; ++q) ob0[q] = (has_ob0 && q < ostride) ? in.obs[ostride * o0_ + q] : 0.f;
   if (threadIdx.x < 32) make_frame_warp(in.x0, in.inv_ds_d, in.sync + 1, sh.fr, EXT && k.jerk);
+  float sin0 = 0.f, cos0 = 0.f;
+  if (has_ob0) sincosf(ob0[4], &sin0, &cos0);
   cp_async_wait_all();
   __syncthreads();
   const Frame& fr = sh.fr;
-  auto stage_obstacle = [&](int o, float cx, float cy, float ax, float ay, float th, float e, float vx, float vy) {
+  auto stage_obstacle = [&](int o, float cx, float cy, float ax, float ay, float sw, float cw_, float e, float vx,
+                            float vy) {
     float* d = S.obs + 8 * o;
     const bool e4 = obs8 && e == 4.0f;
     if (e != 2.0f && !e4) atomicOr(in.sync + 1, ERR_EXPONENT);
     const float Ax = ax + k.r_inflate, Ay = ay + k.r_inflate;
-    d[0] = (cx - fr.ox_h) - fr.ox_l;
-    d[1] = (cy - fr.oy_h) - fr.oy_l;
-    float so, co;
-    sincosf(th, &so, &co);
+    float cxl, cyl;
+    into_frame(fr, cx, cy, d[0], cxl, d[1], cyl);
+    // the obstacle's axes in the frame
+    const float co = fmaf(fr.c0, cw_, fr.s0 * sw), so = fmaf(fr.c0, sw, -(fr.s0 * cw_));
     const float ix = 1.0f / (Ax * Ax), iy = 1.0f / (Ay * Ay);
     if constexpr (!EXT) {
-      // parked ellipses: h = d^T Q d - 1 with d the offset in world axes and
+      // parked ellipses: h = d^T Q d - 1 with d the offset in the frame and
       // Q = R^T diag(ix, iy) R (R the rotation into the obstacle's axes):
       // (Qxx, Qxy) in place of (cos, sin), Qyy in slot 4
       const float c2 = co * co, s2 = so * so;
@@ -591,43 +668,120 @@ __device__ void run_tile(const KConst& k, const Inst& in, int tile, float* uh, c
       d[3] = so;
       d[4] = e4 ? -(ix * ix) : ix;
       d[5] = e4 ? iy * iy : iy;
-      d[6] = co * vx + so * vy;
-      d[7] = co * vy - so * vx;
+      d[6] = cw_ * vx + sw * vy;
+      d[7] = cw_ * vy - sw * vx;
     }
   };
-  // one row past the obstacles: h = -1 everywhere with no gradient, so a
-  // padding slot that reads it adds exactly nothing to the projection's sums
-  if (threadIdx.x < 8) S.obs[8 * in.n_obs + threadIdx.x] = 0.f;
-  if (has_ob0) stage_obstacle(threadIdx.x, ob0[0], ob0[1], ob0[2], ob0[3], ob0[4], ob0[5], ob0[6], ob0[7]);
-  for (int o = threadIdx.x + blockDim.x; o < in.n_obs; o += blockDim.x) {
-    const float* ob = in.obs + ostride * o;
-    stage_obstacle(o, ob[0], ob[1], ob[2], ob[3], ob[4], ob[5], obs8 ? ob[6] : 0.f, obs8 ? ob[7] : 0.f);
-  }
-  shift_path(in, S, fr);
-  for (int j = threadIdx.x; j < 3 * H; j += blockDim.x) {  // nominal inputs in the projection's coordinates
-    const int q = j % 3;
-    S.unom[j] = fmaf(k.qa[q], S.unom[j], k.qb[q]);
-  }
-  if (threadIdx.x < 4) S.chunk[threadIdx.x] = k.pc_am;  // (free until the merge)
-  if constexpr (EXT) {
-#pragma unroll
-    for (int m = 0; m < 8; ++m)
-      if (static_cast<int>(threadIdx.x) == m) {
-        S.disc[2 * m] = k.disc_e1[m];
-        S.disc[2 * m + 1] = k.disc_e2[m];
+  // nominal inputs in the projection's coordinates (threads `first`,
+  // first + stride, ...)
+  auto map_inputs = [&](int first, int stride) {
+    for (int j = first; j < 3 * H; j += stride) {
+      const int q = j % 3;
+      S.unom[j] = fmaf(k.qa[q], S.unom[j], k.qb[q]);
+    }
+  };
+  // Producer warps (latency shapes): while the compute warps move the tables
+  // into the frame, they map the nominal inputs and draw the first step.
+  const int P_drawn = k.proj ? in.P : 1;  // standard MPPI needs the input normals only
+  const int pl = static_cast<int>(threadIdx.x) - nc;
+  const int n_blocks = spb * P_drawn, n_prod = 32 * noise_warps;
+  // what block b's normals sample: block 0 the inputs (around the nominal
+  // ones) and the hitch's rate, others four rows' rates
+  struct Draw {
+    PhiloxBlock pb;
+    PhiloxSample smp;
+    float s0, s1, s2, lo0, lo1, lo2, hi0, hi1, hi2;
+    const float* nom;
+    int nom_stride;
+    float* dst;
+  };
+  auto make_draw = [&](int i) {
+    const int tm = i / P_drawn, b = i - tm * P_drawn;
+    const bool first = b == 0;
+    Draw d;
+    d.pb = load_block(S, b);
+    d.smp = philox_sample(static_cast<uint32_t>(tile * spb + tm));
+    d.s0 = first ? k.qs[0] : k.ps;
+    d.s1 = first ? k.qs[1] : k.ps;
+    d.s2 = first ? k.qs[2] : k.ps;
+    d.lo0 = first ? k.qlo[0] : k.pam_lo;
+    d.lo1 = first ? k.qlo[1] : k.pam_lo;
+    d.lo2 = first ? k.qlo[2] : k.pam_lo;
+    d.hi0 = first ? k.qhi[0] : k.pam_hi;
+    d.hi1 = first ? k.qhi[1] : k.pam_hi;
+    d.hi2 = first ? k.qhi[2] : k.pam_hi;
+    d.nom = first ? S.unom : S.chunk;
+    d.nom_stride = first ? 3 : 0;
+    d.dst = S.noise + tm * S.noise_per_team + 4 * b;
+    return d;
+  };
+  auto produce = [&](const Draw& d, int tau_d) {
+    const uint4 w = philox_words(d.pb, d.smp, philox_step(d.smp, static_cast<uint32_t>(tau_d), in.key0, in.key1),
+                                 in.key0, in.key1);
+    const float* nom = d.nom + tau_d * d.nom_stride;
+    Vec<1> g0, g1, g2, g3;
+    box_muller<1>(&w.x, &w.y, S.tab, g0, g1);
+    box_muller<1>(&w.z, &w.w, S.tab, g2, g3);
+    g0 = vclamp(fma(Vec<1>(d.s0), g0, Vec<1>(nom[0])), d.lo0, d.hi0);
+    g1 = vclamp(fma(Vec<1>(d.s1), g1, Vec<1>(nom[1])), d.lo1, d.hi1);
+    g2 = vclamp(fma(Vec<1>(d.s2), g2, Vec<1>(nom[2])), d.lo2, d.hi2);
+    g3 = sampled_rate(k, g3);
+    *reinterpret_cast<float4*>(d.dst + (tau_d & 1) * 4 * in.P) = make_float4(g0.x, g1.x, g2.x, g3.x);
+  };
+  // Step tau's barrier hands its draws over; the first draws are made before
+  // the staging barrier.
+  if (producer) {
+    map_inputs(pl, n_prod);
+    if (pl < 4) S.chunk[pl] = k.pc_am;  // (free until the merge)
+    asm volatile("bar.sync 2, %0;" ::"r"(n_prod) : "memory");
+    if (n_blocks <= n_prod) {
+      // at most one block a thread (the usual case): what the steps share
+      // stays in registers
+      const Draw d = make_draw(min(pl, n_blocks - 1));
+      for (int tau = 0; tau < H; ++tau) {
+        if (pl < n_blocks) produce(d, tau);
+        if (tau == 0) staging_barrier();
+        step_barrier();
       }
+    } else {
+      for (int tau = 0; tau < H; ++tau) {
+        for (int i = pl; i < n_blocks; i += n_prod) produce(make_draw(i), tau);
+        if (tau == 0) staging_barrier();
+        step_barrier();
+      }
+    }
   }
-  __syncthreads();
+  if (!producer) {
+    // one row past the obstacles: h = -1 everywhere with no gradient, so a
+    // padding slot that reads it adds exactly nothing to the projection's sums
+    if (threadIdx.x < 8) S.obs[8 * in.n_obs + threadIdx.x] = 0.f;
+    if (has_ob0) stage_obstacle(o0_, ob0[0], ob0[1], ob0[2], ob0[3], sin0, cos0, ob0[5], ob0[6], ob0[7]);
+    for (int o = o0_ + n_stage - 32; o0_ >= 0 && o < in.n_obs; o += n_stage - 32) {
+      const float* ob = in.obs + ostride * o;
+      float so, co;
+      sincosf(ob[4], &so, &co);
+      stage_obstacle(o, ob[0], ob[1], ob[2], ob[3], so, co, ob[5], obs8 ? ob[6] : 0.f, obs8 ? ob[7] : 0.f);
+    }
+    shift_path(in, S, fr, n_stage);
+    if constexpr (!PRODUCED) map_inputs(threadIdx.x, blockDim.x);
+    if constexpr (EXT) {
+#pragma unroll
+      for (int m = 0; m < 8; ++m)
+        if (static_cast<int>(threadIdx.x) == m) {
+          S.disc[2 * m] = k.disc_e1[m];
+          S.disc[2 * m + 1] = k.disc_e2[m];
+        }
+    }
+    staging_barrier();
+  }
 
   // --- per-sample state (relative frame)
-  const T c0 = fr.c0, s0 = fr.s0;
   T acc = fr.a0;  // acceleration state of the jerk-input model
   T px = 0.f, pxl = 0.f, py = 0.f, pyl = 0.f, t1 = 0.f, t2 = fr.t2, v = fr.v_h, vl = fr.v_l, dl = fr.dl, ps = 0.f,
     psl = 0.f;
   // obstacle slots per lane of the producer variants: 4 BPT; ROWS > 0: exactly
   // ROWS
   static_assert(ROWS == 0 || kNoiseWarps<TPS, BPT, NS>, "exact row slots need the noise-warp variants");
-  constexpr bool PRODUCED = kNoiseWarps<TPS, BPT, NS>;
   constexpr int OBS_SLOTS = !PRODUCED ? 1 : (ROWS > 0 ? ROWS : 4 * BPT);
   T alpha_h = k.alpha0;  // the hitch's barrier rate (same on every lane)
   T alpha[OBS_SLOTS];    // the rows' rates (producer variants: in registers)
@@ -712,10 +866,13 @@ __device__ void run_tile(const KConst& k, const Inst& in, int tile, float* uh, c
     // path cell: floor of qf by the 1.5 * 2^23 shifter on qf - 1/2 (an exact
     // integer may take the cell below with ff = 1, the same point); the
     // clamp keeps the shifter in range far outside any path
-    const T qf = vclamp(qf0 + fma(x.ps, T(in.inv_ds), x.psl * T(in.inv_ds)), -2.0e6f, 2.0e6f);
+    const T qf = vclamp(fma(x.ps, T(in.inv_ds), qf0), -2.0e6f, 2.0e6f);
     const T tt = (qf + T(-0.5f)) + T(12582912.0f);
-    T ff = qf - (tt + T(-12582912.0f));
-    T x0r, y0r, t0r, x1r, y1r, t1r;
+    const T fl = tt + T(-12582912.0f);
+    // ff = qf - fl, with the cancelling parts in one fused operation and the
+    // reciprocal's and the progress's low parts: rounded at the size of ff
+    T ff = (fma(x.ps, T(in.inv_ds), -fl) + qf0) + fma(x.psl, T(in.inv_ds), x.ps * T(in.inv_ds_l));
+    T x0r, y0r, t0r, x1r, y1r, t1r, x0l, y0l, x1l, y1l;
 #pragma unroll
     for (int i = 0; i < NS; ++i) {
       int ii = i0 + (__float_as_int(tt.get(i)) - 0x4b400000);
@@ -726,27 +883,35 @@ __device__ void run_tile(const KConst& k, const Inst& in, int tile, float* uh, c
         ii = n_pts - 2;
         ff.set(i, 1.f);
       }
-      const float* r = S.path + 3 * ii;
-      x0r.set(i, r[0]);
-      y0r.set(i, r[1]);
-      t0r.set(i, r[2]);
-      x1r.set(i, r[3]);
-      y1r.set(i, r[4]);
-      t1r.set(i, r[5]);
+      const float4 a = *reinterpret_cast<const float4*>(S.path + 4 * ii);
+      const float4 b = *reinterpret_cast<const float4*>(S.path + 4 * ii + 4);
+      x0r.set(i, a.x);
+      y0r.set(i, a.y);
+      t0r.set(i, a.z);
+      x1r.set(i, b.x);
+      y1r.set(i, b.y);
+      t1r.set(i, b.z);
+      x0l.set(i, __uint_as_float(__float_as_uint(a.w) << 16));
+      y0l.set(i, __uint_as_float(__float_as_uint(a.w) & 0xffff0000u));
+      x1l.set(i, __uint_as_float(__float_as_uint(b.w) << 16));
+      y1l.set(i, __uint_as_float(__float_as_uint(b.w) & 0xffff0000u));
     }
-    const T xr = fma(ff, x1r - x0r, x0r), yr = fma(ff, y1r - y0r, y0r), thr = fma(ff, t1r - t0r, t0r);
-    const T dxr = (x.px - xr) + x.pxl, dyr = (x.py - yr) + x.pyl;
+    // offsets from the row, less the part along the segment: sums of small
+    // terms, whatever the distance from the origin
+    const T nf = -ff;
+    const T dxr = fma(nf, x1r - x0r, x.px - x0r) + fma(nf, x1l - x0l, x.pxl - x0l);
+    const T dyr = fma(nf, y1r - y0r, x.py - y0r) + fma(nf, y1l - y0l, x.pyl - y0l);
+    const T seg = t1r - t0r;
     T rc;
     if (k.iso) {
       rc = T(k.Ql) * fma(dxr, dxr, dyr * dyr);
     } else {
-      T sr, cr;
-      state_sincos(thr, &sr, &cr);
-      const T cth = fma(c0, cr, -(s0 * sr)), sth = fma(s0, cr, c0 * sr);  // the path's heading in world axes
+      T sth, cth;  // the path's heading in the frame
+      state_sincos(fma(ff, seg, t0r), &sth, &cth);
       const T ec = fma(sth, dxr, -(cth * dyr)), el = fma(cth, dxr, sth * dyr);
       rc = fma(T(k.Ql) * el, el, T(k.Qc) * ec * ec);
     }
-    const T e1 = wrap_pi(x.t1 - thr), e2 = wrap_pi(x.t2 - thr);
+    const T e1 = wrap_pi(fma(nf, seg, x.t1 - t0r)), e2 = wrap_pi(fma(nf, seg, x.t2 - t0r));
     const T dn = T(k.nu_bar) - x.un;
     rc = fma(T(k.Qth), fma(e1, e1, e2 * e2), rc);
     rc = fma(T(k.R0) * x.ua, x.ua, rc);
@@ -804,8 +969,10 @@ __device__ void run_tile(const KConst& k, const Inst& in, int tile, float* uh, c
     for (int i = 0; i < NS; ++i) {
       if (s + i >= in.S) break;
       float* o = in.states_out + (static_cast<size_t>(s + i) * static_cast<size_t>(H + 1) + tau) * 7;
-      o[0] = (fr.ox_h + px.get(i)) + (fr.ox_l + pxl.get(i));
-      o[1] = (fr.oy_h + py.get(i)) + (fr.oy_l + pyl.get(i));
+      o[0] = fr.ox_h + (fmaf(fr.c0, px.get(i), -(fr.s0 * py.get(i))) +
+                        (fr.ox_l + fmaf(fr.c0, pxl.get(i), -(fr.s0 * pyl.get(i)))));
+      o[1] = fr.oy_h + (fmaf(fr.s0, px.get(i), fr.c0 * py.get(i)) +
+                        (fr.oy_l + fmaf(fr.s0, pxl.get(i), fr.c0 * pyl.get(i))));
       o[2] = (fr.oth_h + t1.get(i)) + fr.oth_l;
       o[3] = (fr.oth_h + t2.get(i)) + fr.oth_l;
       o[4] = v.get(i) + vl.get(i);
@@ -828,77 +995,6 @@ __device__ void run_tile(const KConst& k, const Inst& in, int tile, float* uh, c
   // (inputs and hitch) is needed by the whole team: lane lt draws it for step
   // tau + lt once every TPS steps, and each step takes it from its lane.
   float* nz = S.noise + team * S.noise_per_team;  // [2][P][4] (producer variants)
-  const int P_drawn = k.proj ? in.P : 1;  // standard MPPI needs the input normals only
-  if constexpr (kNoiseWarps<TPS, BPT, NS>) {
-    if (producer) {
-      // thread pl draws block i of the CTA's spb P_drawn each step, i = pl,
-      // pl + 32 noise_warps, ...; with at most one block a thread (the usual
-      // case) what the steps share stays in registers
-      const int pl = static_cast<int>(threadIdx.x) - nc;
-      const int n_blocks = spb * P_drawn, stride = 32 * noise_warps;
-      // what block b's normals sample: block 0 the inputs (around the nominal
-      // ones) and the hitch's rate, others four rows' rates
-      struct Draw {
-        PhiloxBlock pb;
-        PhiloxSample smp;
-        float s0, s1, s2, lo0, lo1, lo2, hi0, hi1, hi2;
-        const float* nom;
-        int nom_stride;
-        float* dst;
-      };
-      auto make_draw = [&](int i) {
-        const int tm = i / P_drawn, b = i - tm * P_drawn;
-        const bool first = b == 0;
-        Draw d;
-        d.pb = load_block(S, b);
-        d.smp = philox_sample(static_cast<uint32_t>(tile * spb + tm));
-        d.s0 = first ? k.qs[0] : k.ps;
-        d.s1 = first ? k.qs[1] : k.ps;
-        d.s2 = first ? k.qs[2] : k.ps;
-        d.lo0 = first ? k.qlo[0] : k.pam_lo;
-        d.lo1 = first ? k.qlo[1] : k.pam_lo;
-        d.lo2 = first ? k.qlo[2] : k.pam_lo;
-        d.hi0 = first ? k.qhi[0] : k.pam_hi;
-        d.hi1 = first ? k.qhi[1] : k.pam_hi;
-        d.hi2 = first ? k.qhi[2] : k.pam_hi;
-        d.nom = first ? S.unom : S.chunk;
-        d.nom_stride = first ? 3 : 0;
-        d.dst = S.noise + tm * S.noise_per_team + 4 * b;
-        return d;
-      };
-      auto produce = [&](const Draw& d, int tau_d) {
-        const uint4 w = philox_words(d.pb, d.smp, philox_step(d.smp, static_cast<uint32_t>(tau_d), in.key0, in.key1),
-                                     in.key0, in.key1);
-        const float* nom = d.nom + tau_d * d.nom_stride;
-        Vec<1> g0, g1, g2, g3;
-        box_muller<1>(&w.x, &w.y, S.tab, g0, g1);
-        box_muller<1>(&w.z, &w.w, S.tab, g2, g3);
-        g0 = vclamp(fma(Vec<1>(d.s0), g0, Vec<1>(nom[0])), d.lo0, d.hi0);
-        g1 = vclamp(fma(Vec<1>(d.s1), g1, Vec<1>(nom[1])), d.lo1, d.hi1);
-        g2 = vclamp(fma(Vec<1>(d.s2), g2, Vec<1>(nom[2])), d.lo2, d.hi2);
-        g3 = sampled_rate(k, g3);
-        *reinterpret_cast<float4*>(d.dst + (tau_d & 1) * 4 * in.P) = make_float4(g0.x, g1.x, g2.x, g3.x);
-      };
-      if (n_blocks <= stride) {
-        const Draw d = make_draw(min(pl, n_blocks - 1));
-        const bool mine = pl < n_blocks;
-        if (mine) produce(d, 0);
-        for (int tau = 0; tau < H; ++tau) {
-          step_barrier();
-          if (mine && tau + 1 < H) produce(d, tau + 1);
-        }
-      } else {
-        auto produce_all = [&](int tau_d) {
-          for (int i = pl; i < n_blocks; i += stride) produce(make_draw(i), tau_d);
-        };
-        produce_all(0);
-        for (int tau = 0; tau < H; ++tau) {
-          step_barrier();
-          if (tau + 1 < H) produce_all(tau + 1);
-        }
-      }
-    }
-  }
   T z0[4];  // in-register noise: this lane's sampled (a, omega, nu) and hitch rate
   // trigonometry of the current state, carried from step to step: the state
   // angles theta1 and phi = theta1 - theta2 of step tau + 1 follow from step
@@ -907,13 +1003,8 @@ __device__ void run_tile(const KConst& k, const Inst& in, int tile, float* uh, c
   // and stay off its dependency chain; only the steer angle's trigonometry
   // waits for the projection.
   T c1, s1, sp, cp;
-  {
-    T sr, cr;
-    state_sincos(t1, &sr, &cr);
-    c1 = fma(c0, cr, -(s0 * sr));
-    s1 = fma(s0, cr, c0 * sr);
-    state_sincos(t1 - t2, &sp, &cp);
-  }
+  state_sincos(t1, &s1, &c1);
+  state_sincos(t1 - t2, &sp, &cp);
   // One step; PROJ is fixed for the whole loop (no branch on the flag
   // inside the step).
   auto step = [&](int tau, auto proj_c) {
@@ -985,7 +1076,6 @@ __device__ void run_tile(const KConst& k, const Inst& in, int tile, float* uh, c
       acc2(py_n, pyl_n, Tv * s1);
       t1_n = fma(T(k.Ts), th1dot, t1);
       t2_n = fma(T(k.Ts), th2dot, t2);
-      T sr, cr;
       if constexpr (TPS > 1) {
         // even lanes take theta1, odd lanes phi, and each pair trades the
         // results: one sin / cos sequence in the warp's stream instead of two
@@ -993,16 +1083,14 @@ __device__ void run_tile(const KConst& k, const Inst& in, int tile, float* uh, c
         T sa, ca;
         state_sincos(odd ? t1_n - t2_n : t1_n, &sa, &ca);
         const T sb = vshfl_xor(sa, 1), cb = vshfl_xor(ca, 1);
-        sr = odd ? sb : sa;
-        cr = odd ? cb : ca;
+        s1_n = odd ? sb : sa;
+        c1_n = odd ? cb : ca;
         sp_n = odd ? sa : sb;
         cp_n = odd ? ca : cb;
       } else {
-        state_sincos(t1_n, &sr, &cr);
+        state_sincos(t1_n, &s1_n, &c1_n);
         state_sincos(t1_n - t2_n, &sp_n, &cp_n);
       }
-      c1_n = fma(c0, cr, -(s0 * sr));
-      s1_n = fma(s0, cr, c0 * sr);
     };
     if constexpr (TPS > 1) state_part();
 
@@ -1073,7 +1161,7 @@ __device__ void run_tile(const KConst& k, const Inst& in, int tile, float* uh, c
       auto obstacle_row = [&](int j, T pam, T& al, T& u, T& w) {  // pam: p_alpha / m_alpha
         T h, Aa, Aw = 0.f, brest;
         if constexpr (!EXT) {
-          // staged as (cx, cy, Qxx, Qxy, Qyy): h = d^T Q d - 1 in world axes
+          // staged as (cx, cy, Qxx, Qxy, Qyy): h = d^T Q d - 1 in the frame
           const float4 o0 = *reinterpret_cast<const float4*>(S.obs + 8 * j);
           const T qxx = o0.z, qxy = o0.w, qyy = S.obs[8 * j + 4];
           const T dx = (px - T(o0.x)) + pxl, dy = (py - T(o0.y)) + pyl;
@@ -1763,7 +1851,7 @@ static __device__ void merge_instance(const KConst& k, const Inst& in, const Sme
   // rejects the solve
   int turn_bad = 0;
   for (int j = threadIdx.x; j + 1 < in.n_pts; j += blockDim.x)
-    turn_bad |= !(fabsf(S.path[3 * j + 5] - S.path[3 * j + 2]) <= kMaxPathTurn + 1e-4f);
+    turn_bad |= !(fabsf(S.path[4 * j + 6] - S.path[4 * j + 2]) <= kMaxPathTurn + 1e-4f);
   const bool turns_bad = __syncthreads_or(turn_bad);
   const float lsum = ustar[3 * H];
   const unsigned err = sh.err | (turns_bad ? ERR_PATH_TURN : 0u);
@@ -1821,8 +1909,9 @@ __device__ __forceinline__ void discard_history(const float* uh, int n_floats) {
 }
 
 // -------------------------------------------------------------- the kernel
-// Launch bound of the two-sample variants: three CTAs of 128 threads an SM
-constexpr int kMaxPairThreads = 128, kPairCtas = 3;
+// Launch bound of the two-sample variants: 384 threads an SM (168 registers),
+// in CTAs of up to 192
+constexpr int kMaxPairThreads = 192, kPairCtas = 2;
 // EXT: the instantiations that also carry the optional terms (moving and
 // e = 4 obstacles, collision cost, buffer cost); the others compile them out.
 template <int TPS, int BPT, bool EXT, int ROWS = 0, int NS = 1, bool LOCAL = false>
@@ -1909,7 +1998,7 @@ __global__ void __launch_bounds__(256) merge_tiles_kernel(const KConst k, const 
   cp_async_wait_all();
   __syncthreads();
   const Frame& fr = sh.fr;
-  shift_path(in, S, fr);  // as the tiles stage it
+  shift_path(in, S, fr, blockDim.x);  // as the tiles stage it
   __syncthreads();
   merge_instance<false>(k, in, S, sh);
 }
