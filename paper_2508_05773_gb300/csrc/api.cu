@@ -360,7 +360,7 @@ bool heuristic_plain(const brmppi_ctx* c, int n_obs, int n_pts, Shape* out) {
         const size_t smem = smem_bytes(make_caps(n_obs, rows, n_pts, c->prm.H, tps, bpt, ext), t / tps);
         return pair_residency(t / 2, smem) * t;
       };
-      threads = (bpt == 3 || tps == 1) && resident(384) > resident(256) ? 384 : 256;
+      threads = brmppi::pair_exists(tps, bpt, ext) && resident(384) > resident(256) ? 384 : 256;
     }
   }
   if (threads < tps) return false;
@@ -566,10 +566,17 @@ bool batch_shape_default(const brmppi_ctx* c, int max_P, Shape* out) {
   if (s.tps == 0 && s.threads == 0 && c->batch_tuned) {
     s = c->batch_shape;
   } else {
-    // the optional terms' rows carry a steer-rate column: teams wide enough
-    // for at most two Philox blocks per lane keep them out of local memory
-    const bool ext = brmppi::needs_ext(make_kconst(c->prm));
-    if (s.tps == 0) s.tps = ext ? ext_team_width(max_P) : 1;
+    // One lane a sample: the step's base is not repeated over a team, and the
+    // rows' state in shared memory leaves registers for any number of rows.
+    // With the optional terms only where the context's capacity (which fixes
+    // the width: a solve's bits must not depend on its batch) can fill the
+    // GPU: their step is long, and few solves finish sooner on wider teams.
+    // Measured on GB300, S = 4096, H = 50, 8 moving rows, one lane against two:
+    // 200 solves 2.53 / 4.06 ms, 8 solves 185 / 238 us, 4 solves 143 / 125 us,
+    // 1 solve 142 / 92 us; collision cost, 200 solves 1.00 / 2.15 ms.
+    const bool wide = brmppi::needs_ext(make_kconst(c->prm)) &&
+                      static_cast<long long>(c->prm.max_batch) * c->prm.S < 216LL * c->num_sms;
+    if (s.tps == 0) s.tps = wide ? ext_team_width(max_P) : 1;
     if (s.threads == 0) s.threads = std::max(128, kMinBatchSpb * s.tps);
   }
   while (!pick_bpt(s.tps, max_P, &s.bpt)) {

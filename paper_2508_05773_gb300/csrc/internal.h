@@ -152,8 +152,8 @@ bool pick_bpt(int tps, int P, int* bpt);
 // from the caps and return false (it goes to local memory).
 bool fit_rows(brmppi::SmemCaps* c, int spb, size_t smem_limit);
 int part_stride_for(int H);
-// Team width of batches and serving when the optional terms are on: at most
-// two Philox blocks per lane.
+// Team width of batches (of small contexts) and serving when the optional
+// terms are on.
 int ext_team_width(int P);
 brmppi_status check_sizes(brmppi_ctx* c, int32_t n_obs, int32_t n_pts, float ds);
 // Options of a single (non-batch) solve launch: the exact-rows variant, with

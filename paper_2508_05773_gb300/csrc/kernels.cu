@@ -22,6 +22,8 @@ void for_each_variant(F f) {
   for (int i = 0; i < n; ++i) f(g[i]);
   const Variant* p = variants_pair(&n);
   for (int i = 0; i < n; ++i) f(p[i]);
+  const Variant* q = variants_pair_ext(&n);
+  for (int i = 0; i < n; ++i) f(q[i]);
 }
 
 // rows = 0: the general instantiation of a shape; rows > 0: the one with

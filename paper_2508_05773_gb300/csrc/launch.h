@@ -29,6 +29,7 @@ const Variant* variants_wide_ext(int* n);
 const Variant* variants_latency(int* n);     // exact rows a lane, noise-warp shapes
 const Variant* variants_latency_ext(int* n); // the same with the optional terms (4 lanes)
 const Variant* variants_pair(int* n);        // two samples a team (throughput shapes)
+const Variant* variants_pair_ext(int* n);    // the same with the optional terms
 
 // Whether a launch with these constants needs the family with the optional terms.
 inline bool needs_ext(const KConst& k) { return k.coll || k.obs8 || k.abuf || k.discs || k.third || k.jerk; }

@@ -99,3 +99,37 @@ def test_unequal_contour_and_lag_weights(pkg, tps):
         assert_solve_matches(device_solve(s, c), ref, p, f"weights tps={tps}")
     finally:
         s.close()
+
+
+@pytest.mark.parametrize("flags", [sc.FLAG_OBS8, sc.FLAG_OBS8 | sc.FLAG_COLLISION_COST | sc.FLAG_ALPHA_BUFFER])
+def test_two_samples_a_lane_equal_one_with_optional_terms(pkg, flags):
+    """The same for the family with the optional terms (one lane a sample in
+    contexts whose capacity fills the GPU): 1, 3 and 11 moving rows."""
+    import torch
+    dev = torch.device("cuda:0")
+    base = sc.with_moving(sc.small_random(451, S=20 * 128 + 1, H=5, n_obs=11), 4)
+    base["params"] = dict(base["params"], flags=flags)
+    cases = [dict(base, obs=base["obs"][:n], seed=900 + n) for n in (1, 3, 11)]
+    n_fill = 14 * 152 // 21
+    s = pkg.Solver(base["params"], max_obstacles=11, max_path_pts=base["path"].shape[0], max_batch=n_fill + len(cases))
+    try:
+        assert s.batch_launch()["threads_per_sample"] == 1
+        mix = [_instance(c, dev) for c in cases]
+        fill = [dict(_instance(cases[1], dev), seed=7000 + i) for i in range(n_fill)]
+        s.solve_batch(mix + fill)
+        torch.cuda.synchronize()
+        for c, d in zip(cases, mix):
+            one = _instance(c, dev)
+            s.solve_batch([one])
+            torch.cuda.synchronize()
+            a, b = host_outputs(d), host_outputs(one)
+            for key in ("U", "traj", "J", "J_lo", "u_hist", "U_next"):
+                assert np.array_equal(a[key], b[key]), (len(c["obs"]), key)
+            p, ref = _oracle(c)
+            extra = None
+            if flags & sc.FLAG_ALPHA_BUFFER:
+                from tests.parity import buffer_conditioning
+                extra = buffer_conditioning(p, c)
+            assert_solve_matches(a, ref, p, f"packed optional terms n_obs={len(c['obs'])}", j_extra=extra)
+    finally:
+        s.close()
