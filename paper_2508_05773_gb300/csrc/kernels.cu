@@ -205,8 +205,17 @@ cudaError_t launch_solve(int tps, int bpt, int blocks, int threads, size_t smem,
   }
   LaunchDesc D = L;
   D.noise_warps = noise_warps(tps, bpt, threads, P, ns);
-  v->fn<<<blocks, block_threads(tps, bpt, threads, P, ns), smem, stream>>>(k, D);
-  return cudaGetLastError();
+  cudaLaunchAttribute early;
+  early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  early.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(static_cast<unsigned>(blocks));
+  cfg.blockDim = dim3(static_cast<unsigned>(block_threads(tps, bpt, threads, P, ns)));
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cfg.attrs = &early;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, v->fn, k, D);
 }
 
 }  // namespace brmppi
