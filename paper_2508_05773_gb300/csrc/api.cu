@@ -242,7 +242,7 @@ brmppi::KConst make_kconst(const brmppi_params& q) {
   return k;
 }
 
-brmppi::SmemCaps make_caps(int n_obs, int n_rows, int n_pts, int H, int tps, int bpt, bool ext) {
+brmppi::SmemCaps make_caps(int n_obs, int n_rows, int n_pts, int H, int tps, int bpt, int family) {
   brmppi::SmemCaps c{};
   c.obs = 8 * (n_obs + 1);  // and the null row
   c.path = 4 * n_pts;
@@ -250,7 +250,8 @@ brmppi::SmemCaps make_caps(int n_obs, int n_rows, int n_pts, int H, int tps, int
   c.ustar = brmppi::SmemCaps::pad4(3 * H + 1);
   c.noise_per_team = tps > 1 && bpt <= 2 ? 8 * philox_blocks(n_rows) : 0;
   // 4 rows a Philox block after the first, in passes of the team's lanes
-  c.rows_per_team = c.noise_per_team > 0 ? 0 : 4 * ((philox_blocks(n_rows) - 1 + tps - 1) / tps) * (ext ? 4 : 2) * tps;
+  c.rows_per_team = c.noise_per_team > 0 ? 0 : 4 * ((philox_blocks(n_rows) - 1 + tps - 1) / tps) *
+                                                         (family == brmppi::kDiscs || family == brmppi::kPoint ? 4 : 2) * tps;
   c.uh_per_team = 0;
   c.merge = 0;
   return c;
@@ -290,10 +291,10 @@ long long pair_residency(int threads, size_t smem) {
   return std::min<long long>(brmppi::kMaxPairBlockThreads * brmppi::kPairCtas / threads, 227 * 1024 / (smem + 2048));
 }
 
-int samples_per_team(const Shape& sh, bool ext, long long tiles, size_t smem, int num_sms) {
+int samples_per_team(const Shape& sh, int family, long long tiles, size_t smem, int num_sms) {
   const int threads = sh.threads / 2;
   if (sh.threads % 64 != 0 || threads < 64 || threads > brmppi::kMaxPairBlockThreads ||
-      !brmppi::pair_exists(sh.tps, sh.bpt, ext))
+      !brmppi::pair_exists(sh.tps, sh.bpt, family))
     return 1;
   return tiles >= pair_residency(threads, smem) * num_sms ? 2 : 1;
 }
@@ -328,7 +329,8 @@ bool heuristic_plain(const brmppi_ctx* c, int n_obs, int n_pts, Shape* out) {
   const int P = philox_blocks(rows);
   const long long S = c->prm.S, sms = c->num_sms;
   const bool fixed_tps = c->prm.threads_per_sample != 0;
-  const bool ext = brmppi::needs_ext(make_kconst(c->prm));
+  const int family = brmppi::family_of(make_kconst(c->prm));
+  const bool ext = family == brmppi::kDiscs || family == brmppi::kPoint;
   int tps = c->prm.threads_per_sample;
   if (!fixed_tps) {
     tps = 2;
@@ -357,14 +359,14 @@ bool heuristic_plain(const brmppi_ctx* c, int n_obs, int n_pts, Shape* out) {
       // 256, or 384 (more samples share the CTA's tables) where that keeps
       // more samples on an SM
       auto resident = [&](int t) {
-        const size_t smem = smem_bytes(make_caps(n_obs, rows, n_pts, c->prm.H, tps, bpt, ext), t / tps);
+        const size_t smem = smem_bytes(make_caps(n_obs, rows, n_pts, c->prm.H, tps, bpt, family), t / tps);
         return pair_residency(t / 2, smem) * t;
       };
-      threads = brmppi::pair_exists(tps, bpt, ext) && resident(384) > resident(256) ? 384 : 256;
+      threads = brmppi::pair_exists(tps, bpt, family) && resident(384) > resident(256) ? 384 : 256;
     }
   }
   if (threads < tps) return false;
-  while (table_bytes(make_caps(n_obs, rows_of(c->prm, n_obs), n_pts, c->prm.H, tps, bpt, ext), threads / tps) >
+  while (table_bytes(make_caps(n_obs, rows_of(c->prm, n_obs), n_pts, c->prm.H, tps, bpt, family), threads / tps) >
          c->smem_limit) {
     if (!fixed_threads && threads > kMinThreads) {
       threads -= 32;
@@ -386,7 +388,7 @@ bool plain_shape(const brmppi_ctx* c, int n_obs, int n_pts, Shape* out) {
     auto it = c->tuned.find(n_obs);
     if (it != c->tuned.end()) {
       const brmppi::SmemCaps caps = make_caps(n_obs, rows_of(c->prm, n_obs), n_pts, c->prm.H, it->second.tps,
-                                              it->second.bpt, brmppi::needs_ext(make_kconst(c->prm)));
+                                              it->second.bpt, brmppi::family_of(make_kconst(c->prm)));
       if (table_bytes(caps, it->second.threads / it->second.tps) <= c->smem_limit) {
         *out = it->second;
         return true;
@@ -479,8 +481,8 @@ brmppi_status enqueue_plain_sized(brmppi_ctx* c, const Shape& sh, int S, int H, 
     L.single.no_merge = 1;
   }
   const brmppi::KConst k = make_kconst(c->prm);
-  const bool ext = brmppi::needs_ext(k);
-  L.caps = make_caps(n_obs, rows_of(c->prm, n_obs), n_pts, H, sh.tps, sh.bpt, ext);
+  const int family = brmppi::family_of(k);
+  L.caps = make_caps(n_obs, rows_of(c->prm, n_obs), n_pts, H, sh.tps, sh.bpt, family);
   brmppi::LaunchMode mode;
   mode.local = !fit_rows(&L.caps, spb, c->smem_limit);
   L.uh = c->d_uh;
@@ -492,7 +494,7 @@ brmppi_status enqueue_plain_sized(brmppi_ctx* c, const Shape& sh, int S, int H, 
   if ((!tiles_out && static_cast<size_t>(tiles) > c->part_tiles) ||
       static_cast<size_t>(tiles) * static_cast<size_t>(L.uh_stride) > c->uh_floats)
     return fail(c, BRMPPI_EINVAL, "launch shape exceeds the context's scratch");
-  if (L.rows == 0 && !mode.local) mode.ns = samples_per_team(sh, ext, tiles, smem, c->num_sms);
+  if (L.rows == 0 && !mode.local) mode.ns = samples_per_team(sh, family, tiles, smem, c->num_sms);
   cudaError_t e = brmppi::launch_solve(sh.tps, sh.bpt, tiles, sh.threads, smem, stream, k, L, L.single.P, mode);
   if (e != cudaSuccess) return cuda_fail(c, e, "kernel launch");
   if (u_safe) {
@@ -571,11 +573,12 @@ bool batch_shape_default(const brmppi_ctx* c, int max_P, Shape* out) {
     // With the optional terms only where the context's capacity (which fixes
     // the width: a solve's bits must not depend on its batch) can fill the
     // GPU: their step is long, and few solves finish sooner on wider teams.
-    // Measured on GB300, S = 4096, H = 50, 8 moving rows, one lane against two:
-    // 200 solves 2.53 / 4.06 ms, 8 solves 185 / 238 us, 4 solves 143 / 125 us,
-    // 1 solve 142 / 92 us; collision cost, 200 solves 1.00 / 2.15 ms.
-    const bool wide = brmppi::needs_ext(make_kconst(c->prm)) &&
-                      static_cast<long long>(c->prm.max_batch) * c->prm.S < 216LL * c->num_sms;
+    // Measured on GB300, S = 4096, H = 50, 8 moving rows, one lane against two
+    // (every optional term compiled in): 200 solves 2.53 / 4.06 ms, 8 solves
+    // 185 / 238 us, 4 solves 143 / 125 us, 1 solve 142 / 92 us; collision cost,
+    // 200 solves 1.00 / 2.15 ms.
+    const bool wide = brmppi::family_of(make_kconst(c->prm)) != brmppi::kPlain &&
+                      static_cast<long long>(c->prm.max_batch) * c->prm.S < 200LL * c->num_sms;
     if (s.tps == 0) s.tps = wide ? ext_team_width(max_P) : 1;
     if (s.threads == 0) s.threads = std::max(128, kMinBatchSpb * s.tps);
   }
@@ -640,8 +643,8 @@ brmppi_status plan_batch(brmppi_ctx* c, Lane& L, const brmppi_instance* inst, in
     return fail(c, BRMPPI_EINVAL, "no batch launch shape for these instances");
   }
   const int spb = sh.threads / sh.tps;
-  const bool ext = brmppi::needs_ext(make_kconst(c->prm));
-  brmppi::SmemCaps caps = make_caps(nobs_max, rows_of(c->prm, nobs_max), npts_max, Hmax, sh.tps, sh.bpt, ext);
+  const int family = brmppi::family_of(make_kconst(c->prm));
+  brmppi::SmemCaps caps = make_caps(nobs_max, rows_of(c->prm, nobs_max), npts_max, Hmax, sh.tps, sh.bpt, family);
   brmppi::LaunchMode mode;
   mode.local = !fit_rows(&caps, spb, c->smem_limit);
   const size_t smem = smem_bytes(caps, spb);
@@ -673,8 +676,8 @@ brmppi_status plan_batch(brmppi_ctx* c, Lane& L, const brmppi_instance* inst, in
                      return a.first > b.first;
                    });
   for (size_t j = 0; j < items.size(); ++j) h_work[j] = items[j].second;
-  if (!mode.local) mode.ns = samples_per_team(sh, ext, static_cast<long long>(items.size()), smem, c->num_sms);
-  const int occ = brmppi::variant_occupancy(sh.tps, sh.bpt, sh.threads, smem, ext, P_cap, mode);
+  if (!mode.local) mode.ns = samples_per_team(sh, family, static_cast<long long>(items.size()), smem, c->num_sms);
+  const int occ = brmppi::variant_occupancy(sh.tps, sh.bpt, sh.threads, smem, family, P_cap, mode);
   if (occ < 1) return fail(c, BRMPPI_EINVAL, "batch launch shape cannot be resident");
   int grid = occ * c->num_sms;
   if (grid > static_cast<int>(items.size())) grid = static_cast<int>(items.size());
@@ -1017,7 +1020,7 @@ brmppi_status brmppi_merge_tiles(brmppi_ctx* c, const brmppi_instance* q, const 
                               q->counter, q->U_out, q->traj_out, q->J_out, q->U_next, q->status,
                               const_cast<float*>(tiles), c->d_sync, spb, c->prm.n_discs);
   const brmppi::SmemCaps caps = make_caps(q->n_obs, rows_of(c->prm, q->n_obs), q->n_pts, q->H, sh.tps, sh.bpt,
-                                          brmppi::needs_ext(make_kconst(c->prm)));
+                                          brmppi::family_of(make_kconst(c->prm)));
   const size_t smem = table_bytes(caps, 1);
   if (smem > c->smem_limit) return fail(c, BRMPPI_EINVAL, "shared memory need exceeds the device limit");
   const cudaError_t e = brmppi::launch_merge_tiles(make_kconst(c->prm), in, caps, smem, static_cast<cudaStream_t>(stream));
@@ -1130,7 +1133,7 @@ brmppi_status brmppi_autotune(brmppi_ctx* c, const double* x0, const float* U_no
     int bpt;
     if (!pick_bpt(tps, P, &bpt)) continue;
     const brmppi::SmemCaps caps = make_caps(n_obs, rows_of(c->prm, n_obs), n_pts, H, tps, bpt,
-                                            brmppi::needs_ext(make_kconst(c->prm)));
+                                            brmppi::family_of(make_kconst(c->prm)));
     for (int threads : {64, 128, 256}) {
       if (threads < tps || threads / tps < 2) continue;
       const int spb = threads / tps;

@@ -46,7 +46,7 @@ struct Shape {
 
 // Samples a team of a launch rolls out together (2: the packed-pair
 // instantiations) for `tiles` tiles of a shape with `smem` bytes a CTA.
-int samples_per_team(const Shape& sh, bool ext, long long tiles, size_t smem, int num_sms);
+int samples_per_team(const Shape& sh, int family, long long tiles, size_t smem, int num_sms);
 
 // Everything one in-flight batch launch needs: instance table, work list,
 // per-tile partial pool, per-instance counters, per-CTA input history, host

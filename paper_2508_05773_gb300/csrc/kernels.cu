@@ -7,31 +7,25 @@ namespace {
 
 template <typename F>
 void for_each_variant(F f) {
-  int n = 0;
-  const Variant* a = variants_narrow(&n);
-  for (int i = 0; i < n; ++i) f(a[i]);
-  const Variant* b = variants_wide(&n);
-  for (int i = 0; i < n; ++i) f(b[i]);
-  const Variant* c = variants_narrow_ext(&n);
-  for (int i = 0; i < n; ++i) f(c[i]);
-  const Variant* d = variants_wide_ext(&n);
-  for (int i = 0; i < n; ++i) f(d[i]);
-  const Variant* e = variants_latency(&n);
-  for (int i = 0; i < n; ++i) f(e[i]);
-  const Variant* g = variants_latency_ext(&n);
-  for (int i = 0; i < n; ++i) f(g[i]);
-  const Variant* p = variants_pair(&n);
-  for (int i = 0; i < n; ++i) f(p[i]);
-  const Variant* q = variants_pair_ext(&n);
-  for (int i = 0; i < n; ++i) f(q[i]);
+  using Table = const Variant* (*)(int*);
+  static const Table tables[] = {
+      variants_narrow_plain,   variants_narrow_discs,   variants_narrow_point,  variants_narrow_moving,
+      variants_wide_plain,     variants_wide_discs,     variants_wide_point,    variants_wide_moving,
+      variants_latency_plain,  variants_latency_discs,  variants_latency_point, variants_latency_moving,
+  };
+  for (const Table t : tables) {
+    int n = 0;
+    const Variant* v = t(&n);
+    for (int i = 0; i < n; ++i) f(v[i]);
+  }
 }
 
 // rows = 0: the general instantiation of a shape; rows > 0: the one with
 // exactly that many constraint rows a lane (null if not compiled)
-const Variant* find(int tps, int bpt, bool ext, int rows = 0, LaunchMode mode = LaunchMode()) {
+const Variant* find(int tps, int bpt, int family, int rows = 0, LaunchMode mode = LaunchMode()) {
   const Variant* hit = nullptr;
   for_each_variant([&](const Variant& v) {
-    if (v.tps == tps && v.bpt == bpt && v.ext == ext && v.rows == rows && v.ns == mode.ns &&
+    if (v.tps == tps && v.bpt == bpt && v.family == family && v.rows == rows && v.ns == mode.ns &&
         v.local == mode.local)
       hit = &v;
   });
@@ -110,7 +104,7 @@ cudaError_t launch_noise_blocks(uint64_t seed, uint64_t counter, int n_samples, 
 
 cudaError_t launch_merge_tiles(const KConst& k, const Inst& in, const SmemCaps& caps, size_t smem,
                                cudaStream_t stream) {
-  if (needs_ext(k)) {
+  if (family_of(k) != kPlain) {
     cudaError_t e = cudaFuncSetAttribute(reinterpret_cast<const void*>(&merge_tiles_kernel<true>),
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (e != cudaSuccess) return e;
@@ -138,9 +132,9 @@ cudaError_t launch_stabilize(const KConst& k, const double* x, const float* u_re
   return cudaGetLastError();
 }
 
-bool pair_exists(int tps, int bpt, bool ext) { return find(tps, bpt, ext, 0, LaunchMode{2, false}) != nullptr; }
+bool pair_exists(int tps, int bpt, int family) { return find(tps, bpt, family, 0, LaunchMode{2, false}) != nullptr; }
 
-bool variant_exists(int tps, int bpt) { return find(tps, bpt, false) != nullptr && find(tps, bpt, true) != nullptr; }
+bool variant_exists(int tps, int bpt) { return find(tps, bpt, kPlain) != nullptr; }
 
 cudaError_t set_smem_limit(size_t bytes) {
   cudaError_t err = cudaSuccess;
@@ -174,12 +168,12 @@ int block_threads(int tps, int bpt, int threads, int P, int ns) {
 int exact_rows_variant(int tps, int bpt, const KConst& k, int n_rows) {
   if (tps <= 1 || bpt > 2 || n_rows <= 0) return 0;
   const int rows = (n_rows + tps - 1) / tps;
-  return find(tps, 1, needs_ext(k), rows) ? rows : 0;
+  return find(tps, 1, family_of(k), rows) ? rows : 0;
 }
 
-int variant_occupancy(int tps, int bpt, int threads, size_t smem, bool ext, int P, LaunchMode mode) {
+int variant_occupancy(int tps, int bpt, int threads, size_t smem, int family, int P, LaunchMode mode) {
   const int ns = mode.ns;
-  const Variant* v = find(tps, bpt, ext, 0, mode);
+  const Variant* v = find(tps, bpt, family, 0, mode);
   if (!v || block_threads(tps, bpt, threads, P, ns) > (ns > 1 ? kMaxPairBlockThreads : kMaxBlockThreads)) return 0;
   int n = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, v->fn, block_threads(tps, bpt, threads, P, ns), smem) !=
@@ -191,7 +185,7 @@ int variant_occupancy(int tps, int bpt, int threads, size_t smem, bool ext, int 
 cudaError_t launch_solve(int tps, int bpt, int blocks, int threads, size_t smem, cudaStream_t stream,
                          const KConst& k, const LaunchDesc& L, int P, LaunchMode mode) {
   const int ns = mode.ns;
-  const Variant* v = find(tps, bpt, needs_ext(k), 0, mode);
+  const Variant* v = find(tps, bpt, family_of(k), 0, mode);
   if (!v || block_threads(tps, bpt, threads, P, ns) > (ns > 1 ? kMaxPairBlockThreads : kMaxBlockThreads))
     return cudaErrorInvalidValue;
   if (L.rows > 0) {
@@ -200,7 +194,7 @@ cudaError_t launch_solve(int tps, int bpt, int blocks, int threads, size_t smem,
     v = (L.work || (!L.single.no_merge && L.caps.merge < L.single.tiles * L.single.part_stride) ||
          L.caps.uh_per_team < 3 * L.single.H)
             ? nullptr
-            : find(tps, 1, needs_ext(k), L.rows);
+            : find(tps, 1, family_of(k), L.rows);
     if (!v) return cudaErrorInvalidValue;
   }
   LaunchDesc D = L;

@@ -11,28 +11,33 @@ using KernelFn = void (*)(const KConst, const LaunchDesc);
 
 struct Variant {
   int tps, bpt;
-  bool ext;  // carries the optional terms (BRMPPI_FLAG_COLLISION_COST, _OBS8, _ALPHA_BUFFER,
-             // footprint discs other than the rear-axle point)
+  int family;  // Family
   KernelFn fn;
   int rows = 0;  // > 0: exactly this many constraint rows a lane (single solves)
   int ns = 1;    // samples a team rolls out together
   bool local = false;  // rows' state in local memory
 };
 
-// Instantiations, one translation unit per group of team widths and family
-// (compiled in parallel); each returns its table and its length.  Both
-// families hold the same (tps, bpt) pairs.
-const Variant* variants_narrow(int* n);      // 1 and 2 lanes per sample
-const Variant* variants_wide(int* n);        // 4 .. 32 lanes per sample
-const Variant* variants_narrow_ext(int* n);  // the same, with the optional terms
-const Variant* variants_wide_ext(int* n);
-const Variant* variants_latency(int* n);     // exact rows a lane, noise-warp shapes
-const Variant* variants_latency_ext(int* n); // the same with the optional terms (4 lanes)
-const Variant* variants_pair(int* n);        // two samples a team (throughput shapes)
-const Variant* variants_pair_ext(int* n);    // the same with the optional terms
+// Instantiations (variants.h): each function returns its table and its length.
+const Variant* variants_narrow_plain(int* n);
+const Variant* variants_narrow_discs(int* n);
+const Variant* variants_narrow_point(int* n);
+const Variant* variants_narrow_moving(int* n);
+const Variant* variants_wide_plain(int* n);
+const Variant* variants_wide_discs(int* n);
+const Variant* variants_wide_point(int* n);
+const Variant* variants_wide_moving(int* n);
+const Variant* variants_latency_plain(int* n);
+const Variant* variants_latency_discs(int* n);
+const Variant* variants_latency_point(int* n);
+const Variant* variants_latency_moving(int* n);
 
-// Whether a launch with these constants needs the family with the optional terms.
-inline bool needs_ext(const KConst& k) { return k.coll || k.obs8 || k.abuf || k.discs || k.third || k.jerk; }
+// The family a launch with these constants takes.
+inline int family_of(const KConst& k) {
+  if (k.discs) return kDiscs;
+  if (k.third || k.jerk || k.abuf) return kPoint;
+  return k.obs8 || k.coll ? kMoving : kPlain;
+}
 
 // Threads of a launch shape.  `threads` / tps is the samples of a CTA's tile;
 // with ns samples a team threads / ns of them roll out.  Teams of one sample
@@ -61,13 +66,13 @@ int exact_rows_variant(int tps, int bpt, const KConst& k, int n_rows);
 // Supported (threads per sample, Philox blocks per lane) pairs.
 bool variant_exists(int tps, int bpt);
 // Whether a pair is compiled with two samples a team.
-bool pair_exists(int tps, int bpt, bool ext);
+bool pair_exists(int tps, int bpt, int family);
 
 // Raise the dynamic shared-memory limit of every variant to `bytes`.
 cudaError_t set_smem_limit(size_t bytes);
 
 // CTAs of a variant resident per SM for a launch shape (0 if it cannot run).
-int variant_occupancy(int tps, int bpt, int threads, size_t smem, bool ext, int P, LaunchMode mode);
+int variant_occupancy(int tps, int bpt, int threads, size_t smem, int family, int P, LaunchMode mode);
 
 // Enqueue the hitch stabilizer for n states (out: n x 4 floats).
 cudaError_t launch_stabilize(const KConst& k, const double* x, const float* u_ref, int n, float* out,

@@ -25,7 +25,7 @@ namespace brmppi_host {
 // defined in api.cu
 std::string check_params(const brmppi_params* p);
 brmppi::KConst make_kconst(const brmppi_params& q);
-brmppi::SmemCaps make_caps(int n_obs, int n_rows, int n_pts, int H, int tps, int bpt, bool ext);
+brmppi::SmemCaps make_caps(int n_obs, int n_rows, int n_pts, int H, int tps, int bpt, int family);
 size_t smem_bytes(const brmppi::SmemCaps& c, int spb);
 brmppi::Inst make_inst(const double* x0, const float* U_nom, const float* obs, int n_obs, const float* path,
                        int n_pts, float ds, int S, int H, uint64_t seed, uint64_t counter, float* U_out,
@@ -127,7 +127,7 @@ extern "C" brmppi_status brmppi_solve_device_noalloc(const brmppi_params* p, con
   L.single = make_inst(x0_dev, U_nom_dev, obs_dev, n_obs, path_dev, n_pts, ds, p->S, p->H, seed, counter, U_out_dev,
                        traj_out_dev, J_out_dev, U_next_dev, status_dev, part, sync, kNaSpb, p->n_discs);
   const brmppi::KConst k = make_kconst(*p);
-  L.caps = make_caps(n_obs, n_rows, n_pts, p->H, kNaTps, bpt, brmppi::needs_ext(k));
+  L.caps = make_caps(n_obs, n_rows, n_pts, p->H, kNaTps, bpt, brmppi::family_of(k));
   brmppi::LaunchMode mode;
   mode.local = !fit_rows(&L.caps, kNaSpb, smem_optin);
   L.uh = part + kNaPartFloats;

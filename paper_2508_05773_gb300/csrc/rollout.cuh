@@ -546,24 +546,24 @@ __device__ __forceinline__ PhiloxBlock load_block(const Smem& S, int b) {
 __device__ __forceinline__ void step_barrier() { asm volatile("bar.sync 1, %0;" ::"r"(blockDim.x) : "memory"); }
 
 // A row's state between steps (variants without producer warps): its rate
-// less the part in y, and its columns u and (EXT) w.
-template <bool EXT, int NS>
-constexpr int kRowFloats = EXT ? 4 * NS : 2 * NS;
+// less the part in y, and its columns u and (W) w.
+template <bool W, int NS>
+constexpr int kRowFloats = W ? 4 * NS : 2 * NS;
 constexpr int kMaxRowSlots = 32;  // a lane's rows: 4 per Philox block, at most 8 blocks
-template <bool EXT, int NS>
+template <bool W, int NS>
 __device__ __forceinline__ void store_row(float* p, Vec<NS> al, Vec<NS> u, Vec<NS> w) {
   if constexpr (NS == 1) {
-    if constexpr (EXT) *reinterpret_cast<float4*>(p) = make_float4(al.x, u.x, w.x, 0.f);
+    if constexpr (W) *reinterpret_cast<float4*>(p) = make_float4(al.x, u.x, w.x, 0.f);
     else *reinterpret_cast<float2*>(p) = make_float2(al.x, u.x);
   } else {
     *reinterpret_cast<float4*>(p) = make_float4(al.x.x, al.x.y, u.x.x, u.x.y);
-    if constexpr (EXT) *reinterpret_cast<float2*>(p + 4) = w.x;
+    if constexpr (W) *reinterpret_cast<float2*>(p + 4) = w.x;
   }
 }
-template <bool EXT, int NS>
+template <bool W, int NS>
 __device__ __forceinline__ void load_row(const float* p, Vec<NS>& al, Vec<NS>& u, Vec<NS>& w) {
   if constexpr (NS == 1) {
-    if constexpr (EXT) {
+    if constexpr (W) {
       const float4 v = *reinterpret_cast<const float4*>(p);
       al = v.x;
       u = v.y;
@@ -577,7 +577,7 @@ __device__ __forceinline__ void load_row(const float* p, Vec<NS>& al, Vec<NS>& u
     const float4 v = *reinterpret_cast<const float4*>(p);
     al = Vec<NS>(make_float2(v.x, v.y));
     u = Vec<NS>(make_float2(v.z, v.w));
-    if constexpr (EXT) w = Vec<NS>(*reinterpret_cast<const float2*>(p + 4));
+    if constexpr (W) w = Vec<NS>(*reinterpret_cast<const float2*>(p + 4));
   }
 }
 
@@ -597,13 +597,27 @@ __device__ __forceinline__ Vec<N> sampled_rate(const KConst& k, Vec<N> n) {
   return vclamp(fma(Vec<N>(k.ps), n, Vec<N>(k.pc_am)), k.pam_lo, k.pam_hi);
 }
 
+// Families of instantiations, by the terms they compile in.  A term that a
+// step does not have costs it: its uniform branch splits the step into separately
+// scheduled parts, its operands hold registers, its code fills the
+// instruction cache.
+//   kPlain   parked ellipses;
+//   kDiscs   every optional term: any footprint, and all below;
+//   kPoint   the rear-axle disc only: third-order rows, jerk-input model, buffer
+//            cost, and all below;
+//   kMoving  moving and e = 4 obstacles, collision cost.
+// S = 4096, H = 50, 8 moving rows: 49.7 / 35.0 us on kDiscs / kMoving; third
+// order and jerk, S = 3001, H = 61, 61.5 / 50.7 us on kDiscs / kPoint.
+enum Family : int { kPlain = 0, kDiscs = 1, kPoint = 2, kMoving = 3 };
+
 // ----------------------------------------------------------- one sample tile
 // NS: samples a team rolls out together (Vec<NS>).
 // LOCAL: the rows' state in local memory (in place of shared memory).
-template <int TPS, int BPT, bool EXT, int ROWS, int NS, bool LOCAL>
+template <int TPS, int BPT, int EXT, int ROWS, int NS, bool LOCAL>
 __device__ void run_tile(const KConst& k, const Inst& in, int tile, float* uh, const Smem& S,
                          Shared& sh, int noise_warps) {
   using T = Vec<NS>;
+  constexpr bool DISCS = EXT == kDiscs, TERMS = EXT == kDiscs || EXT == kPoint;
   // Teams wider than one lane run with extra warps (the last ones) that
   // produce every team's normals a step ahead (warp specialisation: the
   // noise leaves the compute warps' dependency chain).
@@ -615,7 +629,7 @@ __device__ void run_tile(const KConst& k, const Inst& in, int tile, float* uh, c
   const int lt = threadIdx.x % TPS;
   const int s = tile * spb + team * NS;  // the team's first sample
   const int H = in.H;
-  const int n_rows = EXT ? in.n_obs * k.nd : in.n_obs;  // obstacle rows (obstacle x disc)
+  const int n_rows = DISCS ? in.n_obs * k.nd : in.n_obs;  // obstacle rows (obstacle x disc)
 
   if (threadIdx.x == 32) {  // warm the outputs' translations (any CTA may merge)
     prefetch_l2(in.U_out);
@@ -641,7 +655,7 @@ __device__ void run_tile(const KConst& k, const Inst& in, int tile, float* uh, c
   float ob0[8];
 #pragma unroll
   for (int q = 0; q < 8; ++q) ob0[q] = (has_ob0 && q < ostride) ? in.obs[ostride * o0_ + q] : 0.f;
-  if (threadIdx.x < 32) make_frame_warp(in.x0, in.inv_ds_d, in.sync + 1, sh.fr, EXT && k.jerk);
+  if (threadIdx.x < 32) make_frame_warp(in.x0, in.inv_ds_d, in.sync + 1, sh.fr, TERMS && k.jerk);
   float sin0 = 0.f, cos0 = 0.f;
   if (has_ob0) sincosf(ob0[4], &sin0, &cos0);
   cp_async_wait_all();
@@ -768,7 +782,7 @@ __device__ void run_tile(const KConst& k, const Inst& in, int tile, float* uh, c
     }
     shift_path(in, S, fr, n_stage);
     if constexpr (!PRODUCED) map_inputs(threadIdx.x, blockDim.x);
-    if constexpr (EXT) {
+    if constexpr (DISCS) {
 #pragma unroll
       for (int m = 0; m < 8; ++m)
         if (static_cast<int>(threadIdx.x) == m) {
@@ -798,11 +812,11 @@ __device__ void run_tile(const KConst& k, const Inst& in, int tile, float* uh, c
   // a lane the step was 50 KB of code and waited for instructions (stall 0.8
   // an issue), and 64 registers more a lane cost a third of the warps.
   float local_rows[LOCAL ? 4 * kMaxRowSlots * NS : 1];
-  const int row_stride = LOCAL ? kRowFloats<EXT, NS> : kRowFloats<EXT, NS> * static_cast<int>(blockDim.x);
-  float* rows = LOCAL ? local_rows : S.noise + kRowFloats<EXT, NS> * static_cast<int>(threadIdx.x);
+  const int row_stride = LOCAL ? kRowFloats<TERMS, NS> : kRowFloats<TERMS, NS> * static_cast<int>(blockDim.x);
+  float* rows = LOCAL ? local_rows : S.noise + kRowFloats<TERMS, NS> * static_cast<int>(threadIdx.x);
   const int passes = (in.P - 1 + TPS - 1) / TPS;  // Philox blocks 1 .. P - 1 over the team's lanes
   if constexpr (!PRODUCED)
-    for (int q = 0; q < 4 * passes; ++q) store_row<EXT, NS>(rows + q * row_stride, T(k.alpha0), T(0.f), T(0.f));
+    for (int q = 0; q < 4 * passes; ++q) store_row<TERMS, NS>(rows + q * row_stride, T(k.alpha0), T(0.f), T(0.f));
   T ya_p = 0.f, yw_p = 0.f;  // the step before's y
   T Jh = 0.f, Jl = 0.f;
   T ua = 0.f, uw = 0.f, un = 0.f;  // applied input of the previous step
@@ -843,13 +857,20 @@ __device__ void run_tile(const KConst& k, const Inst& in, int tile, float* uh, c
   // the current state and time t (Eq. barrier_function; moving centres at
   // c + t v); (ce1, se1) and (ce2, se2) the unit headings of the state
   auto row_h = [&](int j, float t, T ce1, T se1, T ce2, T se2) -> T {
-    const int o = (k.nd == 1) ? j : __float2int_rz((static_cast<float>(j) + 0.5f) * k.inv_nd);
-    const int m = j - o * k.nd;
+    int o = j;
+    T dx, dy;
+    if constexpr (DISCS) {
+      o = (k.nd == 1) ? j : __float2int_rz((static_cast<float>(j) + 0.5f) * k.inv_nd);
+    }
     const float4 o0 = *reinterpret_cast<const float4*>(S.obs + 8 * o);
     const float4 o1 = *reinterpret_cast<const float4*>(S.obs + 8 * o + 4);
-    const float2 lv = *reinterpret_cast<const float2*>(S.disc + 2 * m);
-    const T dx = fma(T(lv.y), ce2, fma(T(lv.x), ce1, (px - T(o0.x)) + pxl));
-    const T dy = fma(T(lv.y), se2, fma(T(lv.x), se1, (py - T(o0.y)) + pyl));
+    dx = (px - T(o0.x)) + pxl;
+    dy = (py - T(o0.y)) + pyl;
+    if constexpr (DISCS) {
+      const float2 lv = *reinterpret_cast<const float2*>(S.disc + 2 * (j - o * k.nd));
+      dx = fma(T(lv.y), ce2, fma(T(lv.x), ce1, dx));
+      dy = fma(T(lv.y), se2, fma(T(lv.x), se1, dy));
+    }
     const T xp = fma(T(o0.z), dx, fma(T(o0.w), dy, T(-t * o1.z)));
     const T yp = fma(T(o0.z), dy, fma(T(-o0.w), dx, T(-t * o1.w)));
     const bool e4 = o1.x < 0.f;
@@ -1050,7 +1071,7 @@ __device__ void run_tile(const KConst& k, const Inst& in, int tile, float* uh, c
 
     // cost of the previous step, at this state (independent of the rows)
     T c2 = 0.f, s2 = 0.f;  // the trailer's heading, where a term needs it
-    if (EXT && k.discs) {
+    if (DISCS && k.discs) {
       c2 = fma(c1, cp, s1 * sp);
       s2 = fma(s1, cp, -(c1 * sp));
     }
@@ -1117,7 +1138,7 @@ __device__ void run_tile(const KConst& k, const Inst& in, int tile, float* uh, c
         T Aa = fma(-sgT, fma(G, T(k.inv_l2), -tl), T(-k.Ts * k.kappa));
         const T Aw = (sgT * vv) * (sec2 * kcl);
         T c = phidot * fma(-(sgT * vl2), bend, sgTs);
-        if (EXT && k.jerk) {  // a is a state: its terms join the constant; the jerk enters via -kappa
+        if (TERMS && k.jerk) {  // a is a state: its terms join the constant; the jerk enters via -kappa
           c = fma(acc, Aa, c);
           Aa = T(-k.hTs2 * k.kappa);
         }
@@ -1138,7 +1159,7 @@ __device__ void run_tile(const KConst& k, const Inst& in, int tile, float* uh, c
       // row (j = n_rows).
       T Saa = 0.f, ga = 0.f, Saw = 0.f, Sww = 0.f, gw = 0.f;
       T ca[OBS_SLOTS];
-      T cw[EXT ? OBS_SLOTS : 1];  // steer-rate column (footprint discs off the rear axle)
+      T cw[TERMS ? OBS_SLOTS : 1];  // steer-rate column (footprint discs off the rear axle)
       // every slot that the alpha update reads is written below (padding
       // rows as zeros)
       const float tnow = static_cast<float>(tau) * k.Ts;
@@ -1146,7 +1167,7 @@ __device__ void run_tile(const KConst& k, const Inst& in, int tile, float* uh, c
       // heading accelerations of the bodies with the input held (footprint
       // discs): th1ddot = a1a a + a1w omega, th2ddot = a20 + a2a a + a2w omega
       T a1w = 0.f, a20 = 0.f, a2a = 0.f, a2w = 0.f;
-      if (EXT && k.discs) {
+      if (DISCS && k.discs) {
         a1w = vv * sec2 * T(k.inv_l1);
         a2a = G * T(k.inv_l2);
         a2w = -(vv * T(k.khl2) * cp * sec2);
@@ -1174,24 +1195,32 @@ __device__ void run_tile(const KConst& k, const Inst& in, int tile, float* uh, c
           Aa = fma(gx, ax_row, gy * ay_row);
           brest = fma(gx, bx_row, fma(gy, by_row, fma(qxx_row, qxx, fma(qxy_row, qxy, qyy_row * qyy))));
         } else {
-          // row j: obstacle o seen from footprint disc m (obstacle-major)
-          const int o = (k.nd == 1) ? j : __float2int_rz((static_cast<float>(j) + 0.5f) * k.inv_nd);
-          const int m = j - o * k.nd;
+          // row j: obstacle o, seen from the rear axle or (kDiscs) from
+          // footprint disc m (obstacle-major).  Unit headings in the obstacle
+          // frame: e1' = (dirx, diry), n1' = (-diry, dirx), e2' = (d2x, d2y),
+          // n2' = (-d2y, d2x); e = 4 flagged by a negated kx; with
+          // X = xp^(e-2) / Ax^e: h = xp^2 X + ..., h_x = e xp X,
+          // h_xx = e (e-1) X
+          int o = j;
+          if constexpr (DISCS) o = (k.nd == 1) ? j : __float2int_rz((static_cast<float>(j) + 0.5f) * k.inv_nd);
           const float4 o0 = *reinterpret_cast<const float4*>(S.obs + 8 * o);
           const float4 o1 = *reinterpret_cast<const float4*>(S.obs + 8 * o + 4);
-          const float2 lvp = *reinterpret_cast<const float2*>(S.disc + 2 * m);  // lever arms on e1, e2
-          const T lx = lvp.x, ly = lvp.y;
           const T co = o0.z, so = o0.w;
-          // unit headings in the obstacle frame: e1' = (dirx, diry),
-          // n1' = (-diry, dirx), e2' = (d2x, d2y), n2' = (-d2y, d2x)
           const T dirx = fma(co, c1, so * s1), diry = fma(co, s1, -(so * c1));
-          const T d2x = fma(co, c2, so * s2), d2y = fma(co, s2, -(so * c2));
           const T dx = (px - T(o0.x)) + pxl, dy = (py - T(o0.y)) + pyl;
-          // disc centre relative to the (moving) obstacle centre at tnow;
-          // e = 4 flagged by a negated kx; X = xp^(e-2) / Ax^e:
-          // h = xp^2 X + ..., h_x = e xp X, h_xx = e (e-1) X
-          const T xp = fma(lx, dirx, fma(ly, d2x, fma(co, dx, fma(so, dy, T(-tnow * o1.z)))));
-          const T yp = fma(lx, diry, fma(ly, d2y, fma(co, dy, fma(-so, dx, T(-tnow * o1.w)))));
+          // position relative to the (moving) obstacle centre at tnow
+          T xp = fma(co, dx, fma(so, dy, T(-tnow * o1.z)));
+          T yp = fma(co, dy, fma(-so, dx, T(-tnow * o1.w)));
+          T lx = 0.f, ly = 0.f, d2x = 0.f, d2y = 0.f;
+          if constexpr (DISCS) {
+            const float2 lvp = *reinterpret_cast<const float2*>(S.disc + 2 * (j - o * k.nd));  // lever arms on e1, e2
+            lx = lvp.x;
+            ly = lvp.y;
+            d2x = fma(co, c2, so * s2);
+            d2y = fma(co, s2, -(so * c2));
+            xp = fma(lx, dirx, fma(ly, d2x, xp));
+            yp = fma(lx, diry, fma(ly, d2y, yp));
+          }
           const bool e4 = o1.x < 0.f;
           const T kx = fabsf(o1.x), ky = o1.y;
           const T x2 = xp * xp, y2 = yp * yp;
@@ -1199,32 +1228,31 @@ __device__ void run_tile(const KConst& k, const Inst& in, int tile, float* uh, c
           const T ce = e4 ? 4.f : 2.f, cee = e4 ? 12.f : 2.f;
           h = fma(x2, X, fma(y2, Y, T(-1.f)));
           const T hx = ce * xp * X, hy = ce * yp * Y;
-          // disc velocity relative to the obstacle
-          const T lt1 = lx * th1dot, lt2 = ly * th2dot;
-          const T velx = fma(vv, dirx, T(-o1.z)) - fma(lt1, diry, lt2 * d2y);
-          const T vely = fma(vv, diry, T(-o1.w)) + fma(lt1, dirx, lt2 * d2x);
-          // disc acceleration = acc0 + a acc_a + omega acc_w
-          const T la1 = lx * tl, la2 = ly * a2a, lw1 = lx * a1w, lw2 = ly * a2w;
-          const T aax = dirx - fma(la1, diry, la2 * d2y);
-          const T aay = diry + fma(la1, dirx, la2 * d2x);
-          const T awx = -fma(lw1, diry, lw2 * d2y);
-          const T awy = fma(lw1, dirx, lw2 * d2x);
+          const T ge = fma(hx, dirx, hy * diry);     // grad h . e1'
+          const T gn = fma(hy, dirx, -(hx * diry));  // grad h . n1'
+          // velocity relative to the obstacle; acceleration = acc0 + a acc_a
+          // + omega acc_w, at the rear axle v th1dot n1 and a e1
+          T velx = fma(vv, dirx, T(-o1.z)), vely = fma(vv, diry, T(-o1.w));
           const T vw = vv * th1dot;
-          const T q1c = lt1 * th1dot, q2c = lt2 * th2dot, q20 = ly * a20;
-          const T a0x = -fma(vw, diry, fma(q1c, dirx, fma(q20, d2y, q2c * d2x)));
-          const T a0y = fma(vw, dirx, -fma(q1c, diry, fma(-q20, d2x, q2c * d2y)));
+          T ga0 = vw * gn;  // grad h . acc0
+          Aa = T(k.hTs2) * ge;
+          if constexpr (DISCS) {
+            const T lt1 = lx * th1dot, lt2 = ly * th2dot;
+            velx = velx - fma(lt1, diry, lt2 * d2y);
+            vely = vely + fma(lt1, dirx, lt2 * d2x);
+            const T g2 = fma(hx, d2x, hy * d2y), n2 = fma(hy, d2x, -(hx * d2y));  // grad h . e2', n2'
+            Aa = T(k.hTs2) * (ge + fma(lx * tl, gn, ly * a2a * n2));
+            Aw = T(k.hTs2) * fma(lx * a1w, gn, ly * a2w * n2);
+            ga0 = ga0 + fma(-(lt1 * th1dot), ge, fma(ly * a20, n2, -(lt2 * th2dot * g2)));
+          }
           const T hdot = fma(hx, velx, hy * vely);
           const T wHx = cee * X * velx, wHy = cee * Y * vely;  // Hess h w
-          const T hdd0 = fma(hx, a0x, fma(hy, a0y, fma(wHx, velx, wHy * vely)));
-          Aa = T(k.hTs2) * fma(hx, aax, hy * aay);
-          Aw = T(k.hTs2) * fma(hx, awx, hy * awy);
+          const T hdd0 = ga0 + fma(wHx, velx, wHy * vely);
           brest = fma(T(-k.Ts), hdot, T(-k.hTs2) * hdd0);
-          if (k.third) {
+          if (TERMS && k.third) {
             // Ts^3/6 hdddot at the rear axle (lever arms zero), affine in
             // (a, omega): pdddot = 2 a th1dot n1 + v th1ddot n1 - v th1dot^2 e1,
             // hdddot = grad h . pdddot + 3 w^T Hess h pddot + D3 h [w, w, w]
-            const T ge = fma(hx, dirx, hy * diry);     // grad h . e1'
-            const T gn = fma(hy, dirx, -(hx * diry));  // grad h . n1'
             const T ca3 = fma(fma(T(2.f), th1dot, vv * tl), gn, T(3.f) * fma(wHx, dirx, wHy * diry));
             const T cw3 = vv * vv * sec2 * T(k.inv_l1) * gn;
             T c03 = fma(-(vw * th1dot), ge, T(3.f) * vw * fma(wHy, dirx, -(wHx * diry)));
@@ -1234,22 +1262,22 @@ __device__ void run_tile(const KConst& k, const Inst& in, int tile, float* uh, c
             Aw = fma(T(k.Ts3_6), cw3, Aw);
             brest = fma(T(-k.Ts3_6), c03, brest);
           }
-          if (k.jerk) {
+          if (TERMS && k.jerk) {
             // a is a state (rear-axle point): its terms join the constant;
             // the jerk enters only at third order, through grad h . e1'
             brest = fma(-acc, Aa, brest);
-            Aa = k.third ? T(k.Ts3_6) * fma(hx, dirx, hy * diry) : T(0.f);
+            Aa = k.third ? T(k.Ts3_6) * ge : T(0.f);
           }
         }
         const T ht = vmap(h, [&](float x) { return copysignf(fmaxf(fabsf(x), k.h_floor), x); });
         T r = fma(Aa, q0, fma(ht, pam, fma(al, h, -brest)));
-        if constexpr (EXT) r = fma(Aw, q1, r);
+        if constexpr (TERMS) r = fma(Aw, q1, r);
         const T iht = vrcp(ht);  // MUFU reciprocal (~1 ulp)
         u = Aa * iht;
         const T rho = r * iht;
         Saa = fma(u, u, Saa);
         ga = fma(u, rho, ga);
-        if (EXT && k.abuf) {
+        if (TERMS && k.abuf) {
           // buffer zone: positive rates charged with weight clip(1 - h/h_buf)
           const T wz = vclamp(fma(h, T(-k.inv_hbuf), T(1.f)), 0.f, 1.f);
           const T ap = vmap(al, [](float x) { return fmaxf(x, 0.f); });
@@ -1257,7 +1285,7 @@ __device__ void run_tile(const KConst& k, const Inst& in, int tile, float* uh, c
         }
         // the rate's update without its part in y, added after the 2x2 solve
         al = al + (pam - rho);
-        if constexpr (EXT) {
+        if constexpr (TERMS) {
           w = Aw * iht;
           Saw = fma(u, w, Saw);
           Sww = fma(w, w, Sww);
@@ -1280,11 +1308,11 @@ __device__ void run_tile(const KConst& k, const Inst& in, int tile, float* uh, c
             const int j = 4 * (b - 1) + m;
             if (TPS > 1 || j < n_rows) {
               T al, u, w = 0.f;
-              load_row<EXT, NS>(row + m * row_stride, al, u, w);
+              load_row<TERMS, NS>(row + m * row_stride, al, u, w);
               al = fma(u, ya_p, al);
-              if constexpr (EXT) al = fma(w, yw_p, al);
+              if constexpr (TERMS) al = fma(w, yw_p, al);
               obstacle_row(min(j, n_rows), sampled_rate(k, nb[m]), al, u, w);
-              store_row<EXT, NS>(row + m * row_stride, al, u, w);
+              store_row<TERMS, NS>(row + m * row_stride, al, u, w);
             }
           }
         }
@@ -1296,21 +1324,21 @@ __device__ void run_tile(const KConst& k, const Inst& in, int tile, float* uh, c
         for (int slot = 0; slot < OBS_SLOTS; ++slot) {
           if (ROWS == 0) {
             ca[slot] = 0.f;
-            if constexpr (EXT) cw[slot] = 0.f;
+            if constexpr (TERMS) cw[slot] = 0.f;
           }
           if (ROWS > 0 || slot < per_lane) {
             const int j = lt + TPS * slot;
             T w = 0.f;
             obstacle_row(min(j, n_rows), T(cur[4 + min(j, n_rows - 1)]), alpha[slot], ca[slot], w);
-            if constexpr (EXT) cw[slot] = w;
+            if constexpr (TERMS) cw[slot] = w;
           }
         }
       }
-      if (EXT && k.abuf) add_share(cbuf);
+      if (TERMS && k.abuf) add_share(cbuf);
       const T m_a = k.m_a;
       Saa = fma(m_a, fma(u_h, u_h, team_sum<TPS>(Saa)), T(k.m_u0));
       ga = m_a * fma(u_h, rho_h, team_sum<TPS>(ga));
-      if constexpr (EXT) {
+      if constexpr (TERMS) {
         Saw = m_a * fma(u_h, w_h, team_sum<TPS>(Saw));
         Sww = fma(m_a, fma(w_h, w_h, team_sum<TPS>(Sww)), T(k.m_u1));
         gw = m_a * fma(w_h, rho_h, team_sum<TPS>(gw));
@@ -1328,7 +1356,7 @@ __device__ void run_tile(const KConst& k, const Inst& in, int tile, float* uh, c
       alpha_h = alpha_h + fma(w_h, yw, fma(u_h, ya, cc_h));
       auto alpha_update = [&](int slot) {
         alpha[slot] = fma(ca[slot], ya, alpha[slot]);
-        if constexpr (EXT) alpha[slot] = fma(cw[slot], yw, alpha[slot]);
+        if constexpr (TERMS) alpha[slot] = fma(cw[slot], yw, alpha[slot]);
       };
       if constexpr (!PRODUCED) {
         ya_p = ya;
@@ -1351,7 +1379,7 @@ __device__ void run_tile(const KConst& k, const Inst& in, int tile, float* uh, c
     pyl = pyl_n;
     t1 = t1_n;
     t2 = t2_n;
-    if (EXT && k.jerk) {  // input 0 is the jerk; the acceleration state drives the speed
+    if (TERMS && k.jerk) {  // input 0 is the jerk; the acceleration state drives the speed
       acc2(v, vl, T(k.Ts) * acc);
       acc = fma(T(k.Ts), ua, acc);
     } else {
@@ -1913,12 +1941,11 @@ __device__ __forceinline__ void discard_history(const float* uh, int n_floats) {
 }
 
 // -------------------------------------------------------------- the kernel
+// EXT: the family (Family, above run_tile).
 // Launch bound of the two-sample variants: 384 threads an SM (168 registers),
 // in CTAs of up to 192
 constexpr int kMaxPairThreads = 192, kPairCtas = 2;
-// EXT: the instantiations that also carry the optional terms (moving and
-// e = 4 obstacles, collision cost, buffer cost); the others compile them out.
-template <int TPS, int BPT, bool EXT, int ROWS = 0, int NS = 1, bool LOCAL = false>
+template <int TPS, int BPT, int EXT, int ROWS = 0, int NS = 1, bool LOCAL = false>
 // Launch bound: 512 threads (128 registers a thread); the exact-rows
 // single-solve instantiations 384 (up to 170 registers: one CTA per SM on
 // the latency shapes, where registers buy a longer schedule)
