@@ -757,7 +757,7 @@ __device__ void run_tile(const KConst& k, const Inst& in, int tile, float* uh, c
       // stays in registers
       const Draw d = make_draw(min(pl, n_blocks - 1));
       for (int tau = 0; tau < H; ++tau) {
-        if (pl < n_blocks) produce(d, tau);
+        if ((pl & ~31) < n_blocks) produce(d, tau);  // (a warp's threads past the last block draw it again)
         if (tau == 0) staging_barrier();
         step_barrier();
       }
@@ -818,6 +818,17 @@ __device__ void run_tile(const KConst& k, const Inst& in, int tile, float* uh, c
   if constexpr (!PRODUCED)
     for (int q = 0; q < 4 * passes; ++q) store_row<TERMS, NS>(rows + q * row_stride, T(k.alpha0), T(0.f), T(0.f));
   T ya_p = 0.f, yw_p = 0.f;  // the step before's y
+  // exact-rows variants: a lane's rows are the same at every step, so their
+  // table entries stay in registers
+  float4 row_a[ROWS > 0 ? ROWS : 1], row_b[ROWS > 0 ? ROWS : 1];
+  if constexpr (ROWS > 0 && !DISCS) {
+#pragma unroll
+    for (int q = 0; q < ROWS; ++q) {
+      const int j = min(lt + TPS * q, n_rows);
+      row_a[q] = *reinterpret_cast<const float4*>(S.obs + 8 * j);
+      row_b[q] = *reinterpret_cast<const float4*>(S.obs + 8 * j + 4);
+    }
+  }
   T Jh = 0.f, Jl = 0.f;
   T ua = 0.f, uw = 0.f, un = 0.f;  // applied input of the previous step
   const uint32_t sid = static_cast<uint32_t>(s);
@@ -900,14 +911,9 @@ __device__ void run_tile(const KConst& k, const Inst& in, int tile, float* uh, c
     T x0r, y0r, t0r, x1r, y1r, t1r, x0l, y0l, x1l, y1l;
 #pragma unroll
     for (int i = 0; i < NS; ++i) {
-      int ii = i0 + (__float_as_int(tt.get(i)) - 0x4b400000);
-      if (ii < 0) {
-        ii = 0;
-        ff.set(i, 0.f);
-      } else if (ii > n_pts - 2) {
-        ii = n_pts - 2;
-        ff.set(i, 1.f);
-      }
+      const int cell = i0 + (__float_as_int(tt.get(i)) - 0x4b400000);
+      const int ii = max(min(cell, n_pts - 2), 0);
+      ff.set(i, cell == ii ? ff.get(i) : (cell < ii ? 0.f : 1.f));  // beyond an end: that end
       const float4 a = *reinterpret_cast<const float4*>(S.path + 4 * ii);
       const float4 b = *reinterpret_cast<const float4*>(S.path + 4 * ii + 4);
       x0r.set(i, a.x);
@@ -1005,6 +1011,7 @@ __device__ void run_tile(const KConst& k, const Inst& in, int tile, float* uh, c
       o[6] = (fr.psi_h + ps.get(i)) + (fr.psi_l + psl.get(i));
     }
   };
+  const bool per_sample_out = in.states_out || in.inputs_out;
   if (st_out) store_state(0);
 
   // Noise.  Teams of at most two Philox blocks per lane, one sample each (the
@@ -1183,12 +1190,12 @@ __device__ void run_tile(const KConst& k, const Inst& in, int tile, float* uh, c
       const T cg_row = T(-2.f * k.Ts) * vv, vth_row = T(-k.Ts2) * (vv * th1dot), vq_row = T(-k.Ts2) * (vv * vv);
       const T bx_row = fma(cg_row, c1, -(vth_row * s1)), by_row = fma(cg_row, s1, vth_row * c1);
       const T qxx_row = vq_row * (c1 * c1), qyy_row = vq_row * (s1 * s1), qxy_row = (vq_row + vq_row) * (c1 * s1);
-      auto obstacle_row = [&](int j, T pam, T& al, T& u, T& w) {  // pam: p_alpha / m_alpha
+      auto obstacle_row = [&](int j, int slot, T pam, T& al, T& u, T& w) {  // pam: p_alpha / m_alpha
         T h, Aa, Aw = 0.f, brest;
         if constexpr (!EXT) {
           // staged as (cx, cy, Qxx, Qxy, Qyy): h = d^T Q d - 1 in the frame
-          const float4 o0 = *reinterpret_cast<const float4*>(S.obs + 8 * j);
-          const T qxx = o0.z, qxy = o0.w, qyy = S.obs[8 * j + 4];
+          const float4 o0 = ROWS > 0 ? row_a[slot] : *reinterpret_cast<const float4*>(S.obs + 8 * j);
+          const T qxx = o0.z, qxy = o0.w, qyy = ROWS > 0 ? row_b[slot].x : S.obs[8 * j + 4];
           const T dx = (px - T(o0.x)) + pxl, dy = (py - T(o0.y)) + pyl;
           const T gx = fma(qxx, dx, qxy * dy), gy = fma(qxy, dx, qyy * dy);
           h = fma(gx, dx, fma(gy, dy, T(-1.f)));
@@ -1203,8 +1210,9 @@ __device__ void run_tile(const KConst& k, const Inst& in, int tile, float* uh, c
           // h_xx = e (e-1) X
           int o = j;
           if constexpr (DISCS) o = (k.nd == 1) ? j : __float2int_rz((static_cast<float>(j) + 0.5f) * k.inv_nd);
-          const float4 o0 = *reinterpret_cast<const float4*>(S.obs + 8 * o);
-          const float4 o1 = *reinterpret_cast<const float4*>(S.obs + 8 * o + 4);
+          const bool kept_row = ROWS > 0 && !DISCS;
+          const float4 o0 = kept_row ? row_a[ROWS > 0 ? slot : 0] : *reinterpret_cast<const float4*>(S.obs + 8 * o);
+          const float4 o1 = kept_row ? row_b[ROWS > 0 ? slot : 0] : *reinterpret_cast<const float4*>(S.obs + 8 * o + 4);
           const T co = o0.z, so = o0.w;
           const T dirx = fma(co, c1, so * s1), diry = fma(co, s1, -(so * c1));
           const T dx = (px - T(o0.x)) + pxl, dy = (py - T(o0.y)) + pyl;
@@ -1311,7 +1319,7 @@ __device__ void run_tile(const KConst& k, const Inst& in, int tile, float* uh, c
               load_row<TERMS, NS>(row + m * row_stride, al, u, w);
               al = fma(u, ya_p, al);
               if constexpr (TERMS) al = fma(w, yw_p, al);
-              obstacle_row(min(j, n_rows), sampled_rate(k, nb[m]), al, u, w);
+              obstacle_row(min(j, n_rows), 0, sampled_rate(k, nb[m]), al, u, w);
               store_row<TERMS, NS>(row + m * row_stride, al, u, w);
             }
           }
@@ -1329,7 +1337,7 @@ __device__ void run_tile(const KConst& k, const Inst& in, int tile, float* uh, c
           if (ROWS > 0 || slot < per_lane) {
             const int j = lt + TPS * slot;
             T w = 0.f;
-            obstacle_row(min(j, n_rows), T(cur[4 + min(j, n_rows - 1)]), alpha[slot], ca[slot], w);
+            obstacle_row(min(j, n_rows), slot, T(cur[4 + min(j, n_rows - 1)]), alpha[slot], ca[slot], w);
             if constexpr (TERMS) cw[slot] = w;
           }
         }
@@ -1397,6 +1405,7 @@ __device__ void run_tile(const KConst& k, const Inst& in, int tile, float* uh, c
       store_pair(uh + (3 * tau + 1) * spb + team * NS, uw);
       store_pair(uh + (3 * tau + 2) * spb + team * NS, un);
     }
+    if (!per_sample_out) return;  // the same for every thread
     if (st_out) store_state(tau + 1);
     if (in_out) {
 #pragma unroll
