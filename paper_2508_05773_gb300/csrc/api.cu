@@ -272,6 +272,10 @@ bool fit_rows(brmppi::SmemCaps* c, int spb, size_t smem_limit) {
   return false;
 }
 
+int serving_team_width(const brmppi_params& p, int P) {
+  return brmppi::family_of(make_kconst(p)) != brmppi::kPlain ? ext_team_width(P) : 1;
+}
+
 bool pick_bpt(int tps, int P, int* bpt) {
   // Philox blocks of rows a lane holds: up to two of them are drawn by
   // producer warps (bpt 1, 2; teams), more by the lane itself (bpt 3; one
@@ -570,7 +574,8 @@ bool batch_shape_default(const brmppi_ctx* c, int max_P, Shape* out) {
   } else {
     // One lane a sample: the step's base is not repeated over a team, and the
     // rows' state in shared memory leaves registers for any number of rows.
-    // With the optional terms only where the context's capacity (which fixes
+    // A serving context's batches take the served ones' width.  Else, with
+    // the optional terms, only where the context's capacity (which fixes
     // the width: a solve's bits must not depend on its batch) can fill the
     // GPU: their step is long, and few solves finish sooner on wider teams.
     // Measured on GB300, S = 4096, H = 50, 8 moving rows, one lane against two
@@ -579,7 +584,8 @@ bool batch_shape_default(const brmppi_ctx* c, int max_P, Shape* out) {
     // 200 solves 1.00 / 2.15 ms.
     const bool wide = brmppi::family_of(make_kconst(c->prm)) != brmppi::kPlain &&
                       static_cast<long long>(c->prm.max_batch) * c->prm.S < 200LL * c->num_sms;
-    if (s.tps == 0) s.tps = wide ? ext_team_width(max_P) : 1;
+    if (s.tps == 0)
+      s.tps = c->prm.max_vehicles > 0 ? serving_team_width(c->prm, max_P) : (wide ? ext_team_width(max_P) : 1);
     if (s.threads == 0) s.threads = std::max(128, kMinBatchSpb * s.tps);
   }
   while (!pick_bpt(s.tps, max_P, &s.bpt)) {

@@ -152,9 +152,10 @@ bool pick_bpt(int tps, int P, int* bpt);
 // from the caps and return false (it goes to local memory).
 bool fit_rows(brmppi::SmemCaps* c, int spb, size_t smem_limit);
 int part_stride_for(int H);
-// Team width of batches (of small contexts) and serving when the optional
-// terms are on.
-int ext_team_width(int P);
+// Team width of a serving context's batches, the served ones and the caller's
+// (a batch of one reproduces a served solve bit for bit): one lane, or with
+// the optional terms a team that keeps a lightly loaded server's step short.
+int serving_team_width(const brmppi_params& p, int P);
 brmppi_status check_sizes(brmppi_ctx* c, int32_t n_obs, int32_t n_pts, float ds);
 // Options of a single (non-batch) solve launch: the exact-rows variant, with
 // the applied-input history and the merge of the tile partials in shared

@@ -305,9 +305,7 @@ brmppi_status server_create(brmppi_ctx* c) {
   // enough for two Philox blocks a lane when rows carry a steer-rate column)
   // in 128-thread blocks
   const int P_cap = philox_blocks(rows_of(p, p.max_obstacles));
-  sv->shape.tps = p.batch_threads_per_sample != 0
-                      ? p.batch_threads_per_sample
-                      : (brmppi::family_of(make_kconst(p)) != brmppi::kPlain ? ext_team_width(P_cap) : 1);
+  sv->shape.tps = p.batch_threads_per_sample != 0 ? p.batch_threads_per_sample : serving_team_width(p, P_cap);
   sv->shape.threads =
       p.batch_block_threads != 0 ? p.batch_block_threads : std::max(128, kMinBatchSpb * sv->shape.tps);
   if (!pick_bpt(sv->shape.tps, P_cap, &sv->shape.bpt) || sv->shape.threads / sv->shape.tps < kMinBatchSpb) {
