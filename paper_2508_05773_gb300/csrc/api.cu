@@ -97,8 +97,6 @@ brmppi_status cuda_fail(brmppi_ctx* c, cudaError_t e, const char* what) {
 
 int philox_blocks(int n_rows) { return (4 + n_rows + 3) / 4; }  // d = 3 + (1 + n_rows), rows = obstacles x discs
 
-int ext_team_width(int P) { return P <= 4 ? 2 : (P <= 8 ? 4 : (P <= 16 ? 8 : 16)); }
-
 namespace {
 
 bool is_pow2_tps(int t) { return t == 1 || t == 2 || t == 4 || t == 8 || t == 16 || t == 32; }
@@ -273,7 +271,8 @@ bool fit_rows(brmppi::SmemCaps* c, int spb, size_t smem_limit) {
 }
 
 int serving_team_width(const brmppi_params& p, int P) {
-  return brmppi::family_of(make_kconst(p)) != brmppi::kPlain ? ext_team_width(P) : 1;
+  if (brmppi::family_of(make_kconst(p)) == brmppi::kPlain) return 1;
+  return P <= 4 ? 2 : (P <= 8 ? 4 : (P <= 16 ? 8 : 16));
 }
 
 bool pick_bpt(int tps, int P, int* bpt) {
@@ -305,12 +304,9 @@ int samples_per_team(const Shape& sh, int family, long long tiles, size_t smem, 
 
 int part_stride_for(int H) { return static_cast<int>(align_up(3 + 3 * static_cast<size_t>(H) + 1, 4)); }
 
-// Default shape of a plain solve (no autotuning): tiles that spread the
-// samples evenly over the SMs, and a team as wide as keeps an SM at a few
-// warps.
-//
-// Team width.  A team one Philox block a lane wide has the shortest step, but
-// repeats the step's base on every lane: it is halved while that leaves an SM
+// Team width for `samples` samples that run at once.  A team one Philox block a
+// lane wide has the shortest step, but repeats the step's base on every
+// lane: it is halved while that leaves an SM
 // more than `most` warps.  Measured on GB300 (S samples, n ellipses, H = 30
 // or 20; us at the wider / the narrower team): n = 8, P = 3: S = 6500 33.7 /
 // 35.9 with 5.3 warps an SM at the wider, 8192 41.9 / 36.2 with 6.7; two
@@ -321,6 +317,21 @@ int part_stride_for(int H) { return static_cast<int>(align_up(3 + 3 * static_cas
 // P = 1: 4096 27.6 / 29.5 with 1.7 (the noise leaves the chain), 10000 34.0 /
 // 30.8 with 4.1.  The optional terms' longer rows take wider teams further:
 // n = 8: 8000 47.5 / 54.6 with 6.6, two lanes to one 20000 93.6 / 105 with 8.2.
+int team_width(int P, long long samples, bool ext, int num_sms) {
+  int tps = 2, bpt = 0;
+  while (tps < P && tps < 16) tps <<= 1;
+  while (tps > 1 && pick_bpt(tps / 2, P, &bpt)) {
+    double most = ext ? 9.0 : (tps == 2 ? 12.0 : 7.5);
+    if (P <= 4) most = tps == 2 ? (P == 1 ? 3.0 : (ext ? 9.0 : 7.0)) : (ext ? 7.0 : (P == 4 ? 6.5 : 5.75));
+    if (static_cast<double>(samples) * tps <= most * 32.0 * num_sms) break;
+    tps >>= 1;
+  }
+  return tps;
+}
+
+// Default shape of a plain solve (no autotuning): tiles that spread the
+// samples evenly over the SMs, and a team as wide as keeps an SM at a few
+// warps.
 //
 // Tile.  One CTA an SM that holds ceil(S / SMs) samples, where that fits the
 // block: a tile count just over the SM count leaves most of them idle for a
@@ -336,17 +347,7 @@ bool heuristic_plain(const brmppi_ctx* c, int n_obs, int n_pts, Shape* out) {
   const int family = brmppi::family_of(make_kconst(c->prm));
   const bool ext = family == brmppi::kDiscs || family == brmppi::kPoint;
   int tps = c->prm.threads_per_sample;
-  if (!fixed_tps) {
-    tps = 2;
-    while (tps < P && tps < 16) tps <<= 1;
-    int b2 = 0;
-    while (tps > 1 && pick_bpt(tps / 2, P, &b2)) {
-      double most = ext ? 9.0 : (tps == 2 ? 12.0 : 7.5);
-      if (P <= 4) most = tps == 2 ? (P == 1 ? 3.0 : (ext ? 9.0 : 7.0)) : (ext ? 7.0 : (P == 4 ? 6.5 : 5.75));
-      if (static_cast<double>(S) * tps <= most * 32.0 * static_cast<double>(sms)) break;
-      tps >>= 1;
-    }
-  }
+  if (!fixed_tps) tps = team_width(P, S, ext, c->num_sms);
   int bpt = 0;
   if (!pick_bpt(tps, P, &bpt)) return false;
   int threads = c->prm.block_threads;
@@ -572,20 +573,38 @@ bool batch_shape_default(const brmppi_ctx* c, int max_P, Shape* out) {
   if (s.tps == 0 && s.threads == 0 && c->batch_tuned) {
     s = c->batch_shape;
   } else {
-    // One lane a sample: the step's base is not repeated over a team, and the
-    // rows' state in shared memory leaves registers for any number of rows.
-    // A serving context's batches take the served ones' width.  Else, with
-    // the optional terms, only where the context's capacity (which fixes
-    // the width: a solve's bits must not depend on its batch) can fill the
-    // GPU: their step is long, and few solves finish sooner on wider teams.
-    // Measured on GB300, S = 4096, H = 50, 8 moving rows, one lane against two
-    // (every optional term compiled in): 200 solves 2.53 / 4.06 ms, 8 solves
-    // 185 / 238 us, 4 solves 143 / 125 us, 1 solve 142 / 92 us; collision cost,
-    // 200 solves 1.00 / 2.15 ms.
-    const bool wide = brmppi::family_of(make_kconst(c->prm)) != brmppi::kPlain &&
-                      static_cast<long long>(c->prm.max_batch) * c->prm.S < 200LL * c->num_sms;
-    if (s.tps == 0)
-      s.tps = c->prm.max_vehicles > 0 ? serving_team_width(c->prm, max_P) : (wide ? ext_team_width(max_P) : 1);
+    // A serving context's batches take the served ones' width.  Else the team
+    // width for as many samples as the context's capacity allows at once (the
+    // capacity fixes it: a solve's bits must not depend on its batch), as far
+    // as the tables at that capacity fit beside the team's noise.  From 17,000
+    // samples (13 rows; 29,000 with more) one lane a sample: the step's base
+    // is not repeated over a team, and the rows' state in shared memory
+    // leaves registers for any number of rows.  Measured on GB300, S = 4096,
+    // H = 50, 8 rows, one lane against teams of two: 200 solves of moving rows
+    // 2.53 / 4.06 ms, of collision cost 1.00 / 2.15 ms.  One lane against the
+    // rule's width: 1 solve of parked ellipses 96 / 60 us (four lanes), 2 solves
+    // 96 / 70, 4 solves 97 / 95.  The optional terms against teams of two for
+    // any small capacity: 1 solve of third order and jerk 87.6 / 75.3 us (but 2
+    // solves 87.6 / 92.6), 6 solves of moving rows 144 / 133, of collision cost
+    // 103 / 79; four discs on teams of four, 3 solves 208 / 233, 4 solves 248 / 233.
+    if (s.tps == 0) {
+      const int family = brmppi::family_of(make_kconst(c->prm));
+      const auto fits = [&](int tps) {
+        const int threads = s.threads > 0 ? s.threads : std::max(128, kMinBatchSpb * tps);
+        int bpt = 0;
+        if (threads / tps < kMinBatchSpb || !pick_bpt(tps, max_P, &bpt)) return false;
+        return table_bytes(make_caps(c->prm.max_obstacles, rows_of(c->prm, c->prm.max_obstacles), c->prm.max_path_pts,
+                                     c->prm.H, tps, bpt, family),
+                           threads / tps) <= c->smem_limit;
+      };
+      if (c->prm.max_vehicles > 0) {
+        s.tps = serving_team_width(c->prm, max_P);
+      } else {
+        s.tps = team_width(max_P, static_cast<long long>(c->prm.max_batch) * c->prm.S,
+                           family == brmppi::kDiscs || family == brmppi::kPoint, c->num_sms);
+        while (s.tps > 1 && !fits(s.tps)) s.tps >>= 1;
+      }
+    }
     if (s.threads == 0) s.threads = std::max(128, kMinBatchSpb * s.tps);
   }
   while (!pick_bpt(s.tps, max_P, &s.bpt)) {
