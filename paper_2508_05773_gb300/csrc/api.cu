@@ -290,16 +290,22 @@ bool pick_bpt(int tps, int P, int* bpt) {
 }
 
 // CTAs of `threads` threads of the two-sample variants on an SM.
-long long pair_residency(int threads, size_t smem) {
-  return std::min<long long>(brmppi::kMaxPairBlockThreads * brmppi::kPairCtas / threads, 227 * 1024 / (smem + 2048));
+long long pair_residency(int tps, int family, int threads, size_t smem) {
+  return std::min<long long>(brmppi::pair_threads(tps, family) * brmppi::kPairCtas / threads,
+                             227 * 1024 / (smem + 2048));
 }
 
+// Two samples a team where their CTAs fill three quarters of the GPU's places:
+// from there the halved issue slots are worth more than the idle places.
+// Measured on GB300, one lane, S = 4096, H = 50, 8 rows, one sample / two: 32
+// solves (1024 tiles for 1216 places) 318 / 293 us, 36 solves 356 / 297; 24
+// of moving rows (768 for 912) 304 / 268, 22 of collision cost 142 / 144.
 int samples_per_team(const Shape& sh, int family, long long tiles, size_t smem, int num_sms) {
   const int threads = sh.threads / 2;
-  if (sh.threads % 64 != 0 || threads < 64 || threads > brmppi::kMaxPairBlockThreads ||
+  if (sh.threads % 64 != 0 || threads < 64 || threads > brmppi::pair_threads(sh.tps, family) ||
       !brmppi::pair_exists(sh.tps, sh.bpt, family))
     return 1;
-  return tiles >= pair_residency(threads, smem) * num_sms ? 2 : 1;
+  return tiles * 4 >= pair_residency(sh.tps, family, threads, smem) * num_sms * 3 ? 2 : 1;
 }
 
 int part_stride_for(int H) { return static_cast<int>(align_up(3 + 3 * static_cast<size_t>(H) + 1, 4)); }
@@ -365,7 +371,7 @@ bool heuristic_plain(const brmppi_ctx* c, int n_obs, int n_pts, Shape* out) {
       // more samples on an SM
       auto resident = [&](int t) {
         const size_t smem = smem_bytes(make_caps(n_obs, rows, n_pts, c->prm.H, tps, bpt, family), t / tps);
-        return pair_residency(t / 2, smem) * t;
+        return pair_residency(tps, family, t / 2, smem) * t;
       };
       threads = brmppi::pair_exists(tps, bpt, family) && resident(384) > resident(256) ? 384 : 256;
     }

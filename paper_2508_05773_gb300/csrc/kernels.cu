@@ -174,7 +174,7 @@ int exact_rows_variant(int tps, int bpt, const KConst& k, int n_rows) {
 int variant_occupancy(int tps, int bpt, int threads, size_t smem, int family, int P, LaunchMode mode) {
   const int ns = mode.ns;
   const Variant* v = find(tps, bpt, family, 0, mode);
-  if (!v || block_threads(tps, bpt, threads, P, ns) > (ns > 1 ? kMaxPairBlockThreads : kMaxBlockThreads)) return 0;
+  if (!v || block_threads(tps, bpt, threads, P, ns) > (ns > 1 ? pair_threads(tps, v->family) : kMaxBlockThreads)) return 0;
   int n = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, v->fn, block_threads(tps, bpt, threads, P, ns), smem) !=
       cudaSuccess)
@@ -186,7 +186,7 @@ cudaError_t launch_solve(int tps, int bpt, int blocks, int threads, size_t smem,
                          const KConst& k, const LaunchDesc& L, int P, LaunchMode mode) {
   const int ns = mode.ns;
   const Variant* v = find(tps, bpt, family_of(k), 0, mode);
-  if (!v || block_threads(tps, bpt, threads, P, ns) > (ns > 1 ? kMaxPairBlockThreads : kMaxBlockThreads))
+  if (!v || block_threads(tps, bpt, threads, P, ns) > (ns > 1 ? pair_threads(tps, v->family) : kMaxBlockThreads))
     return cudaErrorInvalidValue;
   if (L.rows > 0) {
     // the exact-rows variants merge in shared memory: the launch must have

@@ -47,7 +47,6 @@ inline int family_of(const KConst& k) {
 // their own lanes (0 noise warps).  At most kMaxBlockThreads (the kernels'
 // launch bound).
 constexpr int kMaxBlockThreads = 512;
-constexpr int kMaxPairBlockThreads = kMaxPairThreads;  // the two-sample instantiations' launch bound
 constexpr int kMaxRowsBlockThreads = 384;  // the exact-rows instantiations' launch bound
 // How a shape is run: samples a team, and the rows' state in local memory
 // (where it does not fit in shared memory; one sample a team).

@@ -1952,13 +1952,18 @@ __device__ __forceinline__ void discard_history(const float* uh, int n_floats) {
 // -------------------------------------------------------------- the kernel
 // EXT: the family (Family, above run_tile).
 // Launch bound of the two-sample variants: 384 threads an SM (168 registers),
-// in CTAs of up to 192
-constexpr int kMaxPairThreads = 192, kPairCtas = 2;
+// in CTAs of up to 192.  One lane a sample without optional terms keeps nearly
+// all of its step in 128 registers (36 B spilled), and a fourth warp a
+// scheduler is worth more: on GB300 48 solves of S = 4096, H = 50, 8 rows
+// 410 -> 386 us, 256 uneven ones 1820 -> 1800.  Moving rows lose by it (32
+// solves of S = 4096 338 -> 354 us), and so do third-order rows (422 -> 434).
+constexpr int kPairCtas = 2;
+constexpr int pair_threads(int tps, int family) { return tps == 1 && family == kPlain ? 256 : 192; }
 template <int TPS, int BPT, int EXT, int ROWS = 0, int NS = 1, bool LOCAL = false>
 // Launch bound: 512 threads (128 registers a thread); the exact-rows
 // single-solve instantiations 384 (up to 170 registers: one CTA per SM on
 // the latency shapes, where registers buy a longer schedule)
-__global__ void __launch_bounds__(ROWS > 0 ? 384 : (NS > 1 ? kMaxPairThreads : 512), NS > 1 ? kPairCtas : 1) solve_kernel(const KConst k, const LaunchDesc L) {
+__global__ void __launch_bounds__(ROWS > 0 ? 384 : (NS > 1 ? pair_threads(TPS, EXT) : 512), NS > 1 ? kPairCtas : 1) solve_kernel(const KConst k, const LaunchDesc L) {
   extern __shared__ float dyn[];
   __shared__ Shared sh;
   const int spb = compute_threads<TPS>(L.noise_warps) / TPS * NS;

@@ -35,7 +35,7 @@ def _instance(c, dev):
     return d
 
 
-@pytest.mark.parametrize("tps,threads,most", [(1, 128, 28), (1, 256, 28), (2, 128, 28), (4, 256, 40), (8, 256, 70)])
+@pytest.mark.parametrize("tps,threads,most", [(1, 128, 28), (1, 256, 28), (1, 512, 28), (2, 128, 28), (4, 256, 40), (8, 256, 70)])
 def test_two_samples_a_team_equal_one(pkg, tps, threads, most):
     """A batch with enough tiles runs two samples a team in packed
     registers, the same solve alone one sample a team: every output is the
