@@ -77,16 +77,16 @@ def ops_per_rollout_step(n_obs: int, proj: bool = True) -> int:
 
 # Of those, the elementary functions the step evaluates on the XU (the
 # special-function pipe, 16 lanes a clock per SM against 128 for FP32): per
-# Philox block the reciprocals of the two Box-Muller logarithms' reductions
-# and the two radii (reciprocal square root); per constraint row one
-# reciprocal (1 / h~); per step the steer angle's tangent and the 2x2
-# determinant (one reciprocal each).  The logarithms' series, Box-Muller's
-# sin / cos of 2 pi u and the state angles' sin / cos are FP32 polynomials.
+# Philox block the two Box-Muller radii (reciprocal square root); per
+# constraint row one reciprocal (1 / h~); per step the steer angle's tangent
+# and the 2x2 determinant (one reciprocal each).  Box-Muller's logarithm and
+# sin / cos of 2 pi u are tables with short FP32 series, the state angles'
+# sin / cos FP32 polynomials.
 def xu_ops_per_rollout_step(n_obs: int, proj: bool = True) -> int:
     if not proj:
-        return 4 + 1
+        return 2 + 1
     P = (3 + 1 + n_obs + 3) // 4
-    return 4 * P + 2 + (1 + n_obs)
+    return 2 * P + 2 + (1 + n_obs)
 
 
 # ----------------------------------------------------------------------------
@@ -152,10 +152,10 @@ def _dist_env():
 
 def kernel_source_hash() -> str:
     """First 16 hex digits of the SHA-256 of the solve kernel's device code
-    and launch logic (trig.cuh, rollout.cuh, then kernels.cu)."""
+    and launch logic."""
     import hashlib
     h = hashlib.sha256()
-    for name in ("trig.cuh", "rollout.cuh", "kernels.cu"):
+    for name in ("trig.cuh", "vec.cuh", "noise.cuh", "rollout.cuh", "kernels.cu"):
         with open(os.path.join(ROOT, "paper_2508_05773_gb300", "csrc", name), "rb") as f:
             h.update(f.read())
     return h.hexdigest()[:16]

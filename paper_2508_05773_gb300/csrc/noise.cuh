@@ -6,7 +6,7 @@
 // GB300; an FFMA 1.07), so a block costs as much FMA time as 80 FFMAs.  Its
 // four normals took 64 more FP32 operations with polynomial logarithms and
 // angles.  Both are cut here without changing a Philox word: 16 multiplies a
-// block, and 42 FP32 operations and 2 MUFU for the four normals.
+// block, and 48 FP32 operations and 2 MUFU for the four normals.
 #pragma once
 
 #include <cstdint>

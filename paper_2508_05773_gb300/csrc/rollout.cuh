@@ -42,13 +42,13 @@
 //
 // What bounds it (measured on GB300, before this layout -> with it): the
 // throughput shapes are bound by issue slots and the FMA pipe.  48 solves of
-// 4096 samples, H = 50, 8 ellipses: 493 -> 400 us, 1359 -> 740 thread
+// 4096 samples, H = 50, 8 ellipses: 493 -> 387 us, 1359 -> 740 thread
 // instructions a rollout-step (packed pairs, table-driven normals, the first
 // Philox rounds shared, rows as linear forms in (Q d, Q), no subnormal
-// scaling around the MUFU); 256 uneven solves 2567 -> 1768 us; S = 65536,
-// H = 100, 64 ellipses 2030 -> 1394 us (FMA pipe 58% and ALU pipe 40% busy,
+// scaling around the MUFU); 256 uneven solves 2567 -> 1802 us; S = 65536,
+// H = 100, 64 ellipses 2030 -> 1482 us (FMA pipe 58% and ALU pipe 40% busy,
 // three warps a scheduler).  The latency shapes are bound by one compute
-// warp's dependency chain: S = 4096, H = 50, 8 ellipses 39.6 -> 34.7 us.
+// warp's dependency chain: S = 4096, H = 50, 8 ellipses 39.6 -> 31.7 us.
 //
 // Projection in Woodbury form.  A = [A_u | diag(h~)] where only the a and
 // omega columns of A_u are non-zero, M = diag(m_u, m_alpha):
