@@ -1165,7 +1165,9 @@ brmppi_status brmppi_autotune(brmppi_ctx* c, const double* x0, const float* U_no
     if (!pick_bpt(tps, P, &bpt)) continue;
     const brmppi::SmemCaps caps = make_caps(n_obs, rows_of(c->prm, n_obs), n_pts, H, tps, bpt,
                                             brmppi::family_of(make_kconst(c->prm)));
-    for (int threads : {64, 128, 256}) {
+    // 384: pairs of samples in CTAs of 192 threads, which the default rule
+    // takes too (S = 65536, H = 100, 64 ellipses: 256 / 384 1.60 / 1.48 ms)
+    for (int threads : {64, 128, 256, 384}) {
       if (threads < tps || threads / tps < 2) continue;
       const int spb = threads / tps;
       if (table_bytes(caps, spb) > c->smem_limit) continue;
