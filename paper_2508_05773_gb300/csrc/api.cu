@@ -463,6 +463,19 @@ void single_launch_options(brmppi::LaunchDesc& L, const Shape& sh, const brmppi:
   L.rows = rows;
 }
 
+size_t plan_single(const brmppi_ctx* c, const Shape& sh, const brmppi::KConst& k, int tiles, brmppi::LaunchDesc* L,
+                   brmppi::LaunchMode* mode) {
+  const int spb = sh.threads / sh.tps;
+  const int family = brmppi::family_of(k);
+  const int rows = rows_of(c->prm, L->single.n_obs);
+  L->caps = make_caps(L->single.n_obs, rows, L->single.n_pts, L->single.H, sh.tps, sh.bpt, family);
+  mode->local = !fit_rows(&L->caps, spb, c->smem_limit);
+  single_launch_options(*L, sh, k, rows, L->single.H, c->smem_limit);
+  const size_t smem = smem_bytes(L->caps, spb);
+  if (L->rows == 0 && !mode->local) mode->ns = samples_per_team(sh, family, tiles, smem, c->num_sms);
+  return smem;
+}
+
 brmppi_status check_sizes(brmppi_ctx* c, int32_t n_obs, int32_t n_pts, float ds) {
   if (n_obs < 0 || n_obs > c->prm.max_obstacles) return fail(c, BRMPPI_EINVAL, "n_obs out of [0, max_obstacles]");
   if (n_pts < 2 || n_pts > c->prm.max_path_pts) return fail(c, BRMPPI_EINVAL, "n_pts out of [2, max_path_pts]");
@@ -492,20 +505,15 @@ brmppi_status enqueue_plain_sized(brmppi_ctx* c, const Shape& sh, int S, int H, 
     L.single.no_merge = 1;
   }
   const brmppi::KConst k = make_kconst(c->prm);
-  const int family = brmppi::family_of(k);
-  L.caps = make_caps(n_obs, rows_of(c->prm, n_obs), n_pts, H, sh.tps, sh.bpt, family);
-  brmppi::LaunchMode mode;
-  mode.local = !fit_rows(&L.caps, spb, c->smem_limit);
   L.uh = c->d_uh;
   L.uh_stride = 3 * H * spb;
-  single_launch_options(L, sh, k, rows_of(c->prm, n_obs), H, c->smem_limit);
-  const size_t smem = smem_bytes(L.caps, spb);
   const int tiles = tiles_out ? n_tiles : L.single.tiles;  // CTAs of the launch
+  brmppi::LaunchMode mode;
+  const size_t smem = plan_single(c, sh, k, tiles, &L, &mode);
   if (smem > c->smem_limit) return fail(c, BRMPPI_EINVAL, "shared memory need exceeds the device limit");
   if ((!tiles_out && static_cast<size_t>(tiles) > c->part_tiles) ||
       static_cast<size_t>(tiles) * static_cast<size_t>(L.uh_stride) > c->uh_floats)
     return fail(c, BRMPPI_EINVAL, "launch shape exceeds the context's scratch");
-  if (L.rows == 0 && !mode.local) mode.ns = samples_per_team(sh, family, tiles, smem, c->num_sms);
   cudaError_t e = brmppi::launch_solve(sh.tps, sh.bpt, tiles, sh.threads, smem, stream, k, L, L.single.P, mode);
   if (e != cudaSuccess) return cuda_fail(c, e, "kernel launch");
   if (u_safe) {

@@ -163,6 +163,12 @@ brmppi_status check_sizes(brmppi_ctx* c, int32_t n_obs, int32_t n_pts, float ds)
 // L.caps.uh_per_team, L.caps.merge); L.caps and L.single must be set.
 void single_launch_options(brmppi::LaunchDesc& L, const Shape& sh, const brmppi::KConst& k, int n_rows, int H,
                            size_t smem_limit);
+// The launch shape of a plain solve: autotuned, or the default rule.
+bool plain_shape(const brmppi_ctx* c, int n_obs, int n_pts, Shape* out);
+// Tables, variant and mode of a single solve's launch of `tiles` CTAs
+// (L->single must be set); returns its dynamic shared memory in bytes.
+size_t plan_single(const brmppi_ctx* c, const Shape& sh, const brmppi::KConst& k, int tiles, brmppi::LaunchDesc* L,
+                   brmppi::LaunchMode* mode);
 
 // Allocate / free the buffers of a lane for max_batch instances of at most
 // S samples and H steps.

@@ -98,13 +98,15 @@ __device__ __forceinline__ uint4 philox_words(PhiloxBlock b, PhiloxSample s, Phi
 // multiply-add, |t| <= 2^-8, and 2 ln(1 + t) = t (2 + t (-1 + 2/3 t)):
 // within 1.42 ulp, 3.0e-8 relative in the root mean square, over all 2^23
 // uniforms (neg2_log_unit with an exact division: 2.5 ulp, 4.1e-8).
-struct NoiseTables {
+// (aligned for the 16-byte copies that stage them)
+struct alignas(16) NoiseTables {
   float cosine[640];  // cos(2 pi (i + 1/2) / 512 - pi/2), so sin at i and cos at i + 128
   float rcp[128], log[128];  // 1 / c, 2 ln c
 };
 constexpr int kNoiseTableFloats = 896;
 constexpr uint32_t kLogBase = 0x3f348000u;  // the float 0.705078125: where m's cells begin
 static_assert(sizeof(NoiseTables) == 4 * kNoiseTableFloats, "tables are staged as one array");
+static_assert(alignof(NoiseTables) >= 16, "tables are staged in 16-byte copies");
 
 namespace table_math {  // compile-time series in double
 constexpr double kPi = 3.14159265358979323846;

@@ -550,6 +550,13 @@ __device__ __forceinline__ void step_barrier() { asm volatile("bar.sync 1, %0;" 
 template <bool W, int NS>
 constexpr int kRowFloats = W ? 4 * NS : 2 * NS;
 constexpr int kMaxRowSlots = 32;  // a lane's rows: 4 per Philox block, at most 8 blocks
+// A lane's rows where they are in local memory (N floats), aligned for the
+// vector accesses of store_row and load_row.
+template <int N>
+struct alignas(16) LocalRows {
+  float v[N];
+};
+static_assert(alignof(LocalRows<1>) >= 16, "rows are read and written as float4");
 template <bool W, int NS>
 __device__ __forceinline__ void store_row(float* p, Vec<NS> al, Vec<NS> u, Vec<NS> w) {
   if constexpr (NS == 1) {
@@ -811,9 +818,9 @@ __device__ void run_tile(const KConst& k, const Inst& in, int tile, float* uh, c
   // for any number of rows.  Rows in registers need it unrolled: at 16 rows
   // a lane the step was 50 KB of code and waited for instructions (stall 0.8
   // an issue), and 64 registers more a lane cost a third of the warps.
-  float local_rows[LOCAL ? 4 * kMaxRowSlots * NS : 1];
+  LocalRows<LOCAL ? kRowFloats<TERMS, NS> * kMaxRowSlots : 1> local_rows;
   const int row_stride = LOCAL ? kRowFloats<TERMS, NS> : kRowFloats<TERMS, NS> * static_cast<int>(blockDim.x);
-  float* rows = LOCAL ? local_rows : S.noise + kRowFloats<TERMS, NS> * static_cast<int>(threadIdx.x);
+  float* rows = LOCAL ? local_rows.v : S.noise + kRowFloats<TERMS, NS> * static_cast<int>(threadIdx.x);
   const int passes = (in.P - 1 + TPS - 1) / TPS;  // Philox blocks 1 .. P - 1 over the team's lanes
   if constexpr (!PRODUCED)
     for (int q = 0; q < 4 * passes; ++q) store_row<TERMS, NS>(rows + q * row_stride, T(k.alpha0), T(0.f), T(0.f));
@@ -1964,7 +1971,7 @@ template <int TPS, int BPT, int EXT, int ROWS = 0, int NS = 1, bool LOCAL = fals
 // single-solve instantiations 384 (up to 170 registers: one CTA per SM on
 // the latency shapes, where registers buy a longer schedule)
 __global__ void __launch_bounds__(ROWS > 0 ? 384 : (NS > 1 ? pair_threads(TPS, EXT) : 512), NS > 1 ? kPairCtas : 1) solve_kernel(const KConst k, const LaunchDesc L) {
-  extern __shared__ float dyn[];
+  extern __shared__ __align__(16) float dyn[];
   __shared__ Shared sh;
   const int spb = compute_threads<TPS>(L.noise_warps) / TPS * NS;
   const Smem S(dyn, L.caps, spb);
@@ -2040,7 +2047,7 @@ __global__ void __launch_bounds__(ROWS > 0 ? 384 : (NS > 1 ? pair_threads(TPS, E
 // finishes a single launch's last tile, so the results are the same bits.
 template <bool EXT>
 __global__ void __launch_bounds__(256) merge_tiles_kernel(const KConst k, const Inst in, const SmemCaps caps) {
-  extern __shared__ float dyn[];
+  extern __shared__ __align__(16) float dyn[];
   __shared__ Shared sh;
   const Smem S(dyn, caps, 1);
   stage_path(in, S);
