@@ -335,6 +335,46 @@ int team_width(int P, long long samples, bool ext, int num_sms) {
   return tps;
 }
 
+// Default width of a context's batches, for a capacity of `samples` samples
+// that run at once (the capacity fixes it, not the batch: a solve's bits must
+// not depend on what it is batched with).  Parked ellipses: the width of a
+// single solve of that many samples; from 17,000 samples (13 rows; 29,000 with
+// more) one lane, which does not repeat the step's base over a team.
+//
+// With the optional terms one lane a sample is the fastest for a filled
+// context but, its step being the sum over all rows, the slowest for one or two
+// solves of a large one.  So a team holds at most two Philox blocks a lane
+// (serving_team_width) unless one lane costs nothing there (up to 4 moving
+// rows, up to 12 obstacles of the collision cost) or the rows are few and the
+// capacity fills the GPU's places with pairs.  GB300, S = 4096, H = 50, capacity
+// of 200 solves; 1 / 2 / 16 / 200 solves, us (the rule before: at most two
+// blocks a lane, from rows kept in registers):
+//   8 moving rows    one lane 102 / 103 / 217 / 1679, two 74 / 74 / 291 / 3200
+//                    (before 95 / 96 / 391 / 4382)
+//   4 obstacles x 5 discs   one lane 257 / 258 / 511 / 5131, four 108 / 139 /
+//                    825 / 9083 (before 118 / 149 / 902 / 9985)
+//   third order and jerk, 8 rows    one lane 124 / 125 / 263 / 2110, two 87 /
+//                    88 / 344 / 3843 (before 102 / 103 / 424 / 4766)
+//   collision cost, 8 obstacles   one lane 63 / 64 / 119 / 854, two 59 / 60 /
+//                    192 / 1951 (before 64 / 65 / 221 / 2296); 28 obstacles, at
+//                    most 64 solves: one lane 80 / 81 / 172, two 74 / 75 / 214,
+//                    four 66 / 79 / 392, eight 81 / 132 / 758 (before 75 / 87 / 445)
+// A context that is always filled gains by batch_threads_per_sample = 1 or the
+// batch autotuner.
+int batch_team_width(const brmppi_params& p, int P, long long samples, int num_sms) {
+  const brmppi::KConst k = make_kconst(p);
+  const int family = brmppi::family_of(k);
+  const int tps = team_width(P, samples, family == brmppi::kDiscs || family == brmppi::kPoint, num_sms);
+  if (family == brmppi::kPlain) return tps;
+  const int two_blocks = serving_team_width(p, P);
+  // the collision cost of standard MPPI: a short loop over the obstacles
+  if (!k.proj) return std::min(std::max(tps, P > 4 && P <= 8 ? 2 : 1), two_blocks);
+  const bool fills = samples >= 768LL * num_sms;  // 6 CTAs of 128 samples an SM
+  const bool narrow = family == brmppi::kMoving ? P <= 2 || (P <= 4 && fills)
+                                                : !k.discs && !k.third && !k.jerk && P <= 4 && fills;
+  return std::max(tps, narrow ? 1 : two_blocks);
+}
+
 // Default shape of a plain solve (no autotuning): tiles that spread the
 // samples evenly over the SMs, and a team as wide as keeps an SM at a few
 // warps.
@@ -587,20 +627,9 @@ bool batch_shape_default(const brmppi_ctx* c, int max_P, Shape* out) {
   if (s.tps == 0 && s.threads == 0 && c->batch_tuned) {
     s = c->batch_shape;
   } else {
-    // A serving context's batches take the served ones' width.  Else the team
-    // width for as many samples as the context's capacity allows at once (the
-    // capacity fixes it: a solve's bits must not depend on its batch), as far
-    // as the tables at that capacity fit beside the team's noise.  From 17,000
-    // samples (13 rows; 29,000 with more) one lane a sample: the step's base
-    // is not repeated over a team, and the rows' state in shared memory
-    // leaves registers for any number of rows.  Measured on GB300, S = 4096,
-    // H = 50, 8 rows, one lane against teams of two: 200 solves of moving rows
-    // 2.53 / 4.06 ms, of collision cost 1.00 / 2.15 ms.  One lane against the
-    // rule's width: 1 solve of parked ellipses 96 / 60 us (four lanes), 2 solves
-    // 96 / 70, 4 solves 97 / 95.  The optional terms against teams of two for
-    // any small capacity: 1 solve of third order and jerk 87.6 / 75.3 us (but 2
-    // solves 87.6 / 92.6), 6 solves of moving rows 144 / 133, of collision cost
-    // 103 / 79; four discs on teams of four, 3 solves 208 / 233, 4 solves 248 / 233.
+    // A serving context's batches take the served ones' width; else the
+    // capacity gives it (batch_team_width), as far as the tables at that
+    // capacity fit beside the team's noise.
     if (s.tps == 0) {
       const int family = brmppi::family_of(make_kconst(c->prm));
       const auto fits = [&](int tps) {
@@ -614,8 +643,7 @@ bool batch_shape_default(const brmppi_ctx* c, int max_P, Shape* out) {
       if (c->prm.max_vehicles > 0) {
         s.tps = serving_team_width(c->prm, max_P);
       } else {
-        s.tps = team_width(max_P, static_cast<long long>(c->prm.max_batch) * c->prm.S,
-                           family == brmppi::kDiscs || family == brmppi::kPoint, c->num_sms);
+        s.tps = batch_team_width(c->prm, max_P, static_cast<long long>(c->prm.max_batch) * c->prm.S, c->num_sms);
         while (s.tps > 1 && !fits(s.tps)) s.tps >>= 1;
       }
     }

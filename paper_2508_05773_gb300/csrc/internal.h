@@ -154,7 +154,8 @@ bool fit_rows(brmppi::SmemCaps* c, int spb, size_t smem_limit);
 int part_stride_for(int H);
 // Team width of a serving context's batches, the served ones and the caller's
 // (a batch of one reproduces a served solve bit for bit): one lane, or with
-// the optional terms a team that keeps a lightly loaded server's step short.
+// the optional terms a team of at most two Philox blocks a lane, which keeps a
+// lightly loaded server's step short.
 int serving_team_width(const brmppi_params& p, int P);
 brmppi_status check_sizes(brmppi_ctx* c, int32_t n_obs, int32_t n_pts, float ds);
 // Options of a single (non-batch) solve launch: the exact-rows variant, with

@@ -65,6 +65,7 @@ class HostContext:
     memory of a GB300 block."""
 
     def __init__(self, params, max_obstacles=16, max_path_pts=4096, num_sms=152, smem_limit=231424, **kw):
+        lib()  # (built before the library is loaded)
         from paper_2508_05773_gb300 import _native
         self._p = _native.params_from_dict(params, max_obstacles, max_path_pts, kw.get("threads_per_sample", 0),
                                            kw.get("block_threads", 0), kw.get("max_batch", 0), 0, 0, 0, 0, 0, 0, 0)
