@@ -323,9 +323,13 @@ int part_stride_for(int H) { return static_cast<int>(align_up(3 + 3 * static_cas
 // P = 1: 4096 27.6 / 29.5 with 1.7 (the noise leaves the chain), 10000 34.0 /
 // 30.8 with 4.1.  The optional terms' longer rows take wider teams further:
 // n = 8: 8000 47.5 / 54.6 with 6.6, two lanes to one 20000 93.6 / 105 with 8.2.
+// More than 16 blocks, 32 lanes to 16: 120 rows of discs S = 64 45.6 / 73.2 (with
+// 16 lanes a CTA of 64 threads holds four samples), 512 49.3 / 81.2, 1000 66.4 /
+// 83.0 with 6.6, 1368 78.4 / 88.0 with 9.0, 2000 123.5 / 93.4 with 13.2; 64 moving
+// rows 512 34.3 / 35.8, 1000 42.6 / 41.9, 1368 48.9 / 47.0.
 int team_width(int P, long long samples, bool ext, int num_sms) {
   int tps = 2, bpt = 0;
-  while (tps < P && tps < 16) tps <<= 1;
+  while (tps < P && tps < 32) tps <<= 1;
   while (tps > 1 && pick_bpt(tps / 2, P, &bpt)) {
     double most = ext ? 9.0 : (tps == 2 ? 12.0 : 7.5);
     if (P <= 4) most = tps == 2 ? (P == 1 ? 3.0 : (ext ? 9.0 : 7.0)) : (ext ? 7.0 : (P == 4 ? 6.5 : 5.75));
@@ -364,7 +368,8 @@ int team_width(int P, long long samples, bool ext, int num_sms) {
 int batch_team_width(const brmppi_params& p, int P, long long samples, int num_sms) {
   const brmppi::KConst k = make_kconst(p);
   const int family = brmppi::family_of(k);
-  const int tps = team_width(P, samples, family == brmppi::kDiscs || family == brmppi::kPoint, num_sms);
+  // (16 lanes of the smallest tile and their noise warps fill a block)
+  const int tps = std::min(16, team_width(P, samples, family == brmppi::kDiscs || family == brmppi::kPoint, num_sms));
   if (family == brmppi::kPlain) return tps;
   const int two_blocks = serving_team_width(p, P);
   // the collision cost of standard MPPI: a short loop over the obstacles

@@ -78,6 +78,18 @@ def test_teams_that_draw_three_blocks_a_lane(pkg, family, tps, n_obs):
         s.close()
 
 
+@pytest.mark.parametrize("family,n_obs", [("plain", 61), ("moving", 124), ("point", 70), ("discs", 24)])
+def test_few_samples_of_many_rows_take_32_lanes(pkg, family, n_obs):
+    c = _terms(sc.small_random(477, S=150, H=6, n_obs=n_obs), family)
+    s = pkg.Solver(c["params"], max_obstacles=n_obs, max_path_pts=c["path"].shape[0])
+    try:
+        plan = plan_probe.single(s, n_obs, c["path"].shape[0])
+        assert (plan["family"], plan["tps"]) == (family, 32), plan
+        _check(device_solve(s, c), c, f"32 lanes {family}")
+    finally:
+        s.close()
+
+
 @pytest.mark.parametrize("family,tps,most", [("moving", 2, 25), ("moving", 4, 40), ("moving", 8, 70), ("discs", 1, 5),
                                              ("point", 1, 11)])
 def test_pairs_of_the_optional_terms_equal_one_sample(pkg, family, tps, most):

@@ -1,0 +1,30 @@
+"""The default launch shapes of single solves and of plain batches (no GPU), at
+sizes where another shape took longer."""
+import ctypes
+import shutil
+
+import pytest
+
+from paper_2508_05773_gb300 import scenarios as sc
+
+pytestmark = pytest.mark.skipif(shutil.which("nvcc") is None, reason="nvcc not available")
+MOVING = dict(flags=sc.FLAG_OBS8)
+THIRD = dict(flags=sc.FLAG_OBS8 | sc.FLAG_THIRD_ORDER)
+DISCS = dict(flags=sc.FLAG_OBS8, **sc.FIVE_DISCS)
+
+
+def _single(S, n_obs, terms):
+    from tests import plan_probe
+    c = plan_probe.HostContext(sc.params(S=S, H=30, **terms), max_obstacles=n_obs, max_path_pts=388)
+    try:
+        return plan_probe.single(c, n_obs, 388)
+    finally:
+        c.close()
+
+
+@pytest.mark.parametrize("terms,n_obs,S,width", [(DISCS, 24, 64, 32), (DISCS, 16, 1000, 32), (DISCS, 24, 2000, 16),
+                                                 (THIRD, 100, 256, 32), (MOVING, 124, 512, 32), ({}, 64, 512, 32),
+                                                 ({}, 60, 512, 16), ({}, 100, 2000, 16)])
+def test_more_than_sixteen_blocks_take_32_lanes_for_few_samples(terms, n_obs, S, width):
+    p = _single(S, n_obs, terms)
+    assert p["tps"] == width and p["tiles"] * (p["threads"] // p["tps"]) >= S
