@@ -370,7 +370,10 @@ int batch_team_width(const brmppi_params& p, int P, long long samples, int num_s
   const int family = brmppi::family_of(k);
   // (16 lanes of the smallest tile and their noise warps fill a block)
   const int tps = std::min(16, team_width(P, samples, family == brmppi::kDiscs || family == brmppi::kPoint, num_sms));
-  if (family == brmppi::kPlain) return tps;
+  // parked ellipses, at most four: past one CTA of two-lane teams an SM one lane
+  // is as fast with rows and faster without (10,000 samples: no row 59 / 70 us,
+  // 1 row 72 / 73, 3 rows 75 / 76; 9000: 59 / 57, 71 / 60, 76 / 62)
+  if (family == brmppi::kPlain) return P <= 2 && tps == 2 && samples > 64LL * num_sms ? 1 : tps;
   const int two_blocks = serving_team_width(p, P);
   // the collision cost of standard MPPI: a short loop over the obstacles
   if (!k.proj) return std::min(std::max(tps, P > 4 && P <= 8 ? 2 : 1), two_blocks);

@@ -28,3 +28,15 @@ def _single(S, n_obs, terms):
 def test_more_than_sixteen_blocks_take_32_lanes_for_few_samples(terms, n_obs, S, width):
     p = _single(S, n_obs, terms)
     assert p["tps"] == width and p["tiles"] * (p["threads"] // p["tps"]) >= S
+
+
+@pytest.mark.parametrize("n_obs,S,width", [(1, 9000, 2), (1, 10000, 1), (4, 12000, 1), (4, 17000, 1), (8, 16000, 2),
+                                           (1, 4096, 2)])
+def test_batches_of_few_rows_past_one_block_an_sm_take_one_lane(n_obs, S, width):
+    import paper_2508_05773_gb300 as pkg
+    from tests import plan_probe
+    c = plan_probe.HostContext(sc.params(S=S, H=50), max_obstacles=n_obs, max_path_pts=388, max_batch=1)
+    try:
+        assert pkg.brmppi_get_batch_launch(ctypes.c_void_p(c.ctx))["threads_per_sample"] == width
+    finally:
+        c.close()
