@@ -391,7 +391,11 @@ int batch_team_width(const brmppi_params& p, int P, long long samples, int num_s
 // block: a tile count just over the SM count leaves most of them idle for a
 // second round (S = 5000, n = 8: 4 lanes x 160 threads 31.6 us, x 128 or 64
 // 40 to 52 us).  Else two or three even CTAs an SM (S = 16384, n = 64: 105.5
-// us at 224 threads, 114 at 128); beyond, 256 threads (two samples a lane).
+// us at 224 threads, 114 at 128); beyond, 256 threads (two samples a team).
+// Three even CTAs only where 256 threads would not fill the places of pairs:
+// S = 12000, n = 70 / 100 / 124 (8 lanes) 204 / 261 / 293 us at 224 threads,
+// 160 / 201 / 213 at 256; S = 10000, where they do not, 185 / 235 / 262 at 192,
+// 219 / 285 / 320 at 256; 4 lanes, S = 25000, n = 64 219 / 187.
 // Narrower blocks (then wider teams) while the shared-memory tables do not fit.
 bool heuristic_plain(const brmppi_ctx* c, int n_obs, int n_pts, Shape* out) {
   const int rows = rows_of(c->prm, n_obs);
@@ -410,17 +414,23 @@ bool heuristic_plain(const brmppi_ctx* c, int n_obs, int n_pts, Shape* out) {
     // blocks that the exact-rows variants take, where one holds the rows
     const bool exact = bpt <= 2 && (ext ? tps == 4 : tps <= 8) && (rows + tps - 1) / tps <= 4;
     const long long limit = exact || bpt == 3 || tps == 1 ? 256 : 384;
+    const auto smem_at = [&](int t) {
+      return smem_bytes(make_caps(n_obs, rows, n_pts, c->prm.H, tps, bpt, family), t / tps);
+    };
     for (long long k = 1; k <= 3 && threads == 0; ++k) {
+      const int spb = 256 / tps;
+      if (k == 3 && smem_at(256) <= c->smem_limit &&
+          samples_per_team(Shape{tps, bpt, 256}, family, (S + spb - 1) / spb, smem_at(256), c->num_sms) == 2) {
+        threads = 256;
+        break;
+      }
       const long long even = ((S + k * sms - 1) / (k * sms) * tps + 31) / 32 * 32;
       if (even <= (k == 1 ? limit : 256)) threads = static_cast<int>(std::max<long long>(kMinThreads, even));
     }
     if (threads == 0) {
       // 256, or 384 (more samples share the CTA's tables) where that keeps
       // more samples on an SM
-      auto resident = [&](int t) {
-        const size_t smem = smem_bytes(make_caps(n_obs, rows, n_pts, c->prm.H, tps, bpt, family), t / tps);
-        return pair_residency(tps, family, t / 2, smem) * t;
-      };
+      auto resident = [&](int t) { return pair_residency(tps, family, t / 2, smem_at(t)) * t; };
       threads = brmppi::pair_exists(tps, bpt, family) && resident(384) > resident(256) ? 384 : 256;
     }
   }
@@ -653,6 +663,11 @@ bool batch_shape_default(const brmppi_ctx* c, int max_P, Shape* out) {
       } else {
         s.tps = batch_team_width(c->prm, max_P, static_cast<long long>(c->prm.max_batch) * c->prm.S, c->num_sms);
         while (s.tps > 1 && !fits(s.tps)) s.tps >>= 1;
+        // lanes that draw three or four blocks of parked ellipses: 32 samples a
+        // CTA share its tables (70 / 124 obstacles, S = 4096, H = 50: 1 solve 166 /
+        // 220 us at 128 threads, 158 / 215 at 256; 64 solves 4.45 / 5.98 ms,
+        // 4.30 / 5.86)
+        if (family == brmppi::kPlain && s.tps == 8 && max_P > 17 && s.threads == 0) s.threads = 256;
       }
     }
     if (s.threads == 0) s.threads = std::max(128, kMinBatchSpb * s.tps);

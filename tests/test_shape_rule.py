@@ -40,3 +40,21 @@ def test_batches_of_few_rows_past_one_block_an_sm_take_one_lane(n_obs, S, width)
         assert pkg.brmppi_get_batch_launch(ctypes.c_void_p(c.ctx))["threads_per_sample"] == width
     finally:
         c.close()
+
+
+@pytest.mark.parametrize("n_obs,S,threads,ns", [(100, 10000, 192, 1), (100, 12000, 256, 2), (124, 11000, 256, 2),
+                                                (124, 8500, 224, 1), (64, 25000, 256, 2), (64, 20000, 192, 1)])
+def test_pairs_before_three_even_blocks_an_sm(n_obs, S, threads, ns):
+    p = _single(S, n_obs, {})
+    assert (p["threads"], p["ns"]) == (threads, ns), p
+
+
+@pytest.mark.parametrize("n_obs,threads", [(64, 128), (70, 256), (124, 256)])
+def test_batches_of_many_ellipses_take_larger_tiles(n_obs, threads):
+    import paper_2508_05773_gb300 as pkg
+    from tests import plan_probe
+    c = plan_probe.HostContext(sc.params(S=4096, H=50), max_obstacles=n_obs, max_path_pts=388, max_batch=64)
+    try:
+        assert pkg.brmppi_get_batch_launch(ctypes.c_void_p(c.ctx))["block_threads"] == threads
+    finally:
+        c.close()
