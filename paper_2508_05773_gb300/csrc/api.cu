@@ -289,10 +289,11 @@ bool pick_bpt(int tps, int P, int* bpt) {
   return brmppi::variant_exists(tps, *bpt);
 }
 
-// CTAs of `threads` threads of the two-sample variants on an SM.
+// CTAs of `threads` threads of the two-sample variants on an SM (one that fits
+// the device's limit is resident, whatever the allowance for static memory).
 long long pair_residency(int tps, int family, int threads, size_t smem) {
-  return std::min<long long>(brmppi::pair_threads(tps, family) * brmppi::kPairCtas / threads,
-                             227 * 1024 / (smem + 2048));
+  return std::max<long long>(1, std::min<long long>(brmppi::pair_threads(tps, family) * brmppi::kPairCtas / threads,
+                                                    227 * 1024 / (smem + 2048)));
 }
 
 // Two samples a team where their CTAs fill three quarters of the GPU's places:

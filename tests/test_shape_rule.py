@@ -58,3 +58,17 @@ def test_batches_of_many_ellipses_take_larger_tiles(n_obs, threads):
         assert pkg.brmppi_get_batch_launch(ctypes.c_void_p(c.ctx))["block_threads"] == threads
     finally:
         c.close()
+
+
+@pytest.mark.parametrize("rows", [8100, 8140, 8180])
+def test_few_samples_stay_unpaired_when_a_block_fills_shared_memory(rows):
+    """One block an SM, whatever its tables: three tiles are no reason for two
+    samples a lane, up to the last kilobyte of shared memory."""
+    from tests import plan_probe
+    c = plan_probe.HostContext(sc.params(S=1000, H=140), max_obstacles=28, max_path_pts=rows, threads_per_sample=1,
+                               block_threads=384)
+    try:
+        p = plan_probe.single(c, 28, rows)
+        assert p["tiles"] == 3 and p["smem"] > 228000 and (p["ns"], p["local"]) == (1, 0), p
+    finally:
+        c.close()
