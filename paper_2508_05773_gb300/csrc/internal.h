@@ -6,6 +6,7 @@
 #include <cstdint>
 #include <map>
 #include <string>
+#include <vector>
 
 #include "brmppi.h"
 #include "launch.h"
@@ -166,6 +167,11 @@ void single_launch_options(brmppi::LaunchDesc& L, const Shape& sh, const brmppi:
                            size_t smem_limit);
 // The launch shape of a plain solve: autotuned, or the default rule.
 bool plain_shape(const brmppi_ctx* c, int n_obs, int n_pts, Shape* out);
+// The shapes that the autotuner times for solves of n_obs obstacles and n_pts
+// path rows.
+std::vector<Shape> plain_candidates(const brmppi_ctx* c, int n_obs, int n_pts);
+// The same for batches whose rows need up to max_P Philox blocks a step.
+std::vector<Shape> batch_candidates(const brmppi_ctx* c, int max_P);
 // Tables, variant and mode of a single solve's launch of `tiles` CTAs
 // (L->single must be set); returns its dynamic shared memory in bytes.
 size_t plan_single(const brmppi_ctx* c, const Shape& sh, const brmppi::KConst& k, int tiles, brmppi::LaunchDesc* L,

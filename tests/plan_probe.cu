@@ -56,6 +56,21 @@ extern "C" int probe_batch(brmppi_ctx* c, const brmppi_instance* inst, int n, Pr
   return 0;
 }
 
+// What the autotuners time: (lanes, threads) pairs, at most `room` of them.
+static int shapes_out(const std::vector<Shape>& v, int32_t* out, int room) {
+  for (int i = 0; i < static_cast<int>(v.size()) && i < room; ++i) {
+    out[2 * i] = v[i].tps;
+    out[2 * i + 1] = v[i].threads;
+  }
+  return static_cast<int>(v.size());
+}
+extern "C" int probe_plain_candidates(const brmppi_ctx* c, int n_obs, int n_pts, int32_t* out, int room) {
+  return shapes_out(plain_candidates(c, n_obs, n_pts), out, room);
+}
+extern "C" int probe_batch_candidates(const brmppi_ctx* c, int32_t* out, int room) {
+  return shapes_out(batch_candidates(c, philox_blocks(rows_of(c->prm, c->prm.max_obstacles))), out, room);
+}
+
 extern "C" void probe_alignments(int64_t* tables, int64_t* local_rows) {
   *tables = alignof(brmppi::NoiseTables);
   *local_rows = alignof(brmppi::LocalRows<3>);

@@ -54,6 +54,21 @@ def batch(solver, insts):
     return out.as_dict()
 
 
+def _shapes(count, *args):
+    out = (ctypes.c_int32 * 128)()
+    n = count(*args, out, 64)
+    return [(out[2 * i], out[2 * i + 1]) for i in range(n)]
+
+
+def plain_candidates(context, n_obs, n_pts):
+    """(lanes, threads) of the shapes that the plain autotuner times."""
+    return _shapes(lib().probe_plain_candidates, ctypes.c_void_p(context.ctx), n_obs, n_pts)
+
+
+def batch_candidates(context):
+    return _shapes(lib().probe_batch_candidates, ctypes.c_void_p(context.ctx))
+
+
 def alignments():
     a, b = ctypes.c_int64(), ctypes.c_int64()
     lib().probe_alignments(ctypes.byref(a), ctypes.byref(b))
