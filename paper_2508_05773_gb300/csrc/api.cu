@@ -419,14 +419,12 @@ bool heuristic_plain(const brmppi_ctx* c, int n_obs, int n_pts, Shape* out) {
       return smem_bytes(make_caps(n_obs, rows, n_pts, c->prm.H, tps, bpt, family), t / tps);
     };
     for (long long k = 1; k <= 3 && threads == 0; ++k) {
-      const int spb = 256 / tps;
-      if (k == 3 && smem_at(256) <= c->smem_limit &&
-          samples_per_team(Shape{tps, bpt, 256}, family, (S + spb - 1) / spb, smem_at(256), c->num_sms) == 2) {
-        threads = 256;
-        break;
-      }
       const long long even = ((S + k * sms - 1) / (k * sms) * tps + 31) / 32 * 32;
-      if (even <= (k == 1 ? limit : 256)) threads = static_cast<int>(std::max<long long>(kMinThreads, even));
+      if (even > (k == 1 ? limit : 256)) continue;
+      const int spb = 256 / tps;
+      const bool pairs = k == 3 && smem_at(256) <= c->smem_limit &&
+                         samples_per_team(Shape{tps, bpt, 256}, family, (S + spb - 1) / spb, smem_at(256), c->num_sms) == 2;
+      threads = pairs ? 256 : static_cast<int>(std::max<long long>(kMinThreads, even));
     }
     if (threads == 0) {
       // 256, or 384 (more samples share the CTA's tables) where that keeps

@@ -49,6 +49,17 @@ def test_pairs_before_three_even_blocks_an_sm(n_obs, S, threads, ns):
     assert (p["threads"], p["ns"]) == (threads, ns), p
 
 
+@pytest.mark.parametrize("rows,threads", [(388, 256), (2401, 384)])
+def test_large_solves_share_long_tables_over_more_samples(rows, threads):
+    from tests import plan_probe
+    c = plan_probe.HostContext(sc.params(S=65536, H=100), max_obstacles=64, max_path_pts=rows)
+    try:
+        p = plan_probe.single(c, 64, rows)
+        assert (p["threads"], p["ns"]) == (threads, 2), p
+    finally:
+        c.close()
+
+
 @pytest.mark.parametrize("n_obs,threads", [(64, 128), (70, 256), (124, 256)])
 def test_batches_of_many_ellipses_take_larger_tiles(n_obs, threads):
     import paper_2508_05773_gb300 as pkg
