@@ -10,13 +10,66 @@
 //
 // Every operation rounds by itself: a product is never fused into a sum
 // unless fma() says so.  A step written in Vec<N> gives a sample the same
-// bits in every instantiation (lanes a sample, samples a lane).
+// bits in every instantiation (lanes a sample, samples a lane).  The
+// arithmetic also builds for the host, in the same roundings (without
+// contraction), so that the accuracy tests run what the kernels run.
 #pragma once
 
+#include <cmath>
 #include <cstdint>
+#include <cstring>
 #include <cuda_runtime.h>
 
 namespace brmppi {
+
+#define BRMPPI_HD __host__ __device__ __forceinline__
+
+BRMPPI_HD uint32_t float_bits(float v) {
+#ifdef __CUDA_ARCH__
+  return __float_as_uint(v);
+#else
+  uint32_t b;
+  std::memcpy(&b, &v, sizeof(b));
+  return b;
+#endif
+}
+BRMPPI_HD float bits_float(uint32_t b) {
+#ifdef __CUDA_ARCH__
+  return __uint_as_float(b);
+#else
+  float v;
+  std::memcpy(&v, &b, sizeof(v));
+  return v;
+#endif
+}
+BRMPPI_HD float mul_rn(float a, float b) {
+#ifdef __CUDA_ARCH__
+  return __fmul_rn(a, b);
+#else
+  return a * b;
+#endif
+}
+BRMPPI_HD float add_rn(float a, float b) {
+#ifdef __CUDA_ARCH__
+  return __fadd_rn(a, b);
+#else
+  return a + b;
+#endif
+}
+BRMPPI_HD float sub_rn(float a, float b) {
+#ifdef __CUDA_ARCH__
+  return __fsub_rn(a, b);
+#else
+  return a - b;
+#endif
+}
+BRMPPI_HD float fma_rn(float a, float b, float c) {
+#ifdef __CUDA_ARCH__
+  return __fmaf_rn(a, b, c);
+#else
+  return std::fmaf(a, b, c);
+#endif
+}
 
 template <int N>
 struct Vec;
@@ -25,36 +78,55 @@ template <>
 struct Vec<1> {
   float x;
   Vec() = default;
-  __device__ __forceinline__ Vec(float v) : x(v) {}
-  __device__ __forceinline__ float get(int) const { return x; }
-  __device__ __forceinline__ void set(int, float v) { x = v; }
+  BRMPPI_HD Vec(float v) : x(v) {}
+  BRMPPI_HD float get(int) const { return x; }
+  BRMPPI_HD void set(int, float v) { x = v; }
 };
 
 template <>
 struct Vec<2> {
   float2 x;
   Vec() = default;
-  __device__ __forceinline__ Vec(float v) : x(make_float2(v, v)) {}
-  __device__ __forceinline__ explicit Vec(float2 v) : x(v) {}
-  __device__ __forceinline__ float get(int i) const { return i ? x.y : x.x; }
-  __device__ __forceinline__ void set(int i, float v) {
+  BRMPPI_HD Vec(float v) : x(make_float2(v, v)) {}
+  BRMPPI_HD explicit Vec(float2 v) : x(v) {}
+  BRMPPI_HD float get(int i) const { return i ? x.y : x.x; }
+  BRMPPI_HD void set(int i, float v) {
     if (i) x.y = v;
     else x.x = v;
   }
 };
 
-__device__ __forceinline__ Vec<1> operator*(Vec<1> a, Vec<1> b) { return __fmul_rn(a.x, b.x); }
-__device__ __forceinline__ Vec<1> operator+(Vec<1> a, Vec<1> b) { return __fadd_rn(a.x, b.x); }
-__device__ __forceinline__ Vec<1> operator-(Vec<1> a, Vec<1> b) { return __fsub_rn(a.x, b.x); }
-__device__ __forceinline__ Vec<1> operator-(Vec<1> a) { return -a.x; }
-__device__ __forceinline__ Vec<1> fma(Vec<1> a, Vec<1> b, Vec<1> c) { return __fmaf_rn(a.x, b.x, c.x); }
+BRMPPI_HD Vec<1> operator*(Vec<1> a, Vec<1> b) { return mul_rn(a.x, b.x); }
+BRMPPI_HD Vec<1> operator+(Vec<1> a, Vec<1> b) { return add_rn(a.x, b.x); }
+BRMPPI_HD Vec<1> operator-(Vec<1> a, Vec<1> b) { return sub_rn(a.x, b.x); }
+BRMPPI_HD Vec<1> operator-(Vec<1> a) { return -a.x; }
+BRMPPI_HD Vec<1> fma(Vec<1> a, Vec<1> b, Vec<1> c) { return fma_rn(a.x, b.x, c.x); }
 
-__device__ __forceinline__ Vec<2> operator*(Vec<2> a, Vec<2> b) { return Vec<2>(__fmul2_rn(a.x, b.x)); }
-__device__ __forceinline__ Vec<2> operator+(Vec<2> a, Vec<2> b) { return Vec<2>(__fadd2_rn(a.x, b.x)); }
-__device__ __forceinline__ Vec<2> operator-(Vec<2> a) { return Vec<2>(make_float2(-a.x.x, -a.x.y)); }
-__device__ __forceinline__ Vec<2> fma(Vec<2> a, Vec<2> b, Vec<2> c) { return Vec<2>(__ffma2_rn(a.x, b.x, c.x)); }
+// (the packed forms exist from sm_100 on)
+BRMPPI_HD Vec<2> operator*(Vec<2> a, Vec<2> b) {
+#if defined(__CUDA_ARCH__) && __CUDA_ARCH__ >= 1000
+  return Vec<2>(__fmul2_rn(a.x, b.x));
+#else
+  return Vec<2>(make_float2(mul_rn(a.x.x, b.x.x), mul_rn(a.x.y, b.x.y)));
+#endif
+}
+BRMPPI_HD Vec<2> operator+(Vec<2> a, Vec<2> b) {
+#if defined(__CUDA_ARCH__) && __CUDA_ARCH__ >= 1000
+  return Vec<2>(__fadd2_rn(a.x, b.x));
+#else
+  return Vec<2>(make_float2(add_rn(a.x.x, b.x.x), add_rn(a.x.y, b.x.y)));
+#endif
+}
+BRMPPI_HD Vec<2> operator-(Vec<2> a) { return Vec<2>(make_float2(-a.x.x, -a.x.y)); }
+BRMPPI_HD Vec<2> fma(Vec<2> a, Vec<2> b, Vec<2> c) {
+#if defined(__CUDA_ARCH__) && __CUDA_ARCH__ >= 1000
+  return Vec<2>(__ffma2_rn(a.x, b.x, c.x));
+#else
+  return Vec<2>(make_float2(fma_rn(a.x.x, b.x.x, c.x.x), fma_rn(a.x.y, b.x.y, c.x.y)));
+#endif
+}
 // a - b in one packed instruction: -1 b + a rounds once, as the difference does
-__device__ __forceinline__ Vec<2> operator-(Vec<2> a, Vec<2> b) { return fma(b, Vec<2>(-1.f), a); }
+BRMPPI_HD Vec<2> operator-(Vec<2> a, Vec<2> b) { return fma(b, Vec<2>(-1.f), a); }
 
 // component by component: no packed form exists
 template <int N, typename F>
@@ -87,12 +159,20 @@ __device__ __forceinline__ Vec<N> vrcp(Vec<N> a) {
   });
 }
 template <int N>
-__device__ __forceinline__ Vec<N> vrsqrt(Vec<N> a) {
-  return vmap(a, [](float v) {
-    float r;
-    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
-    return r;
-  });
+BRMPPI_HD Vec<N> vrsqrt(Vec<N> a) {
+  Vec<N> r;
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    const float v = a.get(i);
+    float q;
+#ifdef __CUDA_ARCH__
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(q) : "f"(v));
+#else
+    q = 1.0f / std::sqrt(v);
+#endif
+    r.set(i, q);
+  }
+  return r;
 }
 template <int N>
 __device__ __forceinline__ Vec<N> vshfl_xor(Vec<N> a, int m) {
@@ -107,42 +187,6 @@ __device__ __forceinline__ void acc2(Vec<N>& h, Vec<N>& l, Vec<N> inc) {
   const Vec<N> bp = sum - h;
   l = l + ((h - (sum - bp)) + (inc - bp));
   h = sum;
-}
-
-// turn_sincos and state_sincos of trig.cuh (their derivation and accuracy
-// are stated there), the same operations in the same order.
-template <int N>
-__device__ __forceinline__ void turn_sincos(Vec<N> e, Vec<N>* s, Vec<N>* c) {
-  using T = Vec<N>;
-  const T e2 = e * e, e4 = e2 * e2;
-  *s = fma(e * e2,
-           fma(e4, fma(e2, T(2.7557318844628753e-06f), T(-1.9841270113829523e-04f)),
-               fma(e2, T(8.333333767950535e-03f), T(-0.1666666716337204f))),
-           e);
-  *c = fma(e2,
-           fma(e4 * e4, T(-2.755731998149713e-07f),
-               fma(e4, fma(e2, T(2.4801587642286904e-05f), T(-1.3888889225199820e-03f)),
-                   fma(e2, T(0.0416666679084301f), T(-0.5f)))),
-           T(1.0f));
-}
-
-template <int N>
-__device__ __forceinline__ void state_sincos(Vec<N> x, Vec<N>* s, Vec<N>* c) {
-  using T = Vec<N>;
-  const T t = fma(x, T(0.636619746685028f), T(12582912.0f));
-  const T kf = t + T(-12582912.0f);
-  T r = fma(kf, T(-1.5707963705062866f), x);
-  r = fma(kf, T(4.371138828673793e-08f), r);
-  T sr, cr;
-  turn_sincos(r, &sr, &cr);
-#pragma unroll
-  for (int i = 0; i < N; ++i) {
-    const uint32_t q = __float_as_uint(t.get(i));
-    const bool odd = q & 1u;
-    const float ss = odd ? cr.get(i) : sr.get(i), cc = odd ? sr.get(i) : cr.get(i);
-    s->set(i, (q & 2u) ? -ss : ss);
-    c->set(i, ((q + 1u) & 2u) ? -cc : cc);
-  }
 }
 
 // into [-pi, pi]; only the square of the result is used.  The turn count is
