@@ -310,8 +310,8 @@ struct Frame {
   float c0, s0, c0l, s0l;                      // cos / sin of theta1_0, and their low parts
   float t2, v_h, v_l, dl;                      // theta2 - theta1_0, speed, steer angle
   float a0;                                    // acceleration (jerk-input model)
-  float qf0;                                   // fractional path cell of psi0
-  int i0;                                      // integer path cell of psi0
+  float qf0;                                   // path cell of psi0 less i0
+  int i0;                                      // integer path cell of psi0, within kMaxFirstCell
   float psi_h, psi_l;                          // psi0
   double psi0;
 };
@@ -352,6 +352,11 @@ __device__ __forceinline__ void frame_sincos(float hi, float lo, float* s, float
   *cl = cneg ? -ccl : ccl;
 }
 
+// Path cells are counted from a reference cell of at most this size, as floats
+// within +- 2 kMaxFirstCell (stage_cost): every row of a path (8192 at most) is
+// within that range of the reference.
+constexpr double kMaxFirstCell = 1.0e6;
+
 // The frame of x0, built by warp 0: lane j takes state component j, so the
 // FP64 work runs side by side; the path cell of psi0 uses the host's FP64
 // reciprocal of ds (no device division).
@@ -383,7 +388,9 @@ __device__ __forceinline__ void make_frame_warp(const double* x0, double inv_ds,
       fr.psi_h = hi;
       fr.psi_l = lo;
       const double q0 = x * inv_ds;
-      const double fq = fmin(fmax(floor(q0), -1.0e9), 1.0e9);
+      // within the range of stage_cost's cell count, so that a cell on the path
+      // is counted from here wherever psi0 is
+      const double fq = fmin(fmax(floor(q0), -kMaxFirstCell), kMaxFirstCell);
       fr.i0 = static_cast<int>(fq);
       fr.qf0 = static_cast<float>(q0 - fq);
       break;
@@ -908,8 +915,9 @@ __device__ void run_tile(const KConst& k, const Inst& in, int tile, float* uh, c
   auto stage_cost = [&](const Visit& x) -> T {
     // path cell: floor of qf by the 1.5 * 2^23 shifter on qf - 1/2 (an exact
     // integer may take the cell below with ff = 1, the same point); the
-    // clamp keeps the shifter in range far outside any path
-    const T qf = vclamp(fma(x.ps, T(in.inv_ds), qf0), -2.0e6f, 2.0e6f);
+    // clamp keeps the shifter in range (2^22) far outside any path
+    constexpr float kMost = 2.0 * kMaxFirstCell;
+    const T qf = vclamp(fma(x.ps, T(in.inv_ds), qf0), -kMost, kMost);
     const T tt = (qf + T(-0.5f)) + T(12582912.0f);
     const T fl = tt + T(-12582912.0f);
     // ff = qf - fl, with the cancelling parts in one fused operation and the
