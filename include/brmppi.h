@@ -256,7 +256,12 @@ brmppi_status brmppi_hitch_stabilize_device(brmppi_ctx *ctx, const double *x_dev
    launch of a persistent kernel: work items (instance, sample tile) are
    taken longest-first from an atomic counter; each instance's partials are
    merged in tile order by the CTA that finishes its last tile, so a solve
-   gives the same result alone (as a batch of one) or in any mix.  Uploads
+   gives the same result alone (as a batch of one) or in any mix.  The default
+   launch shape, and with it the last bits of a solve, follows the context:
+   max_batch times S, max_obstacles, the optional terms and the tables'
+   capacities, not the batch.  A context with optional terms keeps a solve or
+   two quick by teams of lanes; one that is always full is faster with
+   batch_threads_per_sample = 1 or brmppi_autotune_batch.  Uploads
    the instance table and work list (host -> device, pinned) and enqueues
    the kernel on `stream`; allocates nothing, does not synchronise (the next
    call on this context waits for the previous upload to be consumed). */
@@ -272,9 +277,10 @@ brmppi_status brmppi_batch_capture(brmppi_ctx *ctx, const brmppi_instance *inst,
 brmppi_status brmppi_graph_launch(brmppi_graph *g, void *stream);
 void brmppi_graph_destroy(brmppi_graph *g);
 
-/* Autotuner: time every supported launch shape (threads per sample x Philox
-   blocks per lane x block size) on the given device inputs, `reps` launches
-   each, and keep the fastest for later plain solves with this obstacle
+/* Autotuner: time the default launch shape and blocks of 64, 128, 256 and 384
+   threads at every supported number of threads per sample on the given device
+   inputs, `reps` launches each back to back, and keep the default, or a shape
+   that is faster by more than 2%, for later plain solves with this obstacle
    count (used when params.threads_per_sample == 0). */
 brmppi_status brmppi_autotune(brmppi_ctx *ctx, const double *x0_dev, const float *U_nom_dev,
                               const float *obs_dev, int32_t n_obs, const float *path_dev,
@@ -320,9 +326,12 @@ brmppi_status brmppi_solve_device_noalloc(const brmppi_params *p, const double *
    counter (+1 per solve) resident; requests of one vehicle run in
    submission order.  Results do not depend on what else is in a batch: the
    serving launch shape is fixed at create (params.batch_threads_per_sample
-   and batch_block_threads when set, else one lane per sample in 128-thread
-   blocks), and a batch of one on the same context (batch shape not changed
-   by brmppi_autotune_batch) reproduces a served solve bit for bit. */
+   and batch_block_threads when set; else one lane per sample without optional
+   terms, and with any (a flag but BRMPPI_FLAG_PROJ_NONE, or footprint discs) 2,
+   4, 8 or 16 lanes for up to 12, 28, 60 or 124 rows, max_obstacles times
+   n_discs; blocks of 128 threads, 256 for 16 lanes), and a batch of one on the same context (batch
+   shape not changed by brmppi_autotune_batch) reproduces a served solve bit for
+   bit. */
 
 /* Register (or re-register) a vehicle: its reference path (host, n_pts*3),
    initial nominal sequence (host H*3, NULL = zeros) and noise seed; its

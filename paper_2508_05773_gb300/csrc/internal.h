@@ -14,7 +14,7 @@
 namespace brmppi_host {
 
 constexpr int kMaxObstacles = 124;  // ceil((4 + n)/4) <= 32 Philox blocks
-constexpr int kMaxPathPts = 8192;  // 5 floats a row in shared memory
+constexpr int kMaxPathPts = 8192;  // 16 bytes a row in shared memory
 constexpr int kMaxH = 1024;
 constexpr int kMinThreads = 64;
 constexpr int kMaxThreads = 512;
@@ -33,8 +33,9 @@ inline bool exponent_ok(const brmppi_params& p, float e) {
   return e == 2.0f || ((p.flags & BRMPPI_FLAG_OBS8) && e == 4.0f);
 }
 
-// Consecutive path headings at most pi/4 apart (and finite): the kernel
-// turns each row's heading direction by the interpolation angle.
+// Consecutive path headings at most pi/4 apart (and finite): the reference
+// heading and position are interpolated linearly between rows, which a wider
+// turn leaves too coarse to follow (or not unwrapped), so it is refused.
 inline bool path_turns_ok(const float* path, int n_pts) {
   for (int j = 0; j + 1 < n_pts; ++j)
     if (!(std::fabs(path[3 * j + 5] - path[3 * j + 2]) <= 0.78539816339744831f)) return false;

@@ -36,9 +36,11 @@
 // (row j on lane j % TPS of the latency shapes, a Philox block's four rows on
 // one lane elsewhere), each with its noise normal 4 + j.  The rank-2
 // structure of the projection makes the cross-lane exchange five floats per
-// step.  The step is written in Vec<NS> (vec.cuh), every rounding explicit:
-// a sample has the same bits in each variant of one team width, so a batch
-// may run two samples a team when it fills the GPU and one when it does not.
+// step.  The step is written in Vec<NS> (vec.cuh), every rounding explicit: a
+// sample has the same bits with one sample a team and with two (of one width,
+// both drawing their noise themselves), so a batch may run pairs when it fills
+// the GPU and not when it does not.  Other widths, and teams with noise warps, add
+// the rows' or the cost's terms in another order.
 //
 // What bounds it (measured on GB300, before this layout -> with it): the
 // throughput shapes are bound by issue slots and the FMA pipe.  48 solves of
@@ -46,8 +48,8 @@
 // instructions a rollout-step (packed pairs, table-driven normals, the first
 // Philox rounds shared, rows as linear forms in (Q d, Q), no subnormal
 // scaling around the MUFU); 256 uneven solves 2567 -> 1802 us; S = 65536,
-// H = 100, 64 ellipses 2030 -> 1482 us (FMA pipe 58% and ALU pipe 40% busy,
-// three warps a scheduler).  The latency shapes are bound by one compute
+// H = 100, 64 ellipses 2030 -> 1482 us (FMA pipe 51% and ALU pipe 36% busy,
+// 2.8 warps a scheduler).  The latency shapes are bound by one compute
 // warp's dependency chain: S = 4096, H = 50, 8 ellipses 39.6 -> 31.7 us.
 //
 // Projection in Woodbury form.  A = [A_u | diag(h~)] where only the a and
@@ -172,8 +174,9 @@ struct LaunchDesc {
 
 enum : unsigned { ERR_EXPONENT = 1u, ERR_NONFINITE_X0 = 2u, ERR_PATH_TURN = 4u };
 
-// Largest heading change between consecutive path rows (rad): the stage
-// cost's interpolated heading turns a row's direction by at most this.
+// Largest heading change between consecutive path rows (rad): the interface
+// refuses wider turns, whose linear interpolation is too coarse to follow (no
+// arithmetic below depends on it).
 constexpr float kMaxPathTurn = 0.78539816339744831f;  // pi / 4
 
 __device__ __forceinline__ float clampf(float v, float lo, float hi) { return fminf(fmaxf(v, lo), hi); }
@@ -1997,7 +2000,8 @@ __global__ void __launch_bounds__(ROWS > 0 ? 384 : (NS > 1 ? pair_threads(TPS, E
   // the wait returns once that kernel has completed and its writes are
   // visible, so everything after it is as in a plain launch.  The next solve
   // may be started at once for the same reason.  Back to back, S = 256, H = 30
-  // 20.5 -> 17.8 us, S = 4096, H = 50 34.8 -> 31.7 us.
+  // 20.5 -> 17.8 us, S = 4096, H = 50 34.8 -> 31.7 us; a solve behind a copy or on
+  // an idle stream gains nothing by it.
   stage_tables(S);
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

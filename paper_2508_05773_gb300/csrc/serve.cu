@@ -301,9 +301,9 @@ brmppi_status server_create(brmppi_ctx* c) {
   sv->wait_ms = wait_limit_ms(p);
   // the launch shape of every serving batch, fixed here so that a solve's
   // bits do not depend on what else is in its batch: the context's batch
-  // shape parameters when given, else one lane per sample (teams just wide
-  // enough for two Philox blocks a lane when rows carry a steer-rate column)
-  // in 128-thread blocks
+  // shape parameters when given, else one lane per sample in 128-thread blocks,
+  // or with any optional term teams just wide enough for two Philox blocks a lane
+  // (2 to 16 lanes, at least 16 teams a block)
   const int P_cap = philox_blocks(rows_of(p, p.max_obstacles));
   sv->shape.tps = p.batch_threads_per_sample != 0 ? p.batch_threads_per_sample : serving_team_width(p, P_cap);
   sv->shape.threads =
