@@ -686,11 +686,6 @@ bool batch_shape_default(const brmppi_ctx* c, int max_P, Shape* out, bool tuned 
       } else {
         s.tps = batch_team_width(c->prm, max_P, static_cast<long long>(c->prm.max_batch) * c->prm.S, c->num_sms);
         while (s.tps > 1 && !fits(s.tps)) s.tps >>= 1;
-        // lanes that draw three or four blocks of parked ellipses: 32 samples a
-        // CTA share its tables (70 / 124 obstacles, S = 4096, H = 50: 1 solve 166 /
-        // 220 us at 128 threads, 158 / 215 at 256; 64 solves 4.45 / 5.98 ms,
-        // 4.30 / 5.86)
-        if (family == brmppi::kPlain && s.tps == 8 && max_P > 17 && s.threads == 0) s.threads = 256;
       }
     }
     if (s.threads == 0) s.threads = std::max(128, kMinBatchSpb * s.tps);

@@ -60,8 +60,8 @@ def test_large_solves_share_long_tables_over_more_samples(rows, threads):
         c.close()
 
 
-@pytest.mark.parametrize("n_obs,threads", [(64, 128), (70, 256), (124, 256)])
-def test_batches_of_many_ellipses_take_larger_tiles(n_obs, threads):
+@pytest.mark.parametrize("n_obs,threads", [(64, 128), (70, 128), (124, 128)])
+def test_batches_of_many_ellipses_keep_small_tiles(n_obs, threads):
     import paper_2508_05773_gb300 as pkg
     from tests import plan_probe
     c = plan_probe.HostContext(sc.params(S=4096, H=50), max_obstacles=n_obs, max_path_pts=388, max_batch=64)
